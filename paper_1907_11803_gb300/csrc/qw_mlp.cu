@@ -26,125 +26,187 @@
 namespace qw {
 namespace {
 
-constexpr int GM = 64, GN = 64, GK = 16, GT = 256;
+// C[m][n] = sum_k A(m, k) B(k, n) over k in [k0, k1), FP32 fused multiply-adds
+// in the order of k (A(m, k) = A[m * sam + k * sak], likewise B; one of the two
+// strides of each is 1).
+// EPI 0: store; 1: add bias; 2: add bias, store the pre-activation to C and
+// ReLU(.) to Aout; 3: zero where gate[m][n] is not positive (ReLU's backward);
+// 4: partial sums of split blockIdx.z (C += z * csplit; the K range is cut in
+// gridDim.z pieces of kper), and from the blocks of column 0 the row sums of A
+// (the bias gradient) to Aout + z * csplit.
+//
+// A block of 256 threads computes a 64 x BN tile, 4 x 4 (BN = 64) or 4 x 2
+// values per thread, read from shared memory as 16- and 8-byte words; the next
+// 16 k are in registers while the current ones are summed.  The weight
+// gradients are 256 x 256 outputs over K = the rows: one block per tile leaves
+// 136 of the 152 SMs idle, hence the split over K with the pieces summed in a
+// fixed order (grad_sum_kernel, adam_kernel).  Loss and gradient of 8,192 rows
+// of a 192-256-256-16 network, one call: 4,250 us unsplit, 354 us so (the three
+// weight-gradient products alone took 3,816 us).
+constexpr int GM = 64, GK = 16, GT = 256;
 
-template <typename TB>
-__device__ __forceinline__ float to_f(TB v);
+template <typename T>
+__device__ __forceinline__ float to_f(T v);
 template <>
 __device__ __forceinline__ float to_f<float>(float v) { return v; }
 template <>
 __device__ __forceinline__ float to_f<__half>(__half v) { return __half2float(v); }
 
-// C[m][n] = sum_k A(m, k) B(k, n) (+ bias[n]) with arbitrary strides.
-// EPI 0: store; 1: add bias; 2: add bias, store pre-activation to C and
-// ReLU(.) to Aout.
-template <typename TB, int EPI>
-__global__ void __launch_bounds__(GT) mlp_gemm_kernel(int M, int N, int K,
-                                                      const float *__restrict__ A, int64_t sam,
-                                                      int64_t sak, const TB *__restrict__ B,
-                                                      int64_t sbk, int64_t sbn,
-                                                      float *__restrict__ C, int64_t ldc,
-                                                      const float *__restrict__ bias,
-                                                      float *__restrict__ Aout)
+template <typename TB, int BN, int EPI>
+__global__ void __launch_bounds__(GT) mlp_gemm_kernel(
+    int M, int N, int K, int kper, const float *__restrict__ A, int64_t sam, int64_t sak,
+    const TB *__restrict__ B, int64_t sbk, int64_t sbn, float *__restrict__ C, int64_t ldc,
+    const float *__restrict__ bias, const float *__restrict__ gate, float *__restrict__ Aout,
+    int64_t csplit)
 {
-    __shared__ float As[GK][GM + 1];
-    __shared__ float Bs[GK][GN + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int m0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += GK) {
-        for (int e = threadIdx.x; e < GM * GK; e += GT) {
-            const int mm = e / GK, kk = e % GK;
+    constexpr int TN = BN / 16;                 // columns per thread
+    constexpr int PA = GM * GK / GT, PB = (BN * GK + GT - 1) / GT;
+    __shared__ __align__(16) float As[GK][GM + 4];
+    __shared__ __align__(16) float Bs[GK][BN + 4];
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int m0 = blockIdx.y * GM, n0 = blockIdx.x * BN;
+    const int kb = EPI == 4 ? (int)blockIdx.z * kper : 0;
+    const int ke = EPI == 4 ? min(K, kb + kper) : K;
+    const bool a_kc = sak == 1, b_kc = sbk == 1;
+    float ra[PA], rb[PB];
+    // piece u of this thread: (row, k) with the contiguous index fastest
+    auto a_at = [&](int u, int &mm, int &kk) {
+        const int e = tid + u * GT;
+        if (a_kc) { mm = e / GK; kk = e % GK; } else { mm = e % GM; kk = e / GM; }
+    };
+    auto b_at = [&](int u, int &nn, int &kk) {
+        const int e = tid + u * GT;
+        if (b_kc) { nn = e / GK; kk = e % GK; } else { nn = e % BN; kk = e / BN; }
+    };
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < PA; ++u) {
+            int mm, kk;
+            a_at(u, mm, kk);
             const int gm = m0 + mm, gk = k0 + kk;
-            As[kk][mm] = (gm < M && gk < K) ? A[gm * sam + gk * sak] : 0.0f;
+            ra[u] = (gm < M && gk < ke) ? A[gm * sam + gk * sak] : 0.0f;
         }
-        for (int e = threadIdx.x; e < GN * GK; e += GT) {
-            const int nn = e / GK, kk = e % GK;
+#pragma unroll
+        for (int u = 0; u < PB; ++u) {
+            int nn, kk;
+            b_at(u, nn, kk);
             const int gn = n0 + nn, gk = k0 + kk;
-            Bs[kk][nn] = (gn < N && gk < K) ? to_f<TB>(B[gk * sbk + gn * sbn]) : 0.0f;
+            rb[u] = (kk < GK && gn < N && gk < ke) ? to_f<TB>(B[gk * sbk + gn * sbn]) : 0.0f;
+        }
+    };
+    float acc[4][TN] = {};
+    float asum[4] = {};
+    fetch(kb);
+    for (int k0 = kb; k0 < ke; k0 += GK) {
+#pragma unroll
+        for (int u = 0; u < PA; ++u) {
+            int mm, kk;
+            a_at(u, mm, kk);
+            As[kk][mm] = ra[u];
+        }
+#pragma unroll
+        for (int u = 0; u < PB; ++u) {
+            int nn, kk;
+            b_at(u, nn, kk);
+            if (kk < GK) Bs[kk][nn] = rb[u];
         }
         __syncthreads();
+        if (k0 + GK < ke) fetch(k0 + GK);
 #pragma unroll
         for (int kk = 0; kk < GK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+            const float4 a4 = *reinterpret_cast<const float4 *>(&As[kk][ty * 4]);
+            const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+            float b[TN];
+            if constexpr (TN == 4) {
+                const float4 b4 = *reinterpret_cast<const float4 *>(&Bs[kk][tx * 4]);
+                b[0] = b4.x; b[1] = b4.y; b[2] = b4.z; b[3] = b4.w;
+            } else {
+                const float2 b2 = *reinterpret_cast<const float2 *>(&Bs[kk][tx * 2]);
+                b[0] = b2.x; b[1] = b2.y;
+            }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            if (EPI == 4 && blockIdx.x == 0)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) asum[i] += a[i];
         }
         __syncthreads();
     }
+    if (EPI == 4) C += blockIdx.z * csplit;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int gm = m0 + ty + 16 * i;
+        const int gm = m0 + ty * 4 + i;
         if (gm >= M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int gn = n0 + tx + 16 * j;
+        for (int j = 0; j < TN; ++j) {
+            const int gn = n0 + tx * TN + j;
             if (gn >= N) continue;
             float v = acc[i][j];
-            if (EPI >= 1) v += bias[gn];
+            if (EPI == 1 || EPI == 2) v += bias[gn];
+            if (EPI == 3 && !(gate[gm * ldc + gn] > 0.0f)) v = 0.0f;
             C[gm * ldc + gn] = v;
             if (EPI == 2) Aout[gm * ldc + gn] = v > 0.0f ? v : 0.0f;
         }
+        if (EPI == 4 && blockIdx.x == 0 && tx == 0) Aout[blockIdx.z * csplit + gm] = asum[i];
     }
 }
 
-// Softmax cross-entropy of one row per warp: adds -log p[y] to *loss_sum and
-// writes d logits = (p - onehot(y)) * inv_n; or, without labels, p.
+// Softmax cross-entropy of one row per warp: adds -log p[y] to *loss_sum (one
+// addition per block) and writes d logits = (p - onehot(y)) * inv_n; or,
+// without labels, p.
 __global__ void softmax_rows_kernel(const float *__restrict__ Z, int n, int C,
                                     const int32_t *__restrict__ y, float inv_n,
                                     float *__restrict__ dZ, float *__restrict__ loss_sum,
                                     float *__restrict__ prob)
 {
+    __shared__ float s_loss[32];
     const int r = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (r >= n) return;
-    const float *z = Z + (int64_t)r * C;
-    float mx = -INFINITY;
-    for (int c = lane; c < C; c += 32) mx = fmaxf(mx, z[c]);
-    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    float s = 0.0f;
-    for (int c = lane; c < C; c += 32) s += __expf(z[c] - mx);
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    const float inv_s = 1.0f / s;
-    for (int c = lane; c < C; c += 32) {
-        const float p = __expf(z[c] - mx) * inv_s;
-        if (prob) prob[(int64_t)r * C + c] = p;
-        if (dZ) dZ[(int64_t)r * C + c] = (p - ((y && c == y[r]) ? 1.0f : 0.0f)) * inv_n;
-    }
-    if (lane == 0 && y && loss_sum) {
-        const float logp = (z[y[r]] - mx) - __logf(s);
-        atomicAdd(loss_sum, -logp);
-    }
-}
-
-// out[c] = sum_r D[r][c]
-__global__ void colsum_kernel(const float *__restrict__ D, int n, int C, float *__restrict__ out)
-{
-    const int c = blockIdx.x;
-    float s = 0.0f;
-    for (int r = threadIdx.x; r < n; r += blockDim.x) s += D[(int64_t)r * C + c];
-    __shared__ float red[32];
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        s = threadIdx.x < (int)(blockDim.x / 32) ? red[threadIdx.x] : 0.0f;
+    float row_loss = 0.0f;
+    if (r < n) {
+        const float *z = Z + (int64_t)r * C;
+        float mx = -INFINITY;
+        for (int c = lane; c < C; c += 32) mx = fmaxf(mx, z[c]);
+        for (int off = 16; off > 0; off >>= 1)
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+        float s = 0.0f;
+        for (int c = lane; c < C; c += 32) s += __expf(z[c] - mx);
         for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (threadIdx.x == 0) out[c] = s;
+        const float inv_s = 1.0f / s;
+        for (int c = lane; c < C; c += 32) {
+            const float p = __expf(z[c] - mx) * inv_s;
+            if (prob) prob[(int64_t)r * C + c] = p;
+            if (dZ) dZ[(int64_t)r * C + c] = (p - ((y && c == y[r]) ? 1.0f : 0.0f)) * inv_n;
+        }
+        if (lane == 0 && y) row_loss = -((z[y[r]] - mx) - __logf(s));
+    }
+    if (!loss_sum) return;
+    if (lane == 0) s_loss[threadIdx.x >> 5] = row_loss;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.0f;
+        for (int w = 0; w < (int)(blockDim.x / 32); ++w) t += s_loss[w];
+        atomicAdd(loss_sum, t);
     }
 }
 
-__global__ void relu_back_kernel(float *__restrict__ dA, const float *__restrict__ Z, int64_t count)
+// g[i] = the sum of the splits' partial gradients (split s at part[s * np + i]).
+__device__ __forceinline__ float split_sum(const float *__restrict__ part, int64_t i, int64_t np,
+                                           int splits)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
+    float v = part[i];
+    for (int s = 1; s < splits; ++s) v += part[s * np + i];
+    return v;
+}
+
+__global__ void grad_sum_kernel(const float *__restrict__ part, int64_t np, int splits,
+                                float *__restrict__ g)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < np;
          i += (int64_t)gridDim.x * blockDim.x)
-        if (!(Z[i] > 0.0f)) dA[i] = 0.0f;
+        g[i] = split_sum(part, i, np, splits);
 }
 
 __global__ void to_half_kernel(const float *__restrict__ p, __half *__restrict__ h, int64_t count)
@@ -154,14 +216,15 @@ __global__ void to_half_kernel(const float *__restrict__ p, __half *__restrict__
         h[i] = __float2half_rn(p[i]);
 }
 
-__global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g,
+// One Adam step; the gradient is the sum of the splits' partial gradients.
+__global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ part, int splits,
                             float *__restrict__ m1, float *__restrict__ m2,
                             __half *__restrict__ h, int64_t count, float lr, float b1, float b2,
                             float eps, float c1, float c2)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
+        const float gi = split_sum(part, i, count, splits);
         const float a = b1 * m1[i] + (1.0f - b1) * gi;
         const float b = b2 * m2[i] + (1.0f - b2) * gi * gi;
         m1[i] = a;
@@ -221,13 +284,20 @@ __global__ void sumsq_kernel(const float *__restrict__ X, int64_t count, double 
 
 template <typename TB, int EPI>
 qw_status gemm(int M, int N, int K, const float *A, int64_t sam, int64_t sak, const TB *B,
-               int64_t sbk, int64_t sbn, float *C, int64_t ldc, const float *bias, float *Aout,
-               cudaStream_t s)
+               int64_t sbk, int64_t sbn, float *C, int64_t ldc, const float *bias,
+               const float *gate, float *Aout, cudaStream_t s, int splits = 1, int kper = 0,
+               int64_t csplit = 0)
 {
     if (M <= 0 || N <= 0) return QW_OK;
-    dim3 grid((unsigned)((N + GN - 1) / GN), (unsigned)((M + GM - 1) / GM));
-    mlp_gemm_kernel<TB, EPI><<<grid, GT, 0, s>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias,
-                                                 Aout);
+    // the classes (N = 16 or so) take the narrow tile
+    const int bn = N <= 32 ? 32 : 64;
+    dim3 grid((unsigned)((N + bn - 1) / bn), (unsigned)((M + GM - 1) / GM), (unsigned)splits);
+    if (bn == 32)
+        mlp_gemm_kernel<TB, 32, EPI><<<grid, GT, 0, s>>>(M, N, K, kper, A, sam, sak, B, sbk, sbn, C,
+                                                         ldc, bias, gate, Aout, csplit);
+    else
+        mlp_gemm_kernel<TB, 64, EPI><<<grid, GT, 0, s>>>(M, N, K, kper, A, sam, sak, B, sbk, sbn, C,
+                                                         ldc, bias, gate, Aout, csplit);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
 }
@@ -241,7 +311,10 @@ struct qw_mlp {
     int n_in = 0, H = 0, C = 0;
     int64_t np = 0;
     int64_t oW1 = 0, ob1 = 0, oW2 = 0, ob2 = 0, oW3 = 0, ob3 = 0;
+    static constexpr int kSplits = 32;
+    static constexpr int64_t kPartBytes = (int64_t)256 << 20;
     DevBuf p32, p16, grad, m1, m2, work, scalar;
+    DevBuf part;  // the weight gradients' partial sums
     DevBuf p16t;  // k-major FP16 copies of W1, W2, W3 for the fused inference kernel
     DevBuf tc_err;  // error word of the tensor-core forward pass
     int cap = 0;  // rows the work buffers hold
@@ -274,40 +347,48 @@ struct qw_mlp {
     {
         const __half *h = p16.as<__half>();
         const float *p = p32.as<float>();
-        QW_TRY((gemm<__half, 2>(n, H, n_in, X, n_in, 1, h + oW1, 1, n_in, Z1, H, p + ob1, A1, s)));
-        QW_TRY((gemm<__half, 2>(n, H, H, A1, H, 1, h + oW2, 1, H, Z2, H, p + ob2, A2, s)));
-        QW_TRY((gemm<__half, 1>(n, C, H, A2, H, 1, h + oW3, 1, H, Z3, C, p + ob3, nullptr, s)));
+        QW_TRY((gemm<__half, 2>(n, H, n_in, X, n_in, 1, h + oW1, 1, n_in, Z1, H, p + ob1, nullptr,
+                                A1, s)));
+        QW_TRY((gemm<__half, 2>(n, H, H, A1, H, 1, h + oW2, 1, H, Z2, H, p + ob2, nullptr, A2, s)));
+        QW_TRY((gemm<__half, 1>(n, C, H, A2, H, 1, h + oW3, 1, H, Z3, C, p + ob3, nullptr, nullptr,
+                                s)));
         return QW_OK;
     }
 
-    // loss sum into scalar[0] and gradient (mean over n rows) into grad
+    // Pieces of the rows in the weight gradients of n rows: at least 64 rows
+    // each, at most kSplits and at most kPartBytes of partial sums (np floats
+    // per piece; a single piece is written to grad).
+    int splits_of(int n) const
+    {
+        const int64_t fit = kPartBytes / (np * (int64_t)sizeof(float));
+        return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(kSplits, n / 64), fit));
+    }
+    const float *partials(int n) const { return (splits_of(n) == 1 ? grad : part).as<float>(); }
+
+    // loss sum into scalar[0] and the pieces' gradients (mean over n rows):
+    // gradient i = the sum over the pieces of partials(n)[piece * np + i]
     qw_status backward(const float *X, const int32_t *y, int n, cudaStream_t s)
     {
         const __half *h = p16.as<__half>();
-        float *g = grad.as<float>();
         float *loss = scalar.as<float>();
+        const int S = splits_of(n);
+        const int kper = ((n + S - 1) / S + GK - 1) / GK * GK;
+        if (S > 1) QW_TRY(part.ensure((size_t)S * np * sizeof(float)));
+        float *g = S > 1 ? part.as<float>() : grad.as<float>();
         softmax_rows_kernel<<<(n + 7) / 8, 256, 0, s>>>(Z3, n, C, y, 1.0f / (float)n, D3, loss,
                                                         nullptr);
         QW_CUDA_TRY(cudaGetLastError());
         // layer 3
-        QW_TRY((gemm<float, 0>(C, H, n, D3, 1, C, A2, H, 1, g + oW3, H, nullptr, nullptr, s)));
-        colsum_kernel<<<C, 256, 0, s>>>(D3, n, C, g + ob3);
-        QW_CUDA_TRY(cudaGetLastError());
-        QW_TRY((gemm<__half, 0>(n, H, C, D3, C, 1, h + oW3, H, 1, DA, H, nullptr, nullptr, s)));
-        relu_back_kernel<<<152 * 4, 256, 0, s>>>(DA, Z2, (int64_t)n * H);
-        QW_CUDA_TRY(cudaGetLastError());
-        // layer 2 (DA now holds d Z2)
-        QW_TRY((gemm<float, 0>(H, H, n, DA, 1, H, A1, H, 1, g + oW2, H, nullptr, nullptr, s)));
-        colsum_kernel<<<H, 256, 0, s>>>(DA, n, H, g + ob2);
-        QW_CUDA_TRY(cudaGetLastError());
-        QW_TRY((gemm<__half, 0>(n, H, H, DA, H, 1, h + oW2, H, 1, DZ, H, nullptr, nullptr, s)));
-        relu_back_kernel<<<152 * 4, 256, 0, s>>>(DZ, Z1, (int64_t)n * H);
-        QW_CUDA_TRY(cudaGetLastError());
+        QW_TRY((gemm<float, 4>(C, H, n, D3, 1, C, A2, H, 1, g + oW3, H, nullptr, nullptr, g + ob3,
+                               s, S, kper, np)));
+        QW_TRY((gemm<__half, 3>(n, H, C, D3, C, 1, h + oW3, H, 1, DA, H, nullptr, Z2, nullptr, s)));
+        // layer 2 (DA holds d Z2)
+        QW_TRY((gemm<float, 4>(H, H, n, DA, 1, H, A1, H, 1, g + oW2, H, nullptr, nullptr, g + ob2,
+                               s, S, kper, np)));
+        QW_TRY((gemm<__half, 3>(n, H, H, DA, H, 1, h + oW2, H, 1, DZ, H, nullptr, Z1, nullptr, s)));
         // layer 1 (DZ holds d Z1)
-        QW_TRY((gemm<float, 0>(H, n_in, n, DZ, 1, H, X, n_in, 1, g + oW1, n_in, nullptr, nullptr,
-                               s)));
-        colsum_kernel<<<H, 256, 0, s>>>(DZ, n, H, g + ob1);
-        QW_CUDA_TRY(cudaGetLastError());
+        QW_TRY((gemm<float, 4>(H, n_in, n, DZ, 1, H, X, n_in, 1, g + oW1, n_in, nullptr, nullptr,
+                               g + ob1, s, S, kper, np)));
         return QW_OK;
     }
 };
@@ -394,6 +475,12 @@ qw_status qw_mlp_loss_grad(qw_mlp *mp, const float *X, const int32_t *y, int64_t
     QW_CUDA_TRY(cudaMemsetAsync(mp->scalar.p, 0, 64, s));
     QW_TRY(mp->forward(X, (int)n, s));
     QW_TRY(mp->backward(X, y, (int)n, s));
+    const int splits = mp->splits_of((int)n);
+    if (grad && splits > 1) {
+        grad_sum_kernel<<<152 * 4, 256, 0, s>>>(mp->partials((int)n), mp->np, splits,
+                                                mp->grad.as<float>());
+        QW_CUDA_TRY(cudaGetLastError());
+    }
     float ls = 0.0f;
     QW_CUDA_TRY(cudaMemcpyAsync(&ls, mp->scalar.p, 4, cudaMemcpyDeviceToHost, s));
     if (grad)
@@ -425,8 +512,8 @@ qw_status qw_mlp_train(qw_mlp *mp, const float *X, const int32_t *y, int64_t n, 
             mp->version += 1;
             const float c1 = 1.0f - powf(b1, (float)mp->step);
             const float c2 = 1.0f - powf(b2, (float)mp->step);
-            adam_kernel<<<152 * 4, 256, 0, s>>>(mp->p32.as<float>(), mp->grad.as<float>(),
-                                                mp->m1.as<float>(), mp->m2.as<float>(),
+            adam_kernel<<<152 * 4, 256, 0, s>>>(mp->p32.as<float>(), mp->partials(nb),
+                                                mp->splits_of(nb), mp->m1.as<float>(), mp->m2.as<float>(),
                                                 mp->p16.as<__half>(), mp->np, lr, b1, b2, eps, c1,
                                                 c2);
             QW_CUDA_TRY(cudaGetLastError());
