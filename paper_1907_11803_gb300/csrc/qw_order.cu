@@ -39,42 +39,47 @@ __global__ void order_key_kernel(const int32_t *__restrict__ HQ, int64_t nq, int
     atomicAdd(hist + key, 1);
 }
 
-// Exclusive scan of kKeyBins counts in one block.
+// Exclusive scan of kKeyBins counts in one block: warp w owns 2,048
+// consecutive counts, read twice as 16 coalesced 512-byte pieces (the first
+// pass sums them, the second scans), so the block waits on two rounds of
+// independent loads.  One thread per 64 consecutive counts, the earlier form,
+// touched 32 lines with every load and took 68 us; a one-query call went from
+// 272 to 211 us with this one.
 __global__ void __launch_bounds__(1024) order_scan_kernel(int32_t *__restrict__ hist)
 {
     __shared__ int32_t wsum[32];
-    constexpr int per = kKeyBins / 1024;
-    const int t = threadIdx.x;
-    int local[per];
+    constexpr int kPieces = kKeyBins / 32 / 128;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int4 *h4 = reinterpret_cast<int4 *>(hist) + warp * kPieces * 32;
     int sum = 0;
 #pragma unroll
-    for (int j = 0; j < per; ++j) {
-        local[j] = hist[t * per + j];
-        sum += local[j];
+    for (int p = 0; p < kPieces; ++p) {
+        const int4 v = h4[p * 32 + lane];
+        sum += v.x + v.y + v.z + v.w;
     }
-    const int lane = t & 31, warp = t >> 5;
-    int incl = sum;
-    for (int off = 1; off < 32; off <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += y;
-    }
-    if (lane == 31) wsum[warp] = incl;
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) wsum[warp] = sum;
     __syncthreads();
-    if (warp == 0) {
-        int v = wsum[lane];
-        int wi = v;
-        for (int off = 1; off < 32; off <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, wi, off);
-            if (lane >= off) wi += y;
-        }
-        wsum[lane] = wi - v;
-    }
-    __syncthreads();
-    int run = wsum[warp] + incl - sum;
+    int run = __reduce_add_sync(0xffffffffu, lane < warp ? wsum[lane] : 0);
+    constexpr int kAhead = 4;  // pieces in flight (a whole warp's share would not fit in registers)
+    for (int p0 = 0; p0 < kPieces; p0 += kAhead) {
+        int4 v[kAhead];
 #pragma unroll
-    for (int j = 0; j < per; ++j) {
-        hist[t * per + j] = run;
-        run += local[j];
+        for (int u = 0; u < kAhead; ++u) v[u] = h4[(p0 + u) * 32 + lane];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int4 c = v[u];
+            const int mine = c.x + c.y + c.z + c.w;
+            int incl = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
+            }
+            const int e = run + incl - mine;
+            h4[(p0 + u) * 32 + lane] = make_int4(e, e + c.x, e + c.x + c.y, e + c.x + c.y + c.z);
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
     }
 }
 
