@@ -20,10 +20,6 @@ namespace qw {
 constexpr int kTile = 32768;
 constexpr int kTileShift = 15;
 
-// Bucket id written by the FP32 projection when the value is too close to a
-// bucket boundary to trust; the FP64 pass replaces every such entry.
-constexpr int32_t kNeedsFp64 = INT32_MIN;
-
 // Per-(query, tile) candidate profile: [0] previous-level candidates,
 // [1 + c] other candidates with collision count c (c <= QW_MAX_M).
 constexpr int kHistBins = QW_MAX_M + 2;
@@ -60,10 +56,11 @@ struct DevBuf {
 };
 
 // ---------------------------------------------------------------- projection
-// H[r * ld_row + i * ld_col] = floor((a_i . V_r + b_i) / w), FP32 with an
-// FP64 recomputation of every entry near a bucket boundary.  err (device int)
-// gets bit 1 set when a bucket id falls outside int32.  fixups (device
-// unsigned long long, may be null) counts FP64 recomputations.
+// H[r * ld_row + i * ld_col] = floor((a_i . V_r + b_i) / w), FP32 with a
+// recomputation (pairs of floats, then FP64) of every entry near a bucket
+// boundary.  err (device int) gets bit 1 set when a bucket id falls outside
+// int32.  fixups (device unsigned long long, may be null) counts the
+// recomputed entries.
 // tensor_cores (m <= 128): the projection on the tensor cores (split BF16
 // products, FP32 accumulation) with its own proven bound; same bucket ids.
 qw_status launch_hash(const float *V, int64_t nv, int d, const float *A, const float *b, int m,
