@@ -137,9 +137,10 @@ typedef struct {
                              qw_index_profile); the call then waits for the stream */
     int32_t path;         /* QW_PATH_AUTO, QW_PATH_CLUSTER or QW_PATH_LEVELS (below) */
     int32_t clusters;     /* cluster path: most clusters resident at once; 0 = all that fit */
-    int32_t order;        /* QW_ORDER_AUTO / QW_ORDER_SIGNATURE: answer queries grouped by a
-                             coarse bucket signature (queries of one region share index
-                             entries in L2); QW_ORDER_GIVEN: in the caller's order.  Results are
+    int32_t order;        /* QW_ORDER_SIGNATURE: answer queries grouped by a coarse bucket
+                             signature (queries of one region share index entries in L2);
+                             QW_ORDER_GIVEN: in the caller's order; QW_ORDER_AUTO: by
+                             signature from 2,048 queries on.  Results are
                              returned in the caller's order either way and do not depend on it */
     int32_t rerank;       /* QW_RERANK_FP32 (default), QW_RERANK_BF16 or QW_RERANK_BF16_TC
                              (both need shadow_bf16): the BF16 pre-filter on CUDA cores, or with
@@ -358,8 +359,9 @@ int32_t qw_qalsh_collision_threshold(int32_t m, float w, int32_t c, int64_t n, i
  * V: nv x d float32, A: m x d float32, b: m float32, H: nv x m int32; all
  * DEVICE pointers.  The projection runs in FP32; every result whose FP32 value
  * lies within a proven error bound (and at least 1e-5 w) of a bucket boundary
- * is recomputed in FP64 with the dot product summed in index order, so H
- * equals the FP64 result.  *n_fixups (optional, host) receives how many were
+ * is recomputed in pairs of floats, and where those leave the floor open in
+ * FP64 with the dot product summed in index order, so H equals the FP64
+ * result.  *n_fixups (optional, host) receives how many were
  * recomputed; passing it makes the call wait for the stream.
  * Errors: QW_ERR_ARG (null pointer, nv < 0, d < 1, m < 1, w <= 0),
  * QW_ERR_RANGE (a bucket id outside int32; H is then unspecified),
@@ -374,7 +376,7 @@ qw_status qw_hash(const float *V, int64_t nv, int32_t d, const float *A, const f
  * (3.01 * 2^-16 + (d - 1) * 2^-22 + 2^-23) * ||a_i|| ||V_r|| for any order of
  * the tensor cores' additions, taking each to lose at most two units in the
  * last place.  Entries within that bound (and at least 1e-5 w) of a bucket
- * boundary are recomputed in FP64 as in qw_hash, so H equals the FP64 result;
+ * boundary are recomputed as in qw_hash, so H equals the FP64 result;
  * the wider bound means more recomputations (*n_fixups).  Arguments, pointer
  * spaces and errors as qw_hash; QW_ERR_ARG also for m > 128. */
 qw_status qw_hash_tc(const float *V, int64_t nv, int32_t d, const float *A, const float *b,
