@@ -583,26 +583,9 @@ static qw_status build_impl(qw_index *ix, const float *data, const float *A, con
         QW_CUDA_TRY(cudaMemcpyAsync(ix->prefix_off.p, poff.data(), m * sizeof(int64_t),
                                     cudaMemcpyHostToDevice, s));
         // internal (locality) order of the bitmaps
-        std::vector<int32_t> h_perm;
-        {
-            std::vector<float> hX, hA;
-            try {
-                hX.resize((size_t)n * d);
-                hA.resize((size_t)m * d);
-            } catch (const std::bad_alloc &) {
-                set_error("qw_build_index: out of host memory for the locality order");
-                return QW_ERR_OOM;
-            }
-            QW_CUDA_TRY(cudaMemcpyAsync(hX.data(), ix->X.p, hX.size() * sizeof(float),
-                                        cudaMemcpyDeviceToHost, s));
-            QW_CUDA_TRY(cudaMemcpyAsync(hA.data(), ix->A.p, hA.size() * sizeof(float),
-                                        cudaMemcpyDeviceToHost, s));
-            QW_CUDA_TRY(cudaStreamSynchronize(s));
-            QW_TRY(locality_order(hX.data(), n, d, hA.data(), m, h_perm));
-        }
         QW_TRY(ix->perm.ensure((size_t)n * sizeof(int32_t)));
-        QW_CUDA_TRY(cudaMemcpyAsync(ix->perm.p, h_perm.data(), (size_t)n * sizeof(int32_t),
-                                    cudaMemcpyHostToDevice, s));
+        QW_TRY(locality_order(ix->X.as<float>(), n, d, ix->A.as<float>(), m,
+                              ix->perm.as<int32_t>(), s));
         QW_TRY(ix->bm_sum.ensure((size_t)lay.total * (kBmUint4 / 32) * sizeof(uint32_t)));
         QW_TRY(launch_bitmap_build(ix->view(), ix->c, ix->bm_maxJ, Ht.as<int32_t>(),
                                    ix->host_bitmaps ? ix->bm_host.as<uint4>() : ix->bm.as<uint4>(),
@@ -618,7 +601,6 @@ static qw_status build_impl(qw_index *ix, const float *data, const float *A, con
         QW_TRY(ix->hloc.ensure((size_t)n * ix->hloc_stride));
         QW_CUDA_TRY(cudaMemsetAsync(ix->hloc.p, 0, ix->hloc.bytes, s));
         QW_TRY(launch_hloc_build(ix->view(), Ht.as<int32_t>(), ix->hloc.p, s));
-        QW_CUDA_TRY(cudaStreamSynchronize(s));  // the host order must outlive its upload
         QW_TRY(launch_bid_prefix(ix->view(), ix->bid_prefix.as<int64_t>(),
                                  ix->prefix_off.as<int64_t>(), s));
     }

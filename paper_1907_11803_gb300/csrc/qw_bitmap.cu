@@ -20,7 +20,7 @@
 // no atomics per entry and no counters kept between levels.
 //
 // Ids are numbered in a locality order (a two-means tree over the data, leaves
-// of 128 ids): a 128-id group holds nearby points.  Every bitmap carries a
+// of 128 ids; qw_tree.cu): a 128-id group holds nearby points.  Every bitmap carries a
 // 256-bit summary (which groups it touches).  A group touched by fewer than l
 // of the query's m buckets cannot hold a candidate, so a level runs in two
 // passes: a filter on the summaries finds the live groups of every (query,
@@ -40,10 +40,6 @@
 #include "qw_tma.cuh"
 
 #include <algorithm>
-#include <thread>
-#include <cmath>
-#include <atomic>
-#include <new>
 #include <vector>
 
 namespace qw {
@@ -1806,180 +1802,6 @@ qw_status launch_bitmap_build(const IndexView &ix, int c, int maxJ, const int32_
     bm_summary_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), BM_THREADS, 0, s>>>(
         bm, total_bitmaps, bm_sum);
     QW_CUDA_TRY(cudaGetLastError());
-    return QW_OK;
-}
-
-namespace {
-
-// Run f(chunk, begin, end) over [0, n) in chunks of `chunk` on the host's
-// cores.  Chunk boundaries do not depend on the thread count, so results
-// combined per chunk in chunk order are deterministic.
-template <class F>
-void parallel_chunks(int64_t n, int64_t chunk, F &&f)
-{
-    const int64_t nc = (n + chunk - 1) / chunk;
-    int64_t nt = (int64_t)std::max(1u, std::thread::hardware_concurrency());
-    nt = std::min(nt, nc);
-    if (nt <= 1) {
-        for (int64_t c = 0; c < nc; ++c) f(c, c * chunk, std::min(n, (c + 1) * chunk));
-        return;
-    }
-    std::atomic<int64_t> next(0);
-    std::vector<std::thread> th;
-    for (int64_t t = 0; t < nt; ++t)
-        th.emplace_back([&] {
-            for (;;) {
-                const int64_t c = next.fetch_add(1);
-                if (c >= nc) break;
-                f(c, c * chunk, std::min(n, (c + 1) * chunk));
-            }
-        });
-    for (auto &x : th) x.join();
-}
-
-struct TreeNode {
-    int64_t lo, hi;
-    int depth;
-};
-
-// Split perm[lo, hi) in two: two centroids seeded by the extremes along LSH
-// projection depth mod m, refined by three rounds of two-means, then the
-// points ordered by their side of the bisecting hyperplane and cut where the
-// two-means boundary falls, rounded to a multiple of kGroupIds (so every
-// 128-id group of the internal order stays inside one leaf).
-void split_node(const float *X, int d, const float *A, int m, std::vector<int32_t> &perm,
-                const TreeNode &nd, bool par, TreeNode *kids)
-{
-    const int64_t lo = nd.lo, len = nd.hi - nd.lo;
-    const int64_t chunk = 4096;
-    const int64_t nc = (len + chunk - 1) / chunk;
-    auto each = [&](auto &&f) {
-        if (par) {
-            parallel_chunks(len, chunk, f);
-        } else {
-            for (int64_t c = 0; c < nc; ++c) f(c, c * chunk, std::min(len, (c + 1) * chunk));
-        }
-    };
-    auto row = [&](int64_t j) { return X + (size_t)perm[(size_t)(lo + j)] * (size_t)d; };
-    // seeds: smallest and largest projection on one LSH direction
-    const float *a = A + (size_t)(nd.depth % m) * (size_t)d;
-    std::vector<double> cmin(nc, HUGE_VAL), cmax(nc, -HUGE_VAL);
-    std::vector<int64_t> amin(nc, 0), amax(nc, 0);
-    each([&](int64_t c, int64_t b, int64_t e) {
-        for (int64_t j = b; j < e; ++j) {
-            const float *x = row(j);
-            double t = 0.0;
-            for (int k = 0; k < d; ++k) t += (double)a[k] * (double)x[k];
-            if (t < cmin[c]) { cmin[c] = t; amin[c] = j; }
-            if (t > cmax[c]) { cmax[c] = t; amax[c] = j; }
-        }
-    });
-    int64_t jmin = amin[0], jmax = amax[0];
-    double vmin = cmin[0], vmax = cmax[0];
-    for (int64_t c = 1; c < nc; ++c) {
-        if (cmin[c] < vmin) { vmin = cmin[c]; jmin = amin[c]; }
-        if (cmax[c] > vmax) { vmax = cmax[c]; jmax = amax[c]; }
-    }
-    std::vector<double> c1(d), c2(d), v(d);
-    for (int k = 0; k < d; ++k) {
-        c1[k] = row(jmin)[k];
-        c2[k] = row(jmax)[k];
-    }
-    double thr = 0.0;
-    std::vector<double> part((size_t)nc * (2 * (size_t)d + 2));
-    for (int it = 0; it < 4; ++it) {
-        double n1 = 0.0, n2 = 0.0;
-        double q1 = 0.0, q2 = 0.0;
-        for (int k = 0; k < d; ++k) {
-            v[k] = c2[k] - c1[k];
-            q1 += c1[k] * c1[k];
-            q2 += c2[k] * c2[k];
-        }
-        thr = 0.5 * (q2 - q1);
-        if (it == 3) break;  // the last round only fixes the hyperplane
-        std::fill(part.begin(), part.end(), 0.0);
-        each([&](int64_t c, int64_t b, int64_t e) {
-            double *ps = part.data() + (size_t)c * (2 * (size_t)d + 2);
-            for (int64_t j = b; j < e; ++j) {
-                const float *x = row(j);
-                double t = 0.0;
-                for (int k = 0; k < d; ++k) t += v[k] * (double)x[k];
-                double *acc = t < thr ? ps : ps + d;
-                for (int k = 0; k < d; ++k) acc[k] += (double)x[k];
-                ps[2 * d + (t < thr ? 0 : 1)] += 1.0;
-            }
-        });
-        std::vector<double> s1(d, 0.0), s2(d, 0.0);
-        for (int64_t c = 0; c < nc; ++c) {
-            const double *ps = part.data() + (size_t)c * (2 * (size_t)d + 2);
-            for (int k = 0; k < d; ++k) {
-                s1[k] += ps[k];
-                s2[k] += ps[d + k];
-            }
-            n1 += ps[2 * d];
-            n2 += ps[2 * d + 1];
-        }
-        if (n1 == 0.0 || n2 == 0.0) break;
-        for (int k = 0; k < d; ++k) {
-            c1[k] = s1[k] / n1;
-            c2[k] = s2[k] / n2;
-        }
-    }
-    // order by side of the hyperplane, cut at the boundary (aligned)
-    std::vector<std::pair<double, int32_t>> key((size_t)len);
-    std::vector<int64_t> below(nc, 0);
-    each([&](int64_t c, int64_t b, int64_t e) {
-        for (int64_t j = b; j < e; ++j) {
-            const float *x = row(j);
-            double t = -thr;
-            for (int k = 0; k < d; ++k) t += v[k] * (double)x[k];
-            key[(size_t)j] = {t, perm[(size_t)(lo + j)]};
-            below[c] += t < 0.0 ? 1 : 0;
-        }
-    });
-    int64_t k1 = 0;
-    for (int64_t c = 0; c < nc; ++c) k1 += below[c];
-    int64_t cut = (k1 + kGroupIds / 2) / kGroupIds * kGroupIds;
-    cut = std::max<int64_t>(kGroupIds, std::min<int64_t>(cut, (len - 1) / kGroupIds * kGroupIds));
-    std::nth_element(key.begin(), key.begin() + cut, key.end());
-    for (int64_t j = 0; j < len; ++j) perm[(size_t)(lo + j)] = key[(size_t)j].second;
-    kids[0] = {lo, lo + cut, nd.depth + 1};
-    kids[1] = {lo + cut, nd.hi, nd.depth + 1};
-}
-
-}  // namespace
-
-qw_status locality_order(const float *X, int64_t n, int d, const float *A, int m,
-                         std::vector<int32_t> &perm)
-{
-    try {
-        perm.resize((size_t)n);
-        for (int64_t j = 0; j < n; ++j) perm[(size_t)j] = (int32_t)j;
-        std::vector<TreeNode> cur;
-        if (n > kGroupIds) cur.push_back({0, n, 0});
-        const int64_t big = (int64_t)1 << 16;
-        while (!cur.empty()) {
-            std::vector<TreeNode> kids(2 * cur.size());
-            // large nodes one at a time, each split on all cores ...
-            std::vector<size_t> small;
-            for (size_t u = 0; u < cur.size(); ++u) {
-                if (cur[u].hi - cur[u].lo >= big) split_node(X, d, A, m, perm, cur[u], true, &kids[2 * u]);
-                else small.push_back(u);
-            }
-            // ... small ones side by side (they touch disjoint ranges of perm)
-            parallel_chunks((int64_t)small.size(), 1, [&](int64_t c, int64_t, int64_t) {
-                const size_t u = small[(size_t)c];
-                split_node(X, d, A, m, perm, cur[u], false, &kids[2 * u]);
-            });
-            std::vector<TreeNode> next;
-            for (const TreeNode &k : kids)
-                if (k.hi - k.lo > kGroupIds) next.push_back(k);
-            cur.swap(next);
-        }
-    } catch (const std::bad_alloc &) {
-        set_error("qw_build_index: out of host memory for the locality order");
-        return QW_ERR_OOM;
-    }
     return QW_OK;
 }
 

@@ -289,11 +289,12 @@ struct BitmapLayout {
     int64_t total = 0;           // bitmaps
 };
 qw_status bitmap_layout(const std::vector<int32_t> &span, int nT, int c, BitmapLayout *out);
-// Internal order of the bitmaps: a two-means tree over the data (host
-// copies X n x d, A m x d), leaves of at most kGroupIds ids aligned to groups.
+// Internal order of the bitmaps (qw_tree.cu): a two-means tree over the data X
+// (n x d, device) seeded along the directions A (m x d, device), leaves of at
+// most kGroupIds ids aligned to groups; perm (device, n) receives the order.
 constexpr int kGroupIds = 128;
-qw_status locality_order(const float *X, int64_t n, int d, const float *A, int m,
-                         std::vector<int32_t> &perm);
+qw_status locality_order(const float *X, int64_t n, int d, const float *A, int m, int32_t *perm,
+                         cudaStream_t s);
 qw_status launch_bitmap_build(const IndexView &ix, int c, int maxJ, const int32_t *Ht, uint4 *bm,
                               uint32_t *bm_sum, int64_t total_bitmaps, cudaStream_t s);
 qw_status launch_bid_prefix(const IndexView &ix, int64_t *prefix, const int64_t *off,
