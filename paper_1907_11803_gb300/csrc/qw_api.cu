@@ -533,7 +533,7 @@ static qw_status build_impl(qw_index *ix, const float *data, const float *A, con
                                 cudaMemcpyHostToDevice, s));
     QW_TRY(launch_tile_sort(Ht.as<int32_t>(), n, m, nT, ix->o.as<int32_t>(), ix->lid.as<uint16_t>(),
                             ix->dir_bid.as<int32_t>(), ix->dir_off.as<int32_t>(),
-                            ix->dir_start.as<int64_t>(), ix->dir_cnt.as<int32_t>(), s));
+                            ix->dir_start.as<int64_t>(), ix->dir_cnt.as<int32_t>(), ix->span_max, s));
     {
         DevBuf acc;
         QW_TRY(acc.ensure(16));
@@ -586,10 +586,6 @@ static qw_status build_impl(qw_index *ix, const float *data, const float *A, con
         QW_TRY(ix->perm.ensure((size_t)n * sizeof(int32_t)));
         QW_TRY(locality_order(ix->X.as<float>(), n, d, ix->A.as<float>(), m,
                               ix->perm.as<int32_t>(), s));
-        QW_TRY(ix->bm_sum.ensure((size_t)lay.total * (kBmUint4 / 32) * sizeof(uint32_t)));
-        QW_TRY(launch_bitmap_build(ix->view(), ix->c, ix->bm_maxJ, Ht.as<int32_t>(),
-                                   ix->host_bitmaps ? ix->bm_host.as<uint4>() : ix->bm.as<uint4>(),
-                                   ix->bm_sum.as<uint32_t>(), lay.total, s));
         QW_TRY(ix->Xloc.ensure((size_t)n * d * sizeof(float)));
         QW_TRY(ix->inv.ensure((size_t)n * sizeof(int32_t)));
         QW_TRY(launch_locality_copy(ix->X.as<float>(), ix->perm.as<int32_t>(), n, d,
@@ -599,8 +595,11 @@ static qw_status build_impl(qw_index *ix, const float *data, const float *A, con
         ix->hloc_bytes = smax < 256 ? 1 : (smax < 65536 ? 2 : 4);
         ix->hloc_stride = (m * ix->hloc_bytes + 15) / 16 * 16;
         QW_TRY(ix->hloc.ensure((size_t)n * ix->hloc_stride));
-        QW_CUDA_TRY(cudaMemsetAsync(ix->hloc.p, 0, ix->hloc.bytes, s));
         QW_TRY(launch_hloc_build(ix->view(), Ht.as<int32_t>(), ix->hloc.p, s));
+        QW_TRY(ix->bm_sum.ensure((size_t)lay.total * (kBmUint4 / 32) * sizeof(uint32_t)));
+        QW_TRY(launch_bitmap_build(ix->view(), ix->c, ix->bm_maxJ,
+                                   ix->host_bitmaps ? ix->bm_host.as<uint4>() : ix->bm.as<uint4>(),
+                                   ix->bm_sum.as<uint32_t>(), lay.total, s));
         QW_TRY(launch_bid_prefix(ix->view(), ix->bid_prefix.as<int64_t>(),
                                  ix->prefix_off.as<int64_t>(), s));
     }

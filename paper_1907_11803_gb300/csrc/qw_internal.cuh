@@ -86,7 +86,8 @@ qw_status launch_minmax(const int32_t *Ht, int64_t n, int m, int32_t *hmin, int3
                         cudaStream_t s);
 qw_status launch_tile_sort(const int32_t *Ht, int64_t n, int m, int nT, const int32_t *o,
                            uint16_t *lid, int32_t *dir_bid, int32_t *dir_off,
-                           const int64_t *dir_start, int32_t *dir_cnt, cudaStream_t s);
+                           const int64_t *dir_start, int32_t *dir_cnt, int32_t span_max,
+                           cudaStream_t s);
 qw_status launch_export(const uint16_t *lid, const int32_t *dir_bid, const int32_t *dir_off,
                         const int64_t *dir_start, const int32_t *dir_cnt, int64_t n, int m,
                         int nT, int32_t *entry_bid, int32_t *entry_id, cudaStream_t s);
@@ -295,8 +296,7 @@ qw_status bitmap_layout(const std::vector<int32_t> &span, int nT, int c, BitmapL
 constexpr int kGroupIds = 128;
 qw_status locality_order(const float *X, int64_t n, int d, const float *A, int m, int32_t *perm,
                          cudaStream_t s);
-qw_status launch_bitmap_build(const IndexView &ix, int c, int maxJ, const int32_t *Ht, uint4 *bm,
-                              uint32_t *bm_sum, int64_t total_bitmaps, cudaStream_t s);
+qw_status launch_bitmap_build(const IndexView &ix, int c, int maxJ, uint4 *bm, uint32_t *bm_sum, int64_t total_bitmaps, cudaStream_t s);
 qw_status launch_bid_prefix(const IndexView &ix, int64_t *prefix, const int64_t *off,
                             cudaStream_t s);
 ScanStats scan_stats_of(const IndexView &ix, int c);
