@@ -172,7 +172,7 @@ typedef struct {
                              FP32 accumulation, m <= 128; see qw_hash_tc).  Same bucket ids */
     int32_t rerank_rows;  /* tile shape of the distance kernels: candidate rows a warp takes
                              at a time (2, 4 or 8; 0 = 4).  Same results */
-    int32_t tiles_per_warp; /* tile shape of the bitmap path's filter and fused kernels: id
+    int32_t tiles_per_warp; /* tile shape of the bitmap path's fused kernel: id
                              tiles a warp walks for one query (4, 8 or 16; 0 = 8).  Same
                              results */
     int32_t probes;       /* multi-probe (Section 2 on probing the neighbouring buckets of the

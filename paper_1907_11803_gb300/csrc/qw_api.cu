@@ -121,6 +121,7 @@ struct qw_index {
     DevBuf bm, bm_base, bm_nb, bm_lvl, bm_J, bid_prefix, prefix_off, perm, bm_sum, Xloc, inv, hloc;
     int hloc_bytes = 0, hloc_stride = 0;
     int bm_maxJ = 0;
+    int64_t bm_total = 0;               // level bitmaps
     float xs = 1.0f;                 // 1 / RMS coordinate of the data (start-model features)
     qw_mlp *start_model = nullptr;   // not owned
     float start_eps = 0.02f;
@@ -160,6 +161,7 @@ struct qw_index {
         v.bid_prefix = bid_prefix.as<int64_t>();
         v.perm = perm.as<int32_t>();
         v.bm_sum = bm_sum.as<uint32_t>();
+        v.bm_total = bm_total;
         v.Xloc = Xloc.as<float>();
         v.inv = inv.as<int32_t>();
         v.prefix_off = prefix_off.as<int64_t>();
@@ -544,7 +546,7 @@ static qw_status build_impl(qw_index *ix, const float *data, const float *A, con
     if (ix->bitmaps) {
         BitmapLayout lay;
         QW_TRY(bitmap_layout(h_span, nT, ix->c, &lay));
-        if (lay.total > (int64_t)INT32_MAX) {  // bitmaps are numbered in 31 bits
+        if (lay.total + nT > (int64_t)INT32_MAX) {  // bitmaps are numbered in 31 bits
             set_error("qw_build_index: bitmap table too large");
             return QW_ERR_RANGE;
         }
@@ -596,7 +598,8 @@ static qw_status build_impl(qw_index *ix, const float *data, const float *A, con
         ix->hloc_stride = (m * ix->hloc_bytes + 15) / 16 * 16;
         QW_TRY(ix->hloc.ensure((size_t)n * ix->hloc_stride));
         QW_TRY(launch_hloc_build(ix->view(), Ht.as<int32_t>(), ix->hloc.p, s));
-        QW_TRY(ix->bm_sum.ensure((size_t)lay.total * (kBmUint4 / 32) * sizeof(uint32_t)));
+        ix->bm_total = lay.total;
+        QW_TRY(ix->bm_sum.ensure((size_t)(lay.total + nT) * (kBmUint4 / 32) * sizeof(uint32_t)));
         QW_TRY(launch_bitmap_build(ix->view(), ix->c, ix->bm_maxJ,
                                    ix->host_bitmaps ? ix->bm_host.as<uint4>() : ix->bm.as<uint4>(),
                                    ix->bm_sum.as<uint32_t>(), lay.total, s));
@@ -787,11 +790,11 @@ static qw_status host_level_loop(qw_index *ix, LaunchTimer &tm, const IndexView 
             if (bitmap && loads != QW_LOADS_TMA) {
                 // the bucket numbers apart, so that QW_K_LEVEL times the filter
                 // and count passes alone
-                QW_TRY(tm.run(QW_K_BUCKET, 1, [&] {
+                QW_TRY(tm.run(QW_K_BUCKET, 2, [&] {
                     return launch_bm_level(view, nb, level, R, Rp, ix->l, ix->c, st, err, loads,
                                            s, nullptr, 1, tpw);
                 }));
-                const int nl = loads == QW_LOADS_FUSED ? 1 : (st.bm_prof ? 3 : 2);
+                const int nl = loads == QW_LOADS_FUSED ? 1 : 3;
                 QW_TRY(tm.run(QW_K_LEVEL, nl, [&] {
                     return launch_bm_level(view, nb, level, R, Rp, ix->l, ix->c, st, err, loads,
                                            s, nullptr, 2, tpw);
@@ -832,33 +835,29 @@ static qw_status host_level_loop(qw_index *ix, LaunchTimer &tm, const IndexView 
     return QW_OK;
 }
 
-// The bitmap path's two-pass work buffers for B queries: byte size, and (when
-// st is given) their places in `base`: counters; per item (query, tile) its
-// (q, t) and its m bitmap numbers (int32, rows padded to 4 entries); per group
-// a work entry and its projection mask; per (parity, item) the live-group
-// mask; per (query, projection) the bucket's bitmap number in tile 0.
+// The bitmap path's level buffers for B queries: byte size, and (when st is
+// given) their places in `base`: the level's counters; per (query, projection)
+// the bucket's bitmap number, summary row and table row; the queries that run;
+// per (parity, query, tile) the live-group mask.
 static size_t bm_work_layout(int64_t B, int nT, int m, QueryState *st, char *base = nullptr)
 {
-    const size_t items = (size_t)B * nT;
-    const size_t mpad = (size_t)(m + 3) / 4 * 4;
-    const size_t mw = (size_t)(m + 63) / 64;
+    const size_t mp = (size_t)(m + 15) / 16 * 16;
     auto up16 = [](size_t x) { return (x + 15) / 16 * 16; };
-    size_t off = 16;
-    const size_t o_qt = off;    off = up16(off + items * sizeof(int2));
-    const size_t o_bi = off;    off = up16(off + items * mpad * sizeof(int32_t));
-    const size_t o_work = off;  off = up16(off + items * kBmUint4 * sizeof(int32_t));
-    const size_t o_amask = off; off = up16(off + 2 * items * (kBmUint4 / 32) * sizeof(uint32_t));
-    const size_t o_wmask = off; off = up16(off + items * kBmUint4 * mw * 8);
-    const size_t o_bq = off;    off = up16(off + (size_t)B * m * sizeof(int64_t));
+    size_t off = 64;
+    const size_t o_b0 = off;    off = up16(off + (size_t)B * mp * sizeof(int32_t));
+    const size_t o_srow = off;  off = up16(off + (size_t)B * mp * sizeof(int32_t));
+    const size_t o_rows = off;  off = up16(off + (size_t)B * mp / 2);
+    const size_t o_run = off;   off = up16(off + (size_t)B * sizeof(int32_t));
+    const size_t o_amask = off;
+    off = up16(off + 2 * (size_t)B * nT * (kBmUint4 / 32) * sizeof(uint32_t));
     if (st && base) {
-        st->bm_nitems = reinterpret_cast<int32_t *>(base);
-        st->bm_nwork = st->bm_nitems + 1;
-        st->bm_item_qt = reinterpret_cast<int2 *>(base + o_qt);
-        st->bm_item_bi = reinterpret_cast<int32_t *>(base + o_bi);
-        st->bm_work = reinterpret_cast<int32_t *>(base + o_work);
+        st->bm_mp = (int32_t)mp;
+        st->bm_ctl = reinterpret_cast<uint32_t *>(base);
+        st->bm_b0 = reinterpret_cast<int32_t *>(base + o_b0);
+        st->bm_srow = reinterpret_cast<int32_t *>(base + o_srow);
+        st->bm_rows = reinterpret_cast<uint32_t *>(base + o_rows);
+        st->bm_run = reinterpret_cast<int32_t *>(base + o_run);
         st->bm_amask = reinterpret_cast<uint32_t *>(base + o_amask);
-        st->bm_wmask = reinterpret_cast<unsigned long long *>(base + o_wmask);
-        st->bm_bq = reinterpret_cast<int64_t *>(base + o_bq);
     }
     return off;
 }
@@ -938,9 +937,8 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
     const int rr_rows = qp && qp->rerank_rows ? qp->rerank_rows : 4;
     // bitmap path, per query: two levels of (tile) candidate bitmaps and lists
     const int64_t cb_bytes = (int64_t)ix->nT * kBmUint4 * (int64_t)sizeof(uint4) * 2;
-    // (per query: two levels of tile candidate counts and candidate lists)
-    const int64_t cl_bytes = (int64_t)ix->nT * (int64_t)sizeof(int32_t) * 2 +
-                             ((int64_t)kQCap * (int64_t)sizeof(uint64_t) + 4) * 2;
+    // (per query: its candidate list, two levels' candidate numbers)
+    const int64_t cl_bytes = (int64_t)kQCap * (int64_t)sizeof(uint64_t) + 4 * 2;
     int64_t B = qp && qp->batch > 0 ? qp->batch : 0;
     if (B == 0 && ix->tuned && ix->tuned_batch > 0 && !use_cluster &&
         (path == QW_PATH_AUTO || path == ix->tuned_path))
@@ -956,7 +954,7 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
     }
     B = std::min<int64_t>(B, std::max<int64_t>(nq, 1));
     B = std::min<int64_t>(B, 65535);
-    // bitmap path: (query, tile) item slots are numbered in 23 bits
+    // bitmap path: the live groups of a level are counted in 32 bits
     if (use_bitmap) B = std::max<int64_t>(1, std::min<int64_t>(B, ((int64_t)1 << 23) / ix->nT));
     auto up16 = [](size_t x) { return (x + 15) / 16 * 16; };
 
@@ -973,8 +971,6 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
                                   (size_t)B * sizeof(RdPlan) +
                                   (size_t)B * 2 * kHistBins * sizeof(int32_t) +
                                   (size_t)B * 2 * QW_MAX_M * sizeof(int64_t)));
-        // two-pass level: one slot per (query, tile), one work entry per group
-        const size_t items = (size_t)B * ix->nT;
         QW_TRY(ix->w_bmwork.ensure(bm_work_layout(B, ix->nT, m, nullptr)));
         // the overflow rebuild's plane store: one wave of slots
         QW_TRY(ix->w_rdstore.ensure((size_t)std::min<int64_t>(B, bm_reduce_wave(ix->nT)) *
@@ -1066,13 +1062,11 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
     st.level_passes = nullptr;
     st.cb_par = B * ix->nT * kBmUint4;
     if (use_bitmap) {
-        // w_clist: qbuf (2 x B x kQCap), then clist_n (2 x B x nT), then qbuf_n (2 x B)
-        st.qb_par = B * (int64_t)kQCap;
+        // w_clist: qbuf (B x kQCap), then qbuf_n (2 x B)
         st.qbuf = ix->w_clist.as<uint64_t>();
         st.cln_par = B * ix->nT;
-        st.clist_n = reinterpret_cast<int32_t *>(st.qbuf + 2 * st.qb_par);
         st.qbn_par = B;
-        st.qbuf_n = st.clist_n + 2 * st.cln_par;
+        st.qbuf_n = reinterpret_cast<int32_t *>(st.qbuf + B * (int64_t)kQCap);
         st.bm_ovf = ix->w_bmsel.as<int32_t>();
         st.recount = st.bm_ovf + B;
         st.eqbuf = st.bm_ovf + 2 * B;
@@ -1089,10 +1083,7 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
             st.rd_bq = reinterpret_cast<int64_t *>((a + 15) & ~(uintptr_t)15);
         }
         st.rd_store = ix->w_rdstore.as<uint4>();
-        const int64_t items = B * (int64_t)ix->nT;
         bm_work_layout(B, ix->nT, m, &st, ix->w_bmwork.as<char>());
-        st.bm_item_cap = (int32_t)std::min<int64_t>(items, (int64_t)1 << 23);
-        st.bm_work_cap = (int32_t)std::min<int64_t>(items * kBmUint4, INT32_MAX);
     }
     // two counters, then the two lists of queries to answer again
     int32_t *ovf_count = use_bitmap ? ix->w_ovf.as<int32_t>() : nullptr;
@@ -1279,14 +1270,15 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
                 QW_TRY(host_level_loop(ix, tm, view, nb, cap, learned, use_bitmap, loads, tpw, err,
                                        st, s, &levels_run));
             }
-            QW_TRY(tm.run(QW_K_SELECT, use_bitmap ? (learned ? 4 : 2) : 2, [&] {
-                if (use_bitmap)
-                    QW_TRY(launch_bm_reduce(view, nb, ix->l, cap, ix->c, st, tma_loads,
+            QW_TRY(tm.run(QW_K_SELECT, use_bitmap ? (learned ? 5 : 3) : 2, [&] {
+                if (use_bitmap) {
+                    QW_TRY(launch_bm_list(view, nb, ix->l, st, tma_loads, s));
+                    QW_TRY(launch_bm_reduce(view, nb, ix->l, cap, ix->c, st,
                                             (int)std::min<int64_t>(B, bm_reduce_wave(ix->nT)), s));
-                if (use_bitmap && learned)
-                    QW_TRY(launch_bm_recount(view, nb, ix->l, cap, ix->c, st, s));
-                return use_bitmap ? launch_bm_collect(view, nb, ix->l, cap, st, stats_b, want_cand, s)
-                                  : launch_collect(view, nb, ix->l, cap, st, stats_b, s);
+                    if (learned) QW_TRY(launch_bm_recount(view, nb, ix->l, cap, ix->c, st, s));
+                    return launch_bm_collect(view, nb, ix->l, cap, st, stats_b, want_cand, s);
+                }
+                return launch_collect(view, nb, ix->l, cap, st, stats_b, s);
             }));
             if (use_bitmap)
                 QW_TRY(launch_bm_overflow_list(st, nb, order ? perm : nullptr, b0, ovf_list,
@@ -1368,11 +1360,11 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
             set_error("qw_run_workload: a staged-copy wait in the bitmap kernel gave up");
             return QW_ERR_TIMEOUT;
         }
-        // per level: the bucket numbers, filter and count (bitmap path, direct
+        // per level: the bucket numbers, filter and both counts (bitmap path, direct
         // loads), else one counting launch
         ix->prof.launches[QW_K_LEVEL] +=
             (int64_t)h_ctl.iters *
-            (use_bitmap && loads == QW_LOADS_DIRECT ? 3 : (use_bitmap && loads == QW_LOADS_FUSED ? 2 : 1));
+            (use_bitmap && loads == QW_LOADS_DIRECT ? 5 : (use_bitmap && loads == QW_LOADS_FUSED ? 3 : 1));
         levels_run = (int)h_ctl.iters;
         ix->prof.launches[QW_K_DECIDE] += 2 * (int64_t)h_ctl.iters + n_batches * (learned ? 3 : 1);
         if (learned) {
@@ -1657,8 +1649,7 @@ qw_status qw_autotune(qw_index *ix, const float *queries, int64_t nq, int32_t k,
                 if (status != QW_OK) break;
             }
             const int64_t cb_b = (int64_t)ix->nT * kBmUint4 * (int64_t)sizeof(uint4) * 2 +
-                                 (int64_t)ix->nT * (int64_t)sizeof(int32_t) * 2 +
-                                 ((int64_t)kQCap * (int64_t)sizeof(uint64_t) + 4) * 2;
+                                 (int64_t)kQCap * (int64_t)sizeof(uint64_t) + 4 * 2;
             const int64_t bdef = std::min<int64_t>(
                 std::min<int64_t>(std::max<int64_t>(1, kBitmapBudget / cb_b), nq), 65535);
             const int64_t bc[2] = {bdef / 16, bdef / 4};

@@ -144,15 +144,24 @@ __global__ void locality_copy_kernel(const float *__restrict__ X, const int32_t 
     }
 }
 
-// Per bitmap, one bit per 128-id group: the group has at least one id.
-__global__ void __launch_bounds__(BM_THREADS) bm_summary_kernel(const uint4 *__restrict__ bm,
-                                                                int64_t total,
+// Per bitmap, one bit per 128-id group: the group has at least one id.  The
+// summaries of one bucket over the tiles lie side by side (row bm_base[i] +
+// k * nT + t for bitmap k of tile t's block of projection i), so that the
+// filter reads four tiles of a bucket as one 128-byte line; nT zero rows at
+// the end stand for buckets without data.
+__global__ void __launch_bounds__(BM_THREADS) bm_summary_kernel(IndexView ix,
+                                                                const uint4 *__restrict__ bm,
                                                                 uint32_t *__restrict__ sum)
 {
-    for (int64_t b = blockIdx.x; b < total; b += gridDim.x) {
-        const uint4 v = bm[b * kBmUint4 + threadIdx.x];
+    const int t = blockIdx.x, i = blockIdx.y;
+    const int nbk = ix.bm_nb[i];
+    const int64_t b0 = ix.bm_base[i] + (int64_t)t * nbk;
+    for (int k = 0; k < nbk; ++k) {
+        const uint4 v = bm[(b0 + k) * kBmUint4 + threadIdx.x];
         const uint32_t word = __ballot_sync(0xffffffffu, (v.x | v.y | v.z | v.w) != 0);
-        if ((threadIdx.x & 31) == 0) sum[b * (kBmUint4 / 32) + (threadIdx.x >> 5)] = word;
+        if ((threadIdx.x & 31) == 0)
+            sum[(ix.bm_base[i] + (int64_t)k * ix.nT + t) * (kBmUint4 / 32) + (threadIdx.x >> 5)] =
+                word;
     }
 }
 
@@ -268,27 +277,6 @@ __device__ __forceinline__ uint4 candidates_of(const Planes &P, int l)
     return cand;
 }
 
-// Append this thread's candidates (128 ids, ascending) to the query's list
-// for the level from position pos: (internal id << 32) | (prev << 8) | count.
-__device__ __forceinline__ void append_candidates(const Planes &P, const uint4 &cand,
-                                                  const uint4 &prev, uint64_t *list, int pos,
-                                                  int64_t id_base)
-{
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        uint32_t x = word_of(cand, w);
-        const uint32_t pw = word_of(prev, w);
-        while (x) {
-            const int b = __ffs(x) - 1;
-            x &= x - 1;
-            if (pos < kQCap)
-                list[pos] = ((uint64_t)(id_base + w * 32 + b) << 32) |
-                            ((uint64_t)((pw >> b) & 1u) << 8) | (uint64_t)count_of(P, w, b);
-            ++pos;
-        }
-    }
-}
-
 // Bitmap number of the level-`level` bucket beta of projection i in tile t,
 // or -1 when the bucket holds no data (beta below zero or past the span).
 // Past the last stored level a single bucket (beta == 0) holds every id.
@@ -308,43 +296,261 @@ __device__ __forceinline__ int64_t bm_index(const IndexView &ix, int i, int t, i
 
 // ---- the same level in two passes (the bitmap path's default)
 //
-// Pass 1, one warp per (query, tile), the tasks taken tile-major (a wave of
-// warps covers one run of tiles for many queries, whose bucket bitmaps then
-// serve all of them from L2): only the bucket summaries are read (8
-// words of 32 bits per projection, one bit per 128-id group), and a carry-save
-// sum over the m projections gives every group the number of the query's
-// buckets that touch it.  Groups below l cannot hold a candidate.  A tile
-// without live groups is done (its candidate count is 0); otherwise its live
-// groups are recorded (a 256-bit mask: only their candidate words are written
-// at this level), the item's m bitmap numbers are stored in a slot, and its
-// live groups go to a work list.
-// Pass 2, one thread per live group: the 128-id group's word of each of the
-// m bitmaps, summed into bit planes; the group's candidates (count >= l) are
-// written to the tile's candidate bitmap and the query's list.
+// Pass 1 (bm_filter_kernel) reads only the bucket summaries (one bit per 128-id
+// group): a bit-sliced sum over the m projections gives every group the number
+// of the query's buckets that touch it, and the groups touched by at least l of
+// them are live: no other can hold a candidate.  Each (query, tile)'s 256
+// live bits are written (bm_amask) and their number summed over the level.
+// Pass 2 counts the live groups from the bitmaps, in one of two forms chosen on
+// the device from that number (both are launched, one returns at once):
+//   bm_count_kernel, few queries per group: a warp takes one query's live
+//     groups of four tiles, one per lane, and each lane reads the m words of its
+//     group from the bitmaps;
+//   bm_dense_kernel, many queries per group: a block keeps the words of every
+//     bucket of a few groups in shared memory and counts them for every query
+//     whose group is live.
+// Both write the candidate word of a group with candidates (count >= l), add its
+// candidates to the query's count, and clear the live bit of a group without:
+// the bit then says that the group's word was written at this level.  Only a
+// query's last level needs its candidates one by one, with their counts: they
+// are listed after the loop (bm_list_kernel).
 constexpr int FL_WARPS = 8;                   // warps per block in pass 1
 constexpr int kSumWords = kBmUint4 / 32;      // summary words per bitmap (8)
 
-// Before pass 1, per (query, projection): the bitmap number of the query's
-// bucket at this level in tile 0 (tile t adds t * bm_nb[i]), or -1 when the
-// bucket holds no data.  Also clears the pass's item and work counters.
-__global__ void bm_bucket_kernel(IndexView ix, int level, int64_t R, int nb, QueryState st,
-                                 const LoopCtl *ctl)
+// The dense form's table of one group: for every projection S rows of 16 bytes,
+// the words of its buckets at the level, then zeros; S, a power of two, is above
+// the most buckets of any projection, so row S - 1 is zero and stands for
+// buckets without data.  A query names its rows in 4 bits each.
+constexpr int kDenseTable = 66 * 1024;       // bytes of tables per block
+constexpr int kDenseGroups = 16;             // most groups per block
+constexpr int kDenseMin = 256;               // live groups per group of the index
+
+// Per level, in st.bm_ctl: [0] live groups, [1] the dense form's next unit,
+// [2] S (0: more than 15 buckets), [3] groups per block, [4] queries that run.
+enum { kCtlLive = 0, kCtlUnit = 1, kCtlRows = 2, kCtlGroups = 3, kCtlRun = 4 };
+
+// The dense form pays when a group's table is read often enough: its words are
+// loaded once per block instead of once per query.  The line lies where both
+// forms take the same time: with 223 live groups per group of the index 112 us
+// dense against 99, with 387 320 against 304, with 646 155 against 183, with
+// 1,211 609 against 906, with 1,762 2.4 ms against 3.6.
+__device__ __forceinline__ bool dense_level(const IndexView &ix, const QueryState &st)
+{
+    return st.bm_ctl[kCtlRows] > 0 &&
+           st.bm_ctl[kCtlLive] >= (uint32_t)kDenseMin * (uint32_t)ix.nT * kBmUint4;
+}
+
+// Buckets of projection i at a level (one past the last stored level).
+__device__ __forceinline__ int buckets_at(const IndexView &ix, int i, int level, int64_t R)
+{
+    return level > ix.bm_J[i] ? 1 : (int)((int64_t)ix.span[i] / R + 1);
+}
+
+// 16-byte words of a group's table (odd: the groups start in different banks).
+__device__ __forceinline__ int table_words(int mp, int S) { return mp * S + 1; }
+
+// The bucket of entry (query of the list at place e / bm_mp, projection e %
+// bm_mp): its bitmap number at this level in tile 0 (tile t adds t * bm_nb[i];
+// -1 when the bucket holds no data), its summary row (the zero rows then), and
+// its row in the dense form's table (S - 1 then).  Rows are padded with empty
+// buckets to multiples of 16 projections; eight lanes pack a word of table rows.
+__device__ __forceinline__ void bucket_entry(const IndexView &ix, const QueryState &st, int level,
+                                             int64_t R, int S, int64_t e)
+{
+    const int m = ix.m, mp = st.bm_mp;
+    const int q = st.bm_run[e / mp], i = (int)(e % mp);
+    const int64_t at = (int64_t)q * mp + i;
+    int64_t b = -1;
+    if (i < m) b = bm_index(ix, i, 0, level, R, floordiv64(st.g[(int64_t)q * m + i], R));
+    st.bm_b0[at] = (int32_t)b;
+    st.bm_srow[at] =
+        (int32_t)(b >= 0 ? ix.bm_base[i] + (b - ix.bm_base[i]) * ix.nT : ix.bm_total);
+    if (S == 0) return;
+    uint32_t row = (uint32_t)S - 1u;
+    if (b >= 0)
+        row = (uint32_t)(b - ix.bm_base[i] - ix.bm_lvl[i * kBmLevels + min(level, ix.bm_J[i])]);
+    row <<= 4 * (threadIdx.x & 7);
+    const uint32_t mask = 0xffu << (threadIdx.x & 24);
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) row |= __shfl_xor_sync(mask, row, off);
+    if ((threadIdx.x & 7) == 0) st.bm_rows[at >> 3] = row;
+}
+
+// Before pass 1 (one block): the queries that run at this level, in order, and
+// the level's counters: the passes walk this list and not the batch, most of
+// which has stopped or not begun at most levels.  With `buckets` also their
+// buckets (small batches: one launch less); else bm_bucket_kernel follows.
+__global__ void __launch_bounds__(1024) bm_active_kernel(IndexView ix, int level, int64_t R, int nb,
+                                                         QueryState st, const LoopCtl *ctl,
+                                                         bool buckets)
+{
+    __shared__ int tmp[32];
+    __shared__ int s_most;
+    if (ctl) {
+        level = ctl->level;
+        R = ctl->R;
+    }
+    if (threadIdx.x == 0) s_most = 0;
+    __syncthreads();
+    if ((int)threadIdx.x < ix.m) atomicMax(&s_most, buckets_at(ix, threadIdx.x, level, R));
+    constexpr int E = 8;
+    int run = 0;
+    for (int q0 = 0; q0 < nb; q0 += 1024 * E) {
+        const int q1 = q0 + (int)threadIdx.x * E;
+        uint32_t on = 0;
+#pragma unroll
+        for (int u = 0; u < E; ++u)
+            if (q1 + u < nb && st.active[q1 + u] && level >= st.start[q1 + u]) on |= 1u << u;
+        int total;
+        int at = run + block_exclusive_scan<1024>(__popc(on), tmp, &total);
+#pragma unroll
+        for (int u = 0; u < E; ++u)
+            if ((on >> u) & 1u) st.bm_run[at++] = q1 + u;
+        run += total;
+    }
+    __syncthreads();
+    const int S = s_most < 4 ? 4 : (s_most < 8 ? 8 : (s_most < 16 ? 16 : 0));
+    if (threadIdx.x == 0) {
+        int G = kDenseGroups;
+        while (G > 2 && table_words(st.bm_mp, S) * 16 * G > kDenseTable) G >>= 1;
+        st.bm_ctl[kCtlLive] = 0;
+        st.bm_ctl[kCtlUnit] = 0;
+        st.bm_ctl[kCtlRows] = S;
+        st.bm_ctl[kCtlGroups] = G;
+        st.bm_ctl[kCtlRun] = run;
+    }
+    if (buckets)
+        for (int64_t e = threadIdx.x; e < (int64_t)run * st.bm_mp; e += 1024)
+            bucket_entry(ix, st, level, R, S, e);
+}
+
+__global__ void __launch_bounds__(256) bm_bucket_kernel(IndexView ix, int level, int64_t R,
+                                                        QueryState st, const LoopCtl *ctl)
 {
     if (ctl) {
         level = ctl->level;
         R = ctl->R;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        st.bm_nitems[0] = 0;
-        st.bm_nwork[0] = 0;
+    const int S = (int)st.bm_ctl[kCtlRows];
+    const int64_t total = (int64_t)st.bm_ctl[kCtlRun] * st.bm_mp;
+    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * 256)
+        bucket_entry(ix, st, level, R, S, e);
+}
+
+// Eight one-bit inputs per lane bit added to one word's planes p[0..7).
+__device__ __forceinline__ void add8_word(uint32_t (&p)[7], const uint32_t (&x)[8])
+{
+    uint32_t t2a, t2b, t4a, t4b, t8;
+    csa(t2a, p[0], p[0], x[0], x[1]);
+    csa(t2b, p[0], p[0], x[2], x[3]);
+    csa(t4a, p[1], p[1], t2a, t2b);
+    csa(t2a, p[0], p[0], x[4], x[5]);
+    csa(t2b, p[0], p[0], x[6], x[7]);
+    csa(t4b, p[1], p[1], t2a, t2b);
+    csa(t8, p[2], p[2], t4a, t4b);
+    uint32_t cy = t8, nx;
+    nx = p[3] & cy; p[3] ^= cy; cy = nx;
+    nx = p[4] & cy; p[4] ^= cy; cy = nx;
+    nx = p[5] & cy; p[5] ^= cy; cy = nx;
+    p[6] ^= cy;  // counts stay below 128
+}
+
+// One warp per (query, four tiles), tasks tile-major: the warps of a wave take
+// the same tiles for many queries, whose summaries (and then bitmaps) serve all
+// of them from L2.  Lane = (tile, summary word): the m summary words of a lane
+// are summed bit-sliced, the four tiles of a bucket being one 128-byte line, and
+// the compare gives the word's live groups.  Issue bound: about 6.5
+// instructions per projection and four tiles.  (One warp per tile with a bit
+// transpose of every word, for each group's own list of projections, issued
+// about 30: 2,638 us per call on 3 million points and 10,000 queries, 584 so.)
+__global__ void __launch_bounds__(FL_WARPS * 32) bm_filter_kernel(IndexView ix, int level, int l,
+                                                                  QueryState st, const LoopCtl *ctl)
+{
+    if (ctl) level = ctl->level;
+    const int lane = threadIdx.x & 31;
+    const int nT = ix.nT, mp = st.bm_mp;
+    const int par = level & 1;
+    const int run = (int)st.bm_ctl[kCtlRun];
+    const int64_t tasks = (int64_t)run * ((nT + 3) >> 2);
+    uint32_t live = 0;
+    unsigned long long items = 0, words = 0;
+    for (int64_t k = (int64_t)blockIdx.x * FL_WARPS + (threadIdx.x >> 5); k < tasks;
+         k += (int64_t)gridDim.x * FL_WARPS) {
+        const int q = st.bm_run[k % run], t0 = (int)(k / run) * 4;
+        const int t = t0 + (lane >> 3);
+        // lanes past the last tile read its row again
+        const int in_row = (min(t, nT - 1) - t0) * kSumWords + (lane & 7);
+        const int4 *rows = reinterpret_cast<const int4 *>(st.bm_srow + (int64_t)q * mp);
+        const uint32_t *sum = ix.bm_sum + (int64_t)t0 * kSumWords + in_row;
+        uint32_t P[7] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 2
+        for (int i = 0; i < mp; i += 8) {
+            const int4 ra = __ldg(rows + (i >> 2)), rb = __ldg(rows + (i >> 2) + 1);
+            const int32_t r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+            uint32_t x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = __ldg(sum + (int64_t)r[u] * kSumWords);
+            add8_word(P, x);
+        }
+        uint32_t gt = 0, eq = 0xffffffffu;
+#pragma unroll
+        for (int b = 6; b >= 0; --b) {
+            if ((l >> b) & 1) {
+                eq &= P[b];
+            } else {
+                gt |= eq & P[b];
+                eq &= ~P[b];
+            }
+        }
+        const uint32_t alive = t < nT ? gt | eq : 0u;
+        if (t < nT)
+            st.bm_amask[((int64_t)par * st.cln_par + (int64_t)q * nT + t0) * kSumWords + lane] = alive;
+        live += __popc(alive);
+        if (st.bm_prof) {
+            // tiles with live groups; words of the buckets touching live groups
+            const uint32_t any = __ballot_sync(0xffffffffu, alive != 0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) items += (any >> (8 * u)) & 0xffu ? 1 : 0;
+#pragma unroll
+            for (int b = 0; b < 7; ++b) words += (unsigned)__popc(alive & P[b]) << b;
+        }
     }
-    const int m = ix.m;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)nb * m;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int q = (int)(e / m), i = (int)(e % m);
-        if (!st.active[q] || level < st.start[q]) continue;
-        st.bm_bq[e] = bm_index(ix, i, 0, level, R, floordiv64(st.g[e], R));
+    live = __reduce_add_sync(0xffffffffu, live);
+    if (lane == 0 && live) atomicAdd(st.bm_ctl + kCtlLive, live);
+    if (st.bm_prof) {
+        words = __reduce_add_sync(0xffffffffu, (unsigned)words);
+        if (lane == 0 && live) {
+            atomicAdd(st.bm_prof + 0, items);
+            atomicAdd(st.bm_prof + 1, (unsigned long long)live);
+            atomicAdd(st.bm_prof + 2, words);
+        }
     }
+}
+
+// What follows the count of a group with nc > 0 candidates.
+__device__ __forceinline__ void emit_group(const QueryState &st, int nT, int level, int q, int t,
+                                           int g, const uint4 &cand, int nc)
+{
+    const int64_t qt = (int64_t)q * nT + t;
+    st.cbits[(int64_t)(level & 1) * st.cb_par + qt * kBmUint4 + g] = cand;
+    atomicAdd(st.qbuf_n + (int64_t)(level & 1) * st.qbn_par + q, nc);
+}
+
+// Position of the n-th (0-based) set bit of v; n < popc(v).
+__device__ __forceinline__ int nth_set_bit(uint32_t v, int n)
+{
+    int pos = 0;
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) {
+        const int c = __popc(v & ((1u << w) - 1u));
+        if (n >= c) {
+            n -= c;
+            v >>= w;
+            pos += w;
+        }
+    }
+    return pos;
 }
 
 // Bit transpose of a 32 x 32 block held one row per lane (bit b of lane i's
@@ -364,219 +570,364 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t a, int lane)
     return a;
 }
 
-// One warp per (query, run of FL_TILES tiles).  Lane j holds the summaries of
-// projections j, j + 32, ... (32 bytes each, two vector loads; the next tile's
-// are loaded while the current one is counted).  For each summary word, the
-// bit transpose of the lanes' rows gives lane g the projections touching group
-// w * 32 + g: their number decides whether the group is live, and the same
-// bits are the group's projection mask for pass 2.
-constexpr int FL_TILES = 8;  // tiles per warp unless the caller picks 4 or 16
+// The set bits of a warp's 32 words x (one per lane), 32 at a time: f(owner,
+// bit, valid) per lane for the entries in order (lanes past the last repeat it,
+// not valid).  With at most 8 of them in all, four lanes take each entry: f's
+// last argument is then the lane's share (0..3 of 4), else 0 of 1, and lane
+// share 0 is the valid one.
+template <class F>
+__device__ __forceinline__ void each_set_bit(uint32_t x, int lane, F &&f)
+{
+    int incl = __popc(x);
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    const bool four = total <= 8;
+    for (int r0 = 0; r0 < total; r0 += 32) {
+        // the (r0 + lane)-th set bit: the first word whose prefix passes it
+        const int e = min(four ? lane >> 2 : r0 + lane, total - 1);
+        int own = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+            const int v = __shfl_sync(0xffffffffu, incl, own + step - 1);
+            if (e >= v) own += step;
+        }
+        const uint32_t xw = __shfl_sync(0xffffffffu, x, own);
+        const int before = __shfl_sync(0xffffffffu, incl, own) - __popc(xw);
+        f(own, nth_set_bit(xw, e - before),
+          four ? (lane >> 2) < total && (lane & 3) == 0 : r0 + lane < total, four);
+    }
+}
 
-template <int NROW>
-__device__ __forceinline__ void load_summaries(const IndexView &ix, const int64_t (&b0)[NROW],
-                                               const int32_t (&nbp)[NROW], int t,
-                                               uint4 (&sv)[NROW][2])
+// Add the planes of another lane (lane ^ off) to this one's.
+__device__ __forceinline__ void add_lane(Planes &P, int off)
 {
 #pragma unroll
-    for (int r = 0; r < NROW; ++r) {
-        if (b0[r] >= 0) {
-            const uint4 *p = reinterpret_cast<const uint4 *>(
-                ix.bm_sum + (b0[r] + (int64_t)t * nbp[r]) * kSumWords);
-            sv[r][0] = __ldg(p);
-            sv[r][1] = __ldg(p + 1);
-        } else {
-            sv[r][0] = make_uint4(0, 0, 0, 0);
-            sv[r][1] = make_uint4(0, 0, 0, 0);
+    for (int w = 0; w < 4; ++w) {
+        uint32_t cy = 0;
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+            const uint32_t o = __shfl_xor_sync(0xffffffffu, P.s[k][w], off);
+            csa(cy, P.s[k][w], P.s[k][w], o, cy);
         }
     }
 }
 
-template <int NROW, int TPW>
-__global__ void __launch_bounds__(FL_WARPS * 32, NROW <= 2 ? 3 : 2) bm_filter_kernel(IndexView ix, int level, int l,
-                                                                  int nb, QueryState st,
-                                                                  const LoopCtl *ctl)
+// Count planes of group g of tile t from the m bitmaps whose numbers in tile 0
+// are b0[0..m) (-1: no data; tile t adds t * nbs[i]), rows padded to 8.  With
+// `four` (uniform over the warp) the four lanes of a quad have the same group and
+// each reads every fourth run of eight projections: a quarter of the dependent
+// rounds of loads where the warp's other lanes would idle.
+__device__ __forceinline__ void count_planes(const IndexView &ix, const int32_t *b0,
+                                             const int *nbs, int t, int g, Planes &P,
+                                             bool four = false)
 {
-    constexpr int MW = (NROW + 1) / 2;
-    // per warp: the projection masks of the current tile's groups
-    __shared__ unsigned long long wmk[FL_WARPS][kSumWords][MW][32];
+#pragma unroll
+    for (int kk = 0; kk < 7; ++kk)
+#pragma unroll
+        for (int w = 0; w < 4; ++w) P.s[kk][w] = 0;
+    const int4 *b4 = reinterpret_cast<const int4 *>(b0);
+    const int step = four ? 32 : 8;
+    for (int i0 = four ? 8 * (threadIdx.x & 3) : 0; i0 < ix.m; i0 += step) {
+        const int4 ba = __ldg(b4 + (i0 >> 2)), bb = __ldg(b4 + (i0 >> 2) + 1);
+        const int32_t bn[8] = {ba.x, ba.y, ba.z, ba.w, bb.x, bb.y, bb.z, bb.w};
+        uint4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            v[u] = bn[u] >= 0
+                       ? __ldg(ix.bm + ((int64_t)bn[u] + (int64_t)t * nbs[i0 + u]) * kBmUint4 + g)
+                       : make_uint4(0, 0, 0, 0);
+        add8(P, v);
+    }
+    if (four) {
+        add_lane(P, 1);
+        add_lane(P, 2);
+    }
+}
+
+// Few queries per group.  A warp takes the live bits of one query's four tiles
+// (a word per lane), and its lanes the set bits, 32 at a time: a lane reads its
+// group's word of each of the query's m bitmaps and sums them into bit planes.
+// Bound by the latency of those 16-byte reads (about 20 sectors a request): see
+// bm_dense_kernel for levels where many queries share a group.
+__global__ void __launch_bounds__(256, 3) bm_count_kernel(IndexView ix, int level, int l,
+                                                          QueryState st, const LoopCtl *ctl)
+{
+    __shared__ int s_nb[QW_MAX_M + 16];
+    __shared__ uint32_t s_keep[8][32];
+    if (dense_level(ix, st)) return;
     if (ctl) level = ctl->level;
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    const int m = ix.m, nT = ix.nT;
-    const int mw = (m + 63) >> 6;
-    const int nch = (nT + TPW - 1) / TPW;
-    const int64_t tasks = (int64_t)nb * nch;
-    const int par = level & 1;
-    for (int64_t k = (int64_t)blockIdx.x * FL_WARPS + (threadIdx.x >> 5); k < tasks;
-         k += (int64_t)gridDim.x * FL_WARPS) {
-        // tile-major: the warps of a wave take one run of tiles for many
-        // queries, so the bitmaps they touch (and the count pass after them)
-        // stay in L2 across queries
-        const int q = (int)(k % nb);
-        const int t0 = (int)(k / nb) * TPW, t1 = min(nT, t0 + TPW);
-        if (!st.active[q] || level < st.start[q]) continue;
-        int64_t b0[NROW];
-        int32_t nbp[NROW];
-#pragma unroll
-        for (int r = 0; r < NROW; ++r) {
-            const int i = lane + 32 * r;
-            b0[r] = i < m ? st.bm_bq[(int64_t)q * m + i] : -1;
-            nbp[r] = i < m ? ix.bm_nb[i] : 0;
-        }
-        uint4 sv[NROW][2];
-        load_summaries<NROW>(ix, b0, nbp, t0, sv);
-        for (int t = t0; t < t1; ++t) {
-            uint4 cur[NROW][2];
-#pragma unroll
-            for (int r = 0; r < NROW; ++r) {
-                cur[r][0] = sv[r][0];
-                cur[r][1] = sv[r][1];
+    const int m = ix.m, nT = ix.nT, mp = st.bm_mp;
+    for (int i = threadIdx.x; i < mp; i += 256) s_nb[i] = i < m ? ix.bm_nb[i] : 0;
+    __syncthreads();
+    const int run = (int)st.bm_ctl[kCtlRun];
+    const int64_t tasks = (int64_t)run * ((nT + 3) >> 2);
+    for (int64_t k = (int64_t)blockIdx.x * 8 + wi; k < tasks; k += (int64_t)gridDim.x * 8) {
+        const int q = st.bm_run[k % run], t0 = (int)(k / run) * 4;
+        uint32_t *am = st.bm_amask +
+                       ((int64_t)(level & 1) * st.cln_par + (int64_t)q * nT + t0) * kSumWords + lane;
+        const uint32_t x = t0 + (lane >> 3) < nT ? *am : 0u;
+        if (!__any_sync(0xffffffffu, x != 0)) continue;
+        s_keep[wi][lane] = x;
+        __syncwarp();
+        each_set_bit(x, lane, [&](int own, int bit, bool valid, bool four) {
+            const int t = t0 + (own >> 3), g = (own & 7) * 32 + bit;
+            Planes P;
+            count_planes(ix, st.bm_b0 + (int64_t)q * mp, s_nb, t, g, P, four);
+            const uint4 cand = candidates_of(P, l);
+            const int nc = __popc(cand.x) + __popc(cand.y) + __popc(cand.z) + __popc(cand.w);
+            if (valid) {
+                if (nc == 0) atomicAnd(&s_keep[wi][own], ~(1u << bit));
+                else emit_group(st, nT, level, q, t, g, cand, nc);
             }
-            if (t + 1 < t1) load_summaries<NROW>(ix, b0, nbp, t + 1, sv);
-            const int64_t qt = (int64_t)q * nT + t;
-            uint32_t x[kSumWords];
-            int n_alive = 0;
-#pragma unroll
-            for (int w = 0; w < kSumWords; ++w) {
-                int cnt = 0;
-                unsigned long long mk[MW];
-#pragma unroll
-                for (int h = 0; h < MW; ++h) mk[h] = 0ull;
-#pragma unroll
-                for (int r = 0; r < NROW; ++r) {
-                    const uint32_t c = transpose32(word_of(cur[r][w >> 2], w & 3), lane);
-                    cnt += __popc(c);
-                    mk[r >> 1] |= (unsigned long long)c << (32 * (r & 1));
-                }
-#pragma unroll
-                for (int h = 0; h < MW; ++h) wmk[wi][w][h][lane] = mk[h];
-                x[w] = __ballot_sync(0xffffffffu, cnt >= l);
-                n_alive += __popc(x[w]);
-            }
-            if (lane == 0) st.clist_n[(int64_t)par * st.cln_par + qt] = 0;
-            if (n_alive == 0) continue;
-            // which groups have a candidate word at this level
-            uint32_t xl = 0;
-#pragma unroll
-            for (int w = 0; w < kSumWords; ++w) xl = lane == w ? x[w] : xl;
-            if (lane < kSumWords) st.bm_amask[((int64_t)par * st.cln_par + qt) * kSumWords + lane] = xl;
-            int slot = 0, base = 0;
-            if (lane == 0) {
-                slot = atomicAdd(st.bm_nitems, 1);
-                base = atomicAdd(st.bm_nwork, n_alive);
-            }
-            slot = __shfl_sync(0xffffffffu, slot, 0);
-            base = __shfl_sync(0xffffffffu, base, 0);
-            if (slot >= st.bm_item_cap) continue;
-            const int mpad = (m + 3) & ~3;
-#pragma unroll
-            for (int r = 0; r < NROW; ++r)
-                if (lane + 32 * r < mpad)
-                    st.bm_item_bi[(int64_t)slot * mpad + lane + 32 * r] =
-                        b0[r] >= 0 ? (int32_t)(b0[r] + (int64_t)t * nbp[r]) : -1;
-            if (lane == 0) st.bm_item_qt[slot] = make_int2(q, t);
-            // live groups of the tile, in ascending order, after `base`
-            int pos = base, words = 0;
-#pragma unroll
-            for (int w = 0; w < kSumWords; ++w) {
-                if ((x[w] >> lane) & 1u) {
-                    const int at = pos + __popc(x[w] & ((1u << lane) - 1u));
-                    if (at < st.bm_work_cap) {
-                        st.bm_work[at] = (slot << 8) | (w * 32 + lane);
-#pragma unroll
-                        for (int h = 0; h < MW; ++h)
-                            if (h < mw) {
-                                const unsigned long long mk = wmk[wi][w][h][lane];
-                                st.bm_wmask[(int64_t)at * mw + h] = mk;
-                                words += __popcll(mk);
-                            }
-                    }
-                }
-                pos += __popc(x[w]);
-            }
-            if (st.bm_prof) {
-                words = __reduce_add_sync(0xffffffffu, words);
-                if (lane == 0) atomicAdd(st.bm_prof + 2, (unsigned long long)words);
-            }
-        }
+        });
+        __syncwarp();
+        const uint32_t keep = s_keep[wi][lane];
+        if (keep != x) *am = keep;
+        __syncwarp();
     }
 }
 
-// Profile mode: add this level's live items and live groups to the totals.
-__global__ void bm_prof_kernel(QueryState st)
+// Many queries per group.  A unit is (G groups of a tile, a slice of the queries
+// that run); blocks take units from a counter.  A block loads the tables of the
+// G groups (every bucket's word of every projection, so any query's count is m
+// shared reads), then goes over its queries 8,192 at a time: the queries' live
+// bits become one bit row per group; warps take pieces of the rows from a
+// counter, and each set bit is an entry (group, query) of the warp's queue,
+// counted 32 at a time, one per lane.  Nearly all of a warp's lanes then read
+// the same group: for a projection, rows of one bucket list, consecutive 16-byte
+// words, so quarter-warps meet no bank twice unless two of their queries are
+// eight buckets apart.  Groups with candidates set a bit in a second set of
+// rows, and the live bits of the others are cleared at the end.
+//
+// Bound by logic operations (35 per 16 projections and 32 ids, at 64 lanes a
+// clock) and by shared memory (4 clocks per warp and projection).  41 million live
+// (query, group) pairs on 3 million points: 2.4 ms, 3.6 by one lane per pair
+// reading the bitmaps.  Two blocks per SM
+// cover each other's loads, queue ends and barriers; with one block of whole
+// rows dealt to the warps, three quarters of their time went into waiting for
+// the warp with the busiest group.
+constexpr int DN_THREADS = 256;
+constexpr int DN_WARPS = DN_THREADS / 32;
+constexpr int kDenseQ = 8192;   // queries of a segment
+constexpr int kDensePiece = 16; // 32-query words of a row a warp takes at a time
+
+struct DenseShared {
+    uint32_t live[kDenseGroups][kDenseQ / 32];  // [group][query / 32]
+    uint32_t some[kDenseGroups][kDenseQ / 32];  // ... with candidates
+    uint32_t queue[DN_WARPS][64];         // group of the unit << 16 | place in the segment
+    int nbk[QW_MAX_M];
+    int64_t base[QW_MAX_M];               // first bitmap of the level in the tile
+    int unit, next;
+};
+
+size_t dense_smem_bytes() { return kDenseTable + sizeof(DenseShared); }
+
+// Sixteen one-bit inputs per id of the four words: two carry-save halves, then
+// one carry into the planes of 16, 32 and 64.
+__device__ __forceinline__ void add16_half(Planes &P, const uint4 (&x)[8], uint32_t (&t8)[4])
 {
-    st.bm_prof[0] += (unsigned long long)min(*st.bm_nitems, st.bm_item_cap);
-    st.bm_prof[1] += (unsigned long long)min(*st.bm_nwork, st.bm_work_cap);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        uint32_t t2a, t2b, t4a, t4b;
+        csa(t2a, P.s[0][w], P.s[0][w], word_of(x[0], w), word_of(x[1], w));
+        csa(t2b, P.s[0][w], P.s[0][w], word_of(x[2], w), word_of(x[3], w));
+        csa(t4a, P.s[1][w], P.s[1][w], t2a, t2b);
+        csa(t2a, P.s[0][w], P.s[0][w], word_of(x[4], w), word_of(x[5], w));
+        csa(t2b, P.s[0][w], P.s[0][w], word_of(x[6], w), word_of(x[7], w));
+        csa(t4b, P.s[1][w], P.s[1][w], t2a, t2b);
+        csa(t8[w], P.s[2][w], P.s[2][w], t4a, t4b);
+    }
 }
 
-__global__ void __launch_bounds__(256, 3) bm_count_kernel(IndexView ix, int level, int l,
-                                                       QueryState st, const LoopCtl *ctl)
+// Count group g of tile t for query q, both the lane's own (every lane of the
+// warp; lanes that are not valid write nothing), from the group's table.  Sets
+// `bit` of *row when the group has a candidate.
+template <int S>
+__device__ __forceinline__ void dense_count(const IndexView &ix, const QueryState &st, int level,
+                                            int l, const unsigned char *tab, int q, bool valid,
+                                            int t, int g, uint32_t *row, int bit)
 {
-    if (ctl) level = ctl->level;
-    const int m = ix.m, nT = ix.nT;
-    const int nwork = min(*st.bm_nwork, st.bm_work_cap);
-    for (int wk = blockIdx.x * blockDim.x + threadIdx.x; wk < nwork;
-         wk += gridDim.x * blockDim.x) {
-        const int e = st.bm_work[wk];
-        const int slot = e >> 8, g = e & 0xff;
-        const int2 qt2 = st.bm_item_qt[slot];
-        const int q = qt2.x, t = qt2.y;
-        const int64_t qt = (int64_t)q * nT + t;
-        const int4 *bi4 = reinterpret_cast<const int4 *>(st.bm_item_bi + (int64_t)slot * ((m + 3) & ~3));
-        Planes P;
+    const int mp = st.bm_mp;
+    // 16 projections: two words of eight 4-bit rows
+    const uint2 *rows = reinterpret_cast<const uint2 *>(st.bm_rows + (int64_t)q * (mp >> 3));
+    Planes P;
 #pragma unroll
-        for (int kk = 0; kk < 7; ++kk)
+    for (int kk = 0; kk < 7; ++kk)
 #pragma unroll
-            for (int w = 0; w < 4; ++w) P.s[kk][w] = 0;
-        // words of projections whose summary misses the group are zero
-        const int mw = (m + 63) >> 6;
-        const unsigned long long mk0 = st.bm_wmask[(int64_t)wk * mw];
-        const unsigned long long mk1 = mw > 1 ? st.bm_wmask[(int64_t)wk * mw + 1] : 0ull;
-        for (int i0 = 0; i0 < m; i0 += 8) {
-            const uint32_t bits = (uint32_t)(((i0 < 64 ? mk0 : mk1) >> (i0 & 63)) & 0xffu);
-            if (bits == 0) continue;
-            // eight bitmap numbers in two vector loads (the row is padded to a
-            // multiple of four; entries past m are never selected by the mask)
-            const int4 ba = bits & 0x0fu ? bi4[i0 >> 2] : make_int4(-1, -1, -1, -1);
-            const int4 bb = bits & 0xf0u ? bi4[(i0 >> 2) + 1] : make_int4(-1, -1, -1, -1);
-            const int32_t bn[8] = {ba.x, ba.y, ba.z, ba.w, bb.x, bb.y, bb.z, bb.w};
-            uint4 x[8];
+        for (int w = 0; w < 4; ++w) P.s[kk][w] = 0;
+    auto sixteen = [&](uint2 r, const unsigned char *tb) {
+        uint32_t ta[4], tc[4];
+        uint4 x[8];
+        auto take = [&](uint32_t v, const unsigned char *at) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                x[u] = (bits >> u) & 1u ? __ldg(ix.bm + (int64_t)bn[u] * kBmUint4 + g)
-                                        : make_uint4(0, 0, 0, 0);
-            add8(P, x);
+            for (int u = 0; u < 8; ++u) {
+                const uint32_t o = u == 0 ? (v << 4) & 0xf0u : (v >> (4 * u - 4)) & 0xf0u;
+                x[u] = *reinterpret_cast<const uint4 *>(at + u * S * 16 + o);
+            }
+        };
+        take(r.x, tb);
+        add16_half(P, x, ta);
+        take(r.y, tb + 8 * S * 16);
+        add16_half(P, x, tc);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            uint32_t cy;
+            csa(cy, P.s[3][w], P.s[3][w], ta[w], tc[w]);
+            uint32_t nx = P.s[4][w] & cy;
+            P.s[4][w] ^= cy;
+            cy = nx;
+            nx = P.s[5][w] & cy;
+            P.s[5][w] ^= cy;
+            P.s[6][w] ^= nx;
         }
-        const uint4 cand = candidates_of(P, l);
-        const int nc = __popc(cand.x) + __popc(cand.y) + __popc(cand.z) + __popc(cand.w);
-        // A group without candidates (most live groups) writes no word: its
-        // live bit is cleared instead, and every reader of candidate words
-        // (the next level, the list rebuild) treats a cleared bit as an empty
-        // word.  Lanes clearing bits of the same mask word combine them.
-        {
-            const int64_t mw = ((int64_t)(level & 1) * st.cln_par + qt) * kSumWords + (g >> 5);
-            const uint32_t clear = nc == 0 ? (1u << (g & 31)) : 0u;
-            const unsigned act = __activemask();
-            const unsigned peers = __match_any_sync(act, (unsigned long long)mw);
-            const uint32_t all = __reduce_or_sync(peers, clear);
-            if (all != 0u && (threadIdx.x & 31) == __ffs(peers) - 1)
-                atomicAnd(st.bm_amask + mw, ~all);
+    };
+    uint2 next = __ldg(rows);
+    for (int i = 0; i < mp; i += 16) {
+        const uint2 r = next;
+        if (i + 16 < mp) next = __ldg(rows + (i >> 4) + 1);
+        sixteen(r, tab + i * S * 16);
+    }
+    const uint4 cand = candidates_of(P, l);
+    const int nc = __popc(cand.x) + __popc(cand.y) + __popc(cand.z) + __popc(cand.w);
+    if (!valid || nc == 0) return;
+    atomicOr(row, 1u << bit);
+    emit_group(st, ix.nT, level, q, t, g, cand, nc);
+}
+
+__global__ void __launch_bounds__(DN_THREADS, 2) bm_dense_kernel(IndexView ix, int level, int64_t R,
+                                                                 int l, QueryState st,
+                                                                 const LoopCtl *ctl)
+{
+    extern __shared__ __align__(16) unsigned char dsm[];
+    if (!dense_level(ix, st)) return;
+    unsigned char *table = dsm;
+    DenseShared &sh = *reinterpret_cast<DenseShared *>(dsm + kDenseTable);
+    if (ctl) {
+        level = ctl->level;
+        R = ctl->R;
+    }
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int m = ix.m, nT = ix.nT, mp = st.bm_mp;
+    const int nb = (int)st.bm_ctl[kCtlRun];  // queries that run
+    const int S = (int)st.bm_ctl[kCtlRows], G = (int)st.bm_ctl[kCtlGroups];
+    const int words = table_words(mp, S);
+    // queries in slices, so that there are several units per block
+    const int per_tile = kBmUint4 / G;
+    const int chunks = nT * per_tile;
+    const int slices = max(1, min((int)(gridDim.x * 4 + chunks - 1) / chunks, (nb + 1023) / 1024));
+    const int per_slice = ((nb + slices - 1) / slices + 31) & ~31;
+    uint32_t *amask = st.bm_amask + (int64_t)(level & 1) * st.cln_par * kSumWords;
+    for (int i = threadIdx.x; i < m; i += DN_THREADS) sh.nbk[i] = buckets_at(ix, i, level, R);
+    for (;;) {
+        __syncthreads();  // the table and the rows of the previous unit are done with
+        if (threadIdx.x == 0) sh.unit = (int)atomicAdd(st.bm_ctl + kCtlUnit, 1u);
+        __syncthreads();
+        const int unit = sh.unit;
+        if (unit >= chunks * slices) break;
+        // slices of one chunk one after the other: its bitmap words are in L2
+        const int chunk = unit / slices, slice = unit % slices;
+        const int t = chunk / per_tile, g0 = chunk % per_tile * G;
+        const int w = g0 >> 5, sh0 = g0 & 31;
+        for (int i = threadIdx.x; i < m; i += DN_THREADS)
+            sh.base[i] = ix.bm_base[i] + (int64_t)t * ix.bm_nb[i] +
+                         ix.bm_lvl[i * kBmLevels + min(level, ix.bm_J[i])];
+        __syncthreads();
+        // the tables: entries (projection, bucket, group), buckets past a
+        // projection's (and projections past m) zero
+#pragma unroll 4
+        for (int e = threadIdx.x; e < mp * S * G; e += DN_THREADS) {
+            const int g = e % G, b = e / G % S, i = e / (G * S);
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (i < m && b < sh.nbk[i]) v = __ldg(ix.bm + (sh.base[i] + b) * kBmUint4 + g0 + g);
+            *reinterpret_cast<uint4 *>(table + ((size_t)g * words + i * S + b) * 16) = v;
         }
-        if (nc == 0) continue;
-        st.cbits[(int64_t)(level & 1) * st.cb_par + qt * kBmUint4 + g] = cand;
-        // the previous level's candidate word, needed only to flag the new
-        // candidates: written there only if the tile had candidates and the
-        // group was live
-        const bool first = level == st.start[q];
-        const int64_t pq = (int64_t)((level - 1) & 1) * st.cln_par + qt;
-        const bool has_prev = !first && st.clist_n[pq] > 0 &&
-                              ((st.bm_amask[pq * kSumWords + (g >> 5)] >> (g & 31)) & 1u);
-        const uint4 prev = has_prev ? st.cbits[(int64_t)((level - 1) & 1) * st.cb_par + qt * kBmUint4 + g]
-                                    : make_uint4(0, 0, 0, 0);
-        atomicAdd(st.clist_n + (int64_t)(level & 1) * st.cln_par + qt, nc);
-        atomicAdd(st.cross + q, nc);
-        const int pos = atomicAdd(st.qbuf_n + (int64_t)(level & 1) * st.qbn_par + q, nc);
-        append_candidates(P, cand, prev, st.qbuf + (int64_t)(level & 1) * st.qb_par + (int64_t)q * kQCap,
-                          pos, (int64_t)t * kTile + (int64_t)g * 128);
+        const int q_end = min(nb, (slice + 1) * per_slice);
+        for (int s0 = slice * per_slice; s0 < q_end; s0 += kDenseQ) {
+            const int s1 = min(q_end, s0 + kDenseQ);
+            const int nblk = (s1 - s0 + 31) >> 5;
+            // live words (lane = query) -> rows (lane = group)
+#pragma unroll 4
+            for (int b = wi; b < nblk; b += DN_WARPS) {
+                const int at = s0 + b * 32 + lane;
+                const uint32_t x =
+                    at < s1 ? amask[((int64_t)st.bm_run[at] * nT + t) * kSumWords + w] >> sh0 : 0u;
+                uint32_t row = 0;
+#pragma unroll
+                for (int g = 0; g < kDenseGroups; ++g) {
+                    const uint32_t y = __ballot_sync(0xffffffffu, (x >> g) & 1u);
+                    row = lane == g ? y : row;
+                }
+                if (lane < G) {
+                    sh.live[lane][b] = row;
+                    sh.some[lane][b] = 0;
+                }
+            }
+            if (threadIdx.x == 0) sh.next = 0;
+            __syncthreads();
+            const int pieces = (nblk + kDensePiece - 1) / kDensePiece;
+            int held = 0;
+            auto count32 = [&](uint32_t e, bool valid) {
+                const int gl = (int)(e >> 16), ql = (int)(e & 0xffffu);
+                const int q = st.bm_run[s0 + ql];
+                const unsigned char *tab = table + (size_t)gl * words * 16;
+                uint32_t *row = &sh.some[gl][ql >> 5];
+                if (S == 4) dense_count<4>(ix, st, level, l, tab, q, valid, t, g0 + gl, row, ql & 31);
+                else if (S == 8) dense_count<8>(ix, st, level, l, tab, q, valid, t, g0 + gl, row, ql & 31);
+                else dense_count<16>(ix, st, level, l, tab, q, valid, t, g0 + gl, row, ql & 31);
+            };
+            for (;;) {
+                int u = 0;
+                if (lane == 0) u = atomicAdd(&sh.next, 1);
+                u = __shfl_sync(0xffffffffu, u, 0);
+                if (u >= G * pieces) break;
+                const int gl = u / pieces, piece = u % pieces;
+                const int b0 = piece * kDensePiece, b1 = min(nblk, b0 + kDensePiece);
+                // the piece's words in the lanes
+                const uint32_t xs = b0 + lane < b1 && lane < kDensePiece ? sh.live[gl][b0 + lane] : 0u;
+                uint32_t full = __ballot_sync(0xffffffffu, xs != 0);
+                while (full) {
+                    const int o = __ffs(full) - 1;
+                    full &= full - 1;
+                    const uint32_t x = __shfl_sync(0xffffffffu, xs, o);
+                    if ((x >> lane) & 1u)
+                        sh.queue[wi][held + __popc(x & ((1u << lane) - 1u))] =
+                            (uint32_t)gl << 16 | (uint32_t)((b0 + o) * 32 + lane);
+                    held += __popc(x);
+                    __syncwarp();
+                    if (held >= 32) {
+                        const uint32_t e = sh.queue[wi][lane];
+                        const uint32_t rest = sh.queue[wi][32 + lane];
+                        __syncwarp();
+                        sh.queue[wi][lane] = rest;
+                        held -= 32;
+                        __syncwarp();
+                        count32(e, true);
+                    }
+                }
+            }
+            if (held > 0) count32(sh.queue[wi][min(lane, held - 1)], lane < held);
+            __syncthreads();
+            // clear the live bits of groups without candidates
+#pragma unroll 2
+            for (int b = wi; b < nblk; b += DN_WARPS) {
+                const int at = s0 + b * 32 + lane;
+                const uint32_t none =
+                    lane < G ? sh.live[lane][b] & ~sh.some[lane][b] : 0u;
+                uint32_t gone = 0;
+#pragma unroll
+                for (int g = 0; g < kDenseGroups; ++g)
+                    gone |= ((__shfl_sync(0xffffffffu, none, g) >> lane) & 1u) << g;
+                if (at < s1 && gone)
+                    atomicAnd(&amask[((int64_t)st.bm_run[at] * nT + t) * kSumWords + w],
+                              ~(gone << sh0));
+            }
+            __syncthreads();
+        }
     }
 }
 
@@ -589,23 +940,22 @@ __global__ void __launch_bounds__(256, 3) bm_count_kernel(IndexView ix, int leve
 // of the tile): the m bitmap numbers of the tile stay in the lanes' registers
 // (lane j holds projections j and j + 32) and are broadcast by shuffles, so a
 // group's m word loads depend on nothing but its own projection mask, which
-// the filter step left in shared memory.  No work list, item slots or masks go
-// through global memory.  Results (candidate words, live-group masks, tile
-// counts, candidate lists, profile counters) are those of the two passes.
-// Position of the n-th (0-based) set bit of v; n < popc(v).
-__device__ __forceinline__ int nth_set_bit(uint32_t v, int n)
+// the filter step left in shared memory.  Results (candidate words and counts, profile counters)
+// are those of the two passes; every live group's bit stays set and its word is
+// written.
+constexpr int FL_TILES = 8;  // tiles per warp unless the caller picks 4 or 16
+
+template <int NROW>
+__device__ __forceinline__ void load_summaries(const IndexView &ix, const int32_t (&srow)[NROW],
+                                               int t, uint4 (&sv)[NROW][2])
 {
-    int pos = 0;
 #pragma unroll
-    for (int w = 16; w > 0; w >>= 1) {
-        const int c = __popc(v & ((1u << w) - 1u));
-        if (n >= c) {
-            n -= c;
-            v >>= w;
-            pos += w;
-        }
+    for (int r = 0; r < NROW; ++r) {
+        const uint4 *p =
+            reinterpret_cast<const uint4 *>(ix.bm_sum + ((int64_t)srow[r] + t) * kSumWords);
+        sv[r][0] = __ldg(p);
+        sv[r][1] = __ldg(p + 1);
     }
-    return pos;
 }
 
 template <int NROW, int TPW>
@@ -631,17 +981,17 @@ __global__ void __launch_bounds__(FL_WARPS * 32, 2) bm_fused_kernel(IndexView ix
         const int q = (int)(k % nb);
         const int t0 = (int)(k / nb) * TPW, t1 = min(nT, t0 + TPW);
         if (!st.active[q] || level < st.start[q]) continue;
-        const bool first = level == st.start[q];
         int64_t b0[NROW];
-        int32_t nbp[NROW];
+        int32_t nbp[NROW], srow[NROW];
 #pragma unroll
         for (int r = 0; r < NROW; ++r) {
             const int i = lane + 32 * r;
-            b0[r] = i < m ? st.bm_bq[(int64_t)q * m + i] : -1;
+            b0[r] = i < m ? st.bm_b0[(int64_t)q * st.bm_mp + i] : -1;
+            srow[r] = i < m ? st.bm_srow[(int64_t)q * st.bm_mp + i] : (int32_t)ix.bm_total;
             nbp[r] = i < m ? ix.bm_nb[i] : 0;
         }
         uint4 sv[NROW][2];
-        load_summaries<NROW>(ix, b0, nbp, t0, sv);
+        load_summaries<NROW>(ix, srow, t0, sv);
         for (int t = t0; t < t1; ++t) {
             const int64_t qt = (int64_t)q * nT + t;
             int n_alive = 0;
@@ -665,20 +1015,14 @@ __global__ void __launch_bounds__(FL_WARPS * 32, 2) bm_fused_kernel(IndexView ix
             }
             __syncwarp();
             // the next tile's summaries load while this tile is counted
-            if (t + 1 < t1) load_summaries<NROW>(ix, b0, nbp, t + 1, sv);
-            if (n_alive == 0) {
-                if (lane == 0) st.clist_n[(int64_t)par * st.cln_par + qt] = 0;
-                continue;
-            }
+            if (t + 1 < t1) load_summaries<NROW>(ix, srow, t + 1, sv);
             if (lane < kSumWords)
                 st.bm_amask[((int64_t)par * st.cln_par + qt) * kSumWords + lane] = wlive[wi][lane];
+            if (n_alive == 0) continue;
             // this tile's bitmap numbers, one per lane and row
             int64_t bt[NROW];
 #pragma unroll
             for (int r = 0; r < NROW; ++r) bt[r] = b0[r] >= 0 ? b0[r] + (int64_t)t * nbp[r] : -1;
-            const int64_t pq = (int64_t)((level - 1) & 1) * st.cln_par + qt;
-            const bool tile_prev = !first && st.clist_n[pq] > 0;
-            int tile_n = 0;
             for (int base = 0; base < n_alive; base += 32) {
                 // the (base + lane)-th live group of the tile
                 const int kk = base + lane;
@@ -697,12 +1041,6 @@ __global__ void __launch_bounds__(FL_WARPS * 32, 2) bm_fused_kernel(IndexView ix
 #pragma unroll
                 for (int h = 0; h < MW; ++h)
                     mk[h] = g >= 0 ? wmk[wi][g >> 5][h][g & 31] : 0ull;
-                const bool has_prev =
-                    g >= 0 && tile_prev &&
-                    ((st.bm_amask[pq * kSumWords + (g >> 5)] >> (g & 31)) & 1u);
-                const uint4 prev = has_prev ? st.cbits[(int64_t)((level - 1) & 1) * st.cb_par +
-                                                       qt * kBmUint4 + g]
-                                            : make_uint4(0, 0, 0, 0);
                 Planes P;
 #pragma unroll
                 for (int kq = 0; kq < 7; ++kq)
@@ -734,27 +1072,8 @@ __global__ void __launch_bounds__(FL_WARPS * 32, 2) bm_fused_kernel(IndexView ix
                     nc = __popc(cand.x) + __popc(cand.y) + __popc(cand.z) + __popc(cand.w);
                     p_words += (unsigned long long)words;
                 }
-                // list positions: one reservation per warp
-                int incl = nc;
-#pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int y = __shfl_up_sync(0xffffffffu, incl, off);
-                    if (lane >= off) incl += y;
-                }
-                const int tot = __shfl_sync(0xffffffffu, incl, 31);
-                int pos0 = 0;
-                if (lane == 0 && tot)
-                    pos0 = atomicAdd(st.qbuf_n + (int64_t)par * st.qbn_par + q, tot);
-                pos0 = __shfl_sync(0xffffffffu, pos0, 0);
-                if (nc)
-                    append_candidates(P, cand, prev,
-                                      st.qbuf + (int64_t)par * st.qb_par + (int64_t)q * kQCap,
-                                      pos0 + incl - nc, (int64_t)t * kTile + (int64_t)g * 128);
-                tile_n += tot;
-            }
-            if (lane == 0) {
-                st.clist_n[(int64_t)par * st.cln_par + qt] = tile_n;
-                if (tile_n) atomicAdd(st.cross + q, tile_n);
+                const int tot = __reduce_add_sync(0xffffffffu, nc);
+                if (lane == 0 && tot) atomicAdd(st.qbuf_n + (int64_t)par * st.qbn_par + q, tot);
             }
             p_items += 1;
             p_groups += (unsigned long long)n_alive;
@@ -782,70 +1101,32 @@ __global__ void __launch_bounds__(FL_WARPS * 32, 2) bm_fused_kernel(IndexView ix
 // bitmaps are present, first / last stage of the item, end of work).  Eight
 // consumer warps follow the stage stream: each adds a stage into its bit
 // planes straight from shared memory and, at an item's last stage, writes the
-// item's candidate bitmap, list and profile.  Consumers never wait on a
-// global load for control flow.
+// item's candidate words, their group bits (a warp holds one word of them) and
+// count.  Consumers never wait on a global load for control flow.
 constexpr int kRing = 6;
 constexpr int kPerStage = 8;                       // bitmaps per stage
 constexpr int kStageBytesBm = kPerStage * kTile / 8;  // 32 KiB
 constexpr int TMA_CONSUMERS = BM_THREADS;          // 8 warps, one 16-byte word each
 constexpr int TMA_THREADS = TMA_CONSUMERS + 32;    // + the producer warp
-constexpr uint32_t kFirstStage = 1, kLastStage = 2, kFirstLevel = 4, kDone = 8;
+constexpr uint32_t kFirstStage = 1, kLastStage = 2, kDone = 4;
 
 struct StageHdr {
     int32_t q, t;
     uint32_t mask;   // which of the stage's bitmaps are present
-    uint32_t flags;  // kFirstStage | kLastStage | kFirstLevel | kDone
+    uint32_t flags;  // kFirstStage | kLastStage | kDone
 };
 
 struct TmaShared {
     uint64_t full[kRing];
     uint64_t empty[kRing];
-    uint64_t group;                // consumer-only barrier (one arrival per warp)
     StageHdr hdr[kRing];
     int64_t pt[QW_MAX_M + 8];      // bitmap numbers of the current item (-1: empty)
     int64_t lbase[QW_MAX_M];       // per projection: bm_base + bm_lvl[min(level, J)]
     int32_t nbk[QW_MAX_M];         // per projection: buckets at this level (0: past J)
     int32_t pnb[QW_MAX_M];         // per projection: bitmaps per tile
-    int base[2];                   // list position of the current item (alternating)
-    int wsum[TMA_CONSUMERS / 32];
 };
 
 size_t tma_smem_bytes() { return sizeof(TmaShared) + 128 + (size_t)kRing * kStageBytesBm; }
-
-// The consumer warps meet on an mbarrier (bounded wait) rather than a named
-// barrier, so a warp that gave up on a wait cannot leave the others waiting.
-__device__ __forceinline__ void group_sync(uint64_t *bar, uint32_t &ph, int *err, bool &stuck)
-{
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-    mbar_wait(bar, ph & 1, err, stuck);
-    ++ph;
-}
-
-// Exclusive prefix sum over the consumer threads (see block_exclusive_scan).
-__device__ __forceinline__ int consumer_scan(int v, int *tmp, int *total, uint64_t *bar,
-                                             uint32_t &ph, int *err, bool &stuck)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += y;
-    }
-    group_sync(bar, ph, err, stuck);  // tmp of the previous scan has been read
-    if (lane == 31) tmp[warp] = incl;
-    group_sync(bar, ph, err, stuck);
-    int wbase = 0, tot = 0;
-#pragma unroll
-    for (int w = 0; w < TMA_CONSUMERS / 32; ++w) {
-        int s = tmp[w];
-        if (w < warp) wbase += s;
-        tot += s;
-    }
-    *total = tot;
-    return wbase + incl - v;
-}
 
 __global__ void __launch_bounds__(TMA_THREADS, 1) bm_level_tma_kernel(IndexView ix, int level,
                                                                       int64_t R, int l, int nb,
@@ -869,7 +1150,6 @@ __global__ void __launch_bounds__(TMA_THREADS, 1) bm_level_tma_kernel(IndexView 
             mbar_init(&sh.full[k], 1);
             mbar_init(&sh.empty[k], TMA_CONSUMERS / 32);
         }
-        mbar_init(&sh.group, TMA_CONSUMERS / 32);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int i = tid; i < m; i += TMA_THREADS) {
@@ -907,7 +1187,6 @@ __global__ void __launch_bounds__(TMA_THREADS, 1) bm_level_tma_kernel(IndexView 
 #pragma unroll
             for (int u = 0; u < kPL; ++u) g[u] = gn[u];
             const bool runs = act_n && level >= start_n;
-            const bool first = level == start_n;
             prefetch(k + gridDim.x);  // in flight while this item is issued
             if (!runs) continue;
 #pragma unroll
@@ -939,8 +1218,7 @@ __global__ void __launch_bounds__(TMA_THREADS, 1) bm_level_tma_kernel(IndexView 
                     h.q = q;
                     h.t = t;
                     h.mask = mask;
-                    h.flags = (j == 0 ? kFirstStage : 0u) | (j == nst - 1 ? kLastStage : 0u) |
-                              (first ? kFirstLevel : 0u);
+                    h.flags = (j == 0 ? kFirstStage : 0u) | (j == nst - 1 ? kLastStage : 0u);
                     mbar_arrive_expect_tx(&sh.full[slot], (uint32_t)__popc(mask) * (kTile / 8));
 #pragma unroll
                     for (int u = 0; u < kPerStage; ++u)
@@ -978,10 +1256,8 @@ __global__ void __launch_bounds__(TMA_THREADS, 1) bm_level_tma_kernel(IndexView 
         return;
     }
     // ---- consumers: thread tid owns 16-byte word tid (128 ids) of every bitmap
-    uint32_t it = 0, gph = 0;
-    int par = 0;
+    uint32_t it = 0;
     Planes P;
-    uint4 prev = make_uint4(0, 0, 0, 0);
     for (;; ++it) {
         const int slot = (int)(it % kRing);
         mbar_wait(&sh.full[slot], (it / kRing) & 1, err, stuck);
@@ -994,9 +1270,6 @@ __global__ void __launch_bounds__(TMA_THREADS, 1) bm_level_tma_kernel(IndexView 
             for (int kk = 0; kk < 7; ++kk)
 #pragma unroll
                 for (int w = 0; w < 4; ++w) P.s[kk][w] = 0;
-            prev = (h.flags & kFirstLevel)
-                       ? make_uint4(0, 0, 0, 0)
-                       : st.cbits[(int64_t)((level - 1) & 1) * st.cb_par + qt * kBmUint4 + tid];
         }
         const uint4 *stage = reinterpret_cast<const uint4 *>(ring + (size_t)slot * kStageBytesBm);
         uint4 x[kPerStage];
@@ -1009,26 +1282,118 @@ __global__ void __launch_bounds__(TMA_THREADS, 1) bm_level_tma_kernel(IndexView 
         if (!(h.flags & kLastStage)) continue;
         // ---- the item's epilogue (consumers only: the producer does not take part)
         const uint4 cand = candidates_of(P, l);
-        st.cbits[(int64_t)(level & 1) * st.cb_par + qt * kBmUint4 + tid] = cand;
-        const int my_count = __popc(cand.x) + __popc(cand.y) + __popc(cand.z) + __popc(cand.w);
-        int tot_count;
-        const int pos = consumer_scan(my_count, sh.wsum, &tot_count, &sh.group, gph, err, stuck);
-        if (tid == 0) {
-            st.clist_n[(int64_t)(level & 1) * st.cln_par + qt] = tot_count;
-            sh.base[par] = tot_count ? atomicAdd(st.qbuf_n + (int64_t)(level & 1) * st.qbn_par + h.q,
-                                                 tot_count)
-                                     : 0;
-            if (tot_count) atomicAdd(st.cross + h.q, tot_count);
+        const int nc = __popc(cand.x) + __popc(cand.y) + __popc(cand.z) + __popc(cand.w);
+        if (nc) st.cbits[(int64_t)(level & 1) * st.cb_par + qt * kBmUint4 + tid] = cand;
+        const uint32_t some = __ballot_sync(0xffffffffu, nc != 0);
+        const int tot = __reduce_add_sync(0xffffffffu, nc);
+        if (lane == 0) {
+            st.bm_amask[((int64_t)(level & 1) * st.cln_par + qt) * kSumWords + warp] = some;
+            if (tot) atomicAdd(st.qbuf_n + (int64_t)(level & 1) * st.qbn_par + h.q, tot);
         }
-        group_sync(&sh.group, gph, err, stuck);
-        if (stuck) break;
-        append_candidates(P, cand, prev,
-                          st.qbuf + (int64_t)(level & 1) * st.qb_par + (int64_t)h.q * kQCap,
-                          sh.base[par] + pos, (int64_t)h.t * kTile + tid * 128);
-        par ^= 1;
     }
 }
 
+// ---- the candidates of the queries' last levels
+//
+// bm_final_bucket_kernel: the bitmap numbers of every query's buckets at its
+// last level (the two-pass and fused levels leave them in bm_b0).
+__global__ void bm_final_bucket_kernel(IndexView ix, int nb, QueryState st)
+{
+    const int m = ix.m, mp = st.bm_mp;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)nb * mp;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int q = (int)(e / mp), i = (int)(e % mp);
+        const int L = st.levels[q] - 1;
+        const int64_t R = st.finalR[q];
+        st.bm_b0[e] = L >= 0 && i < m ? (int32_t)bm_index(ix, i, 0, L, R,
+                                                          floordiv64(st.g[(int64_t)q * m + i], R))
+                                      : -1;
+    }
+}
+
+// Append this thread's candidates (128 ids, ascending) to the query's list
+// from position pos: (internal id << 32) | (prev << 8) | count.
+__device__ __forceinline__ void append_candidates(const Planes &P, const uint4 &cand,
+                                                  const uint4 &prev, uint64_t *list, int pos,
+                                                  int64_t id_base)
+{
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        uint32_t x = word_of(cand, w);
+        const uint32_t pw = word_of(prev, w);
+        while (x) {
+            const int b = __ffs(x) - 1;
+            x &= x - 1;
+            if (pos < kQCap)
+                list[pos] = ((uint64_t)(id_base + w * 32 + b) << 32) |
+                            ((uint64_t)((pw >> b) & 1u) << 8) | (uint64_t)count_of(P, w, b);
+            ++pos;
+        }
+    }
+}
+
+// The candidate word of group g of a (query, tile) at level L (zero where the
+// level wrote none).
+__device__ __forceinline__ uint4 rd_word(const QueryState &st, int L, int64_t qt, int g)
+{
+    const int64_t pc = (int64_t)(L & 1) * st.cln_par + qt;
+    if (!((st.bm_amask[pc * kSumWords + (g >> 5)] >> (g & 31)) & 1u)) return make_uint4(0, 0, 0, 0);
+    return st.cbits[(int64_t)(L & 1) * st.cb_par + qt * kBmUint4 + g];
+}
+
+// Lists the last level's candidates of every query that has at most kQCap of
+// them: the counts of its groups with candidates once more from the bitmaps
+// (few of the groups counted on the way there), and whether each was a candidate
+// of the previous level (its word there, if the query ran it).  A warp takes
+// four tiles of a query, as bm_count_kernel does.  Listing during the levels
+// instead, every candidate of every level behind a returning atomic, took most
+// of the count pass where candidates are many (606 queries whose last level
+// takes in all 300,000 points: 2.3 ms of a level of 0.17).
+__global__ void __launch_bounds__(256, 3) bm_list_kernel(IndexView ix, int l, int nb, QueryState st)
+{
+    __shared__ int s_nb[QW_MAX_M + 16];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int m = ix.m, nT = ix.nT, mp = st.bm_mp;
+    for (int i = threadIdx.x; i < mp; i += 256) s_nb[i] = i < m ? ix.bm_nb[i] : 0;
+    __syncthreads();
+    const int64_t tasks = (int64_t)nb * ((nT + 3) >> 2);
+    for (int64_t k = (int64_t)blockIdx.x * 8 + wi; k < tasks; k += (int64_t)gridDim.x * 8) {
+        const int q = (int)(k % nb), t0 = (int)(k / nb) * 4;
+        const int L = st.levels[q] - 1;
+        if (L < 0) continue;
+        const int n = st.qbuf_n[(int64_t)(L & 1) * st.qbn_par + q];
+        if (n == 0 || n > kQCap) continue;
+        const bool ran_prev = L > st.start[q];
+        const uint32_t x =
+            t0 + (lane >> 3) < nT
+                ? st.bm_amask[((int64_t)(L & 1) * st.cln_par + (int64_t)q * nT + t0) * kSumWords + lane]
+                : 0u;
+        if (!__any_sync(0xffffffffu, x != 0)) continue;
+        uint64_t *list = st.qbuf + (int64_t)q * kQCap;
+        each_set_bit(x, lane, [&](int own, int bit, bool valid, bool four) {
+            const int t = t0 + (own >> 3), g = (own & 7) * 32 + bit;
+            const int64_t qt = (int64_t)q * nT + t;
+            const uint4 prev = ran_prev ? rd_word(st, L - 1, qt, g) : make_uint4(0, 0, 0, 0);
+            Planes P;
+            count_planes(ix, st.bm_b0 + (int64_t)q * mp, s_nb, t, g, P, four);
+            const uint4 cand = candidates_of(P, l);
+            int nc = __popc(cand.x) + __popc(cand.y) + __popc(cand.z) + __popc(cand.w);
+            if (!valid) nc = 0;
+            int incl = nc;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
+            }
+            int pos = 0;
+            if (lane == 31 && incl) pos = atomicAdd(st.cross + q, incl);
+            pos = __shfl_sync(0xffffffffu, pos, 31);
+            if (nc)
+                append_candidates(P, cand, prev, list, pos + incl - nc,
+                                  (int64_t)t * kTile + (int64_t)g * 128);
+        });
+    }
+}
 // Sort keys[0..n) ascending in shared memory (n padded to P2 with ~0).
 __device__ __forceinline__ void smem_bitonic(uint64_t *keys, int n, int P2)
 {
@@ -1082,7 +1447,7 @@ __global__ void __launch_bounds__(SEL_THREADS) bm_select_kernel(IndexView ix, in
     const int jf = st.levels[q] - 1;
     const int n = st.qbuf_n[(int64_t)(jf & 1) * st.qbn_par + q];
     const int nc = st.ncand[q];
-    const uint64_t *E = st.qbuf + (int64_t)(jf & 1) * st.qb_par + (int64_t)q * kQCap;
+    const uint64_t *E = st.qbuf + (int64_t)q * kQCap;
     int32_t *cand = st.cand + (int64_t)q * cap;
     int32_t *col = st.cand_col + (int64_t)q * cap;
     int32_t *eq = st.eqbuf + (int64_t)q * kEqCap;
@@ -1261,12 +1626,11 @@ __global__ void __launch_bounds__(SEL_THREADS) bm_select_kernel(IndexView ix, in
 
 // ---- a last level that overflows the candidate list
 //
-// The count kernels list every candidate of a level, up to kQCap per query.
-// When one doubling of the radius sweeps whole clusters into a query's last
-// level, that level can hold more.  Of them the k + v bound keeps only the
-// previous level's candidates, every candidate whose count is above the
-// boundary count c*, and the smallest original ids of the tie class at c*
-// (Section 3.1, readings R4/R5).  The kernels below rebuild the list of such
+// A query's list holds up to kQCap candidates.  When one doubling of the radius
+// sweeps whole clusters into a query's last level, that level can hold more.  Of
+// them the k + v bound keeps only the previous level's candidates, every
+// candidate whose count is above the boundary count c*, and the smallest
+// original ids of the tie class at c* (Section 3.1, readings R4/R5).  The kernels below rebuild the list of such
 // a query with only those entries, from the candidate words of its last level
 // (still in place: a stopped query's tiles are not touched by later levels)
 // and the level bitmaps, each read once:
@@ -1294,16 +1658,6 @@ constexpr int kRdTieList = 4096;   // larger tie classes are cut by the original
 constexpr int kRdStoreWords = 8;  // uint4 per group: 7 count planes, previous-level word
 constexpr int RD_THREADS = 256;
 static_assert(RD_THREADS == kBmUint4, "one block covers the groups of one tile");
-
-// The candidate word of group g at level L (zero where the level wrote none).
-__device__ __forceinline__ uint4 rd_word(const QueryState &st, int L, int64_t qt, int g, bool tma)
-{
-    const int64_t pc = (int64_t)(L & 1) * st.cln_par + qt;
-    if (st.clist_n[pc] == 0) return make_uint4(0, 0, 0, 0);
-    if (!tma && !((st.bm_amask[pc * kSumWords + (g >> 5)] >> (g & 31)) & 1u))
-        return make_uint4(0, 0, 0, 0);
-    return st.cbits[(int64_t)(L & 1) * st.cb_par + qt * kBmUint4 + g];
-}
 
 // Count planes of group g of tile t from the bitmaps of one level: bq[i] is
 // the bucket's bitmap in tile 0 (-1: no data), tile t adds t * bm_nb[i].
@@ -1363,11 +1717,14 @@ __global__ void rd_compact_kernel(IndexView ix, int cgrow, QueryState st, int nb
 }
 
 // One block per (slot, tile) at a time, one thread per group.
-__global__ void __launch_bounds__(RD_THREADS, 2) rd_count_kernel(IndexView ix, int l,
-                                                                  QueryState st, bool tma, int s0,
+__global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, int l,
+                                                                  QueryState st, int s0,
                                                                   int wave)
 {
     __shared__ int sh_hist[kHistBins];
+    __shared__ int s_nb[QW_MAX_M + 16];
+    for (int i = threadIdx.x; i < st.bm_mp; i += RD_THREADS) s_nb[i] = i < ix.m ? ix.bm_nb[i] : 0;
+    __syncthreads();
     const int nslot = min(st.rd_ctl[0] - s0, wave);
     const int nT = ix.nT, g = threadIdx.x;
     for (int64_t it = blockIdx.x; it < (int64_t)max(nslot, 0) * nT; it += gridDim.x) {
@@ -1375,22 +1732,27 @@ __global__ void __launch_bounds__(RD_THREADS, 2) rd_count_kernel(IndexView ix, i
         const RdPlan pl = st.rd_plan[slot];
         const int q = pl.q, L = st.levels[q] - 1;
         const int64_t qt = (int64_t)q * nT + t;
-        if (st.clist_n[(int64_t)(L & 1) * st.cln_par + qt] == 0) continue;  // block-uniform
+        // tiles without candidates (block-uniform)
+        if (!__syncthreads_or(st.bm_amask[((int64_t)(L & 1) * st.cln_par + qt) * kSumWords +
+                                          (threadIdx.x & 7)] != 0))
+            continue;
         for (int c = threadIdx.x; c < kHistBins; c += RD_THREADS) sh_hist[c] = 0;
         __syncthreads();
-        const uint4 cw = rd_word(st, L, qt, g, tma);
+        const uint4 cw = rd_word(st, L, qt, g);
         int my_np = 0;
+        Planes P;
+        uint32_t oth[4] = {0, 0, 0, 0};  // candidates not of the previous level
+        int n_oth = 0;
         if (cw.x | cw.y | cw.z | cw.w) {
             const int64_t *bq = st.rd_bq + (int64_t)slot * 2 * QW_MAX_M;
-            Planes P;
             uint4 pw = make_uint4(0, 0, 0, 0);
             if (pl.prev_recount) {
                 rd_planes(ix, bq + QW_MAX_M, t, g, P);
                 pw = candidates_of(P, l);
             } else if (L > 0) {
-                pw = rd_word(st, L - 1, qt, g, tma);
+                pw = rd_word(st, L - 1, qt, g);
             }
-            rd_planes(ix, bq, t, g, P);
+            count_planes(ix, st.bm_b0 + (int64_t)q * st.bm_mp, s_nb, t, g, P);
             uint4 *store = st.rd_store +
                            ((int64_t)(slot - s0) * nT * kBmUint4 + (int64_t)t * kBmUint4 + g) *
                                kRdStoreWords;
@@ -1400,7 +1762,26 @@ __global__ void __launch_bounds__(RD_THREADS, 2) rd_count_kernel(IndexView ix, i
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
                 my_np += __popc(word_of(cw, w) & word_of(pw, w));
-                uint32_t x = word_of(cw, w) & ~word_of(pw, w);
+                oth[w] = word_of(cw, w) & ~word_of(pw, w);
+                n_oth += __popc(oth[w]);
+            }
+        }
+        // the histogram of their counts: a warp with many of them compares the
+        // planes with every count (one addition per warp and count); adding one
+        // by one meets the same few shared words over and over
+        if (__reduce_add_sync(0xffffffffu, n_oth) > 256) {
+            for (int c = l; c <= ix.m; ++c) {
+                int here = 0;
+#pragma unroll
+                for (int w = 0; w < 4; ++w)
+                    if (oth[w]) here += __popc(count_eq_planes(P, w, c) & oth[w]);
+                here = __reduce_add_sync(0xffffffffu, here);
+                if ((threadIdx.x & 31) == 0 && here) atomicAdd(&sh_hist[c], here);
+            }
+        } else {
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                uint32_t x = oth[w];
                 while (x) {
                     const int b = __ffs(x) - 1;
                     x &= x - 1;
@@ -1488,7 +1869,7 @@ __device__ __forceinline__ void rd_stored(const QueryState &st, int slot, int nT
 // The kept entries of every rebuilt slot, one thread per group: previous-level
 // candidates, counts above c*, and (a short tie class) the tie class.
 __global__ void __launch_bounds__(RD_THREADS, 3) rd_emit_kernel(IndexView ix, QueryState st,
-                                                                 bool tma, int wave)
+                                                                 int wave)
 {
     const int nslot = min(st.rd_ctl[0], wave);
     const int m = ix.m, nT = ix.nT, g = threadIdx.x;
@@ -1498,7 +1879,7 @@ __global__ void __launch_bounds__(RD_THREADS, 3) rd_emit_kernel(IndexView ix, Qu
         if (pl.mode == 0) continue;
         const int q = pl.q, L = st.levels[q] - 1;
         const int64_t qt = (int64_t)q * nT + t;
-        const uint4 cw = rd_word(st, L, qt, g, tma);
+        const uint4 cw = rd_word(st, L, qt, g);
         if (!(cw.x | cw.y | cw.z | cw.w)) continue;
         Planes P;
         uint4 pw;
@@ -1518,7 +1899,7 @@ __global__ void __launch_bounds__(RD_THREADS, 3) rd_emit_kernel(IndexView ix, Qu
             my_n += __popc(kw);
         }
         if (my_n) {
-            uint64_t *E = st.qbuf + (int64_t)(L & 1) * st.qb_par + (int64_t)q * kQCap;
+            uint64_t *E = st.qbuf + (int64_t)q * kQCap;
             int pos = atomicAdd(&st.rd_plan[slot].pos, my_n);
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
@@ -1548,7 +1929,7 @@ __global__ void __launch_bounds__(RD_THREADS, 3) rd_emit_kernel(IndexView ix, Qu
 constexpr int kScanPer = 4;
 
 __global__ void __launch_bounds__(RD_THREADS) rd_scan_kernel(IndexView ix, QueryState st,
-                                                              bool tma, int wave)
+                                                              int wave)
 {
     constexpr int NW = RD_THREADS / 32;
     __shared__ int s_wc[kScanPer][NW];
@@ -1560,7 +1941,7 @@ __global__ void __launch_bounds__(RD_THREADS) rd_scan_kernel(IndexView ix, Query
         const RdPlan pl = st.rd_plan[slot];
         if (pl.mode != 2 || pl.take <= 0) continue;
         const int q = pl.q, L = st.levels[q] - 1;
-        uint64_t *E = st.qbuf + (int64_t)(L & 1) * st.qb_par + (int64_t)q * kQCap;
+        uint64_t *E = st.qbuf + (int64_t)q * kQCap;
         if (threadIdx.x == 0) s_base = atomicAdd(&st.rd_plan[slot].pos, pl.take);
         __syncthreads();
         const int base = s_base;
@@ -1577,7 +1958,7 @@ __global__ void __launch_bounds__(RD_THREADS) rd_scan_kernel(IndexView ix, Query
             for (int u = 0; u < kScanPer; ++u) {
                 const int64_t id = iid[u] >= 0 ? iid[u] : 0;
                 const int t = (int)(id / kTile), g = (int)((id % kTile) >> 7);
-                cw[u] = iid[u] >= 0 ? rd_word(st, L, (int64_t)q * ix.nT + t, g, tma)
+                cw[u] = iid[u] >= 0 ? rd_word(st, L, (int64_t)q * ix.nT + t, g)
                                     : make_uint4(0, 0, 0, 0);
             }
             bool tie[kScanPer];
@@ -1678,7 +2059,7 @@ __global__ void __launch_bounds__(RC_THREADS) bm_recount_kernel(IndexView ix, in
     const int L = st.levels[q] - 1;
     const int64_t R = st.finalR[q] / cgrow;  // radius of level L - 1
     const int n = st.qbuf_n[(int64_t)(L & 1) * st.qbn_par + q];
-    uint64_t *E = st.qbuf + (int64_t)(L & 1) * st.qb_par + (int64_t)q * kQCap;
+    uint64_t *E = st.qbuf + (int64_t)q * kQCap;
     if (n > kQCap) return;  // the selection marks the query for the level path
     if (R > st.top[q]) {
         // the plain path stops at level L - 1 by radius: not this answer
@@ -1842,9 +2223,9 @@ qw_status launch_bitmap_build(const IndexView &ix, int c, int maxJ, uint4 *bm, u
         bm_or_level_kernel<<<grid, BM_THREADS, 0, s>>>(ix, bm, L, R, c);
         QW_CUDA_TRY(cudaGetLastError());
     }
-    const int64_t blocks = std::min<int64_t>(total_bitmaps, 152 * 64);
-    bm_summary_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), BM_THREADS, 0, s>>>(
-        bm, total_bitmaps, bm_sum);
+    QW_CUDA_TRY(cudaMemsetAsync(bm_sum + total_bitmaps * (kBmUint4 / 32), 0,
+                                (size_t)ix.nT * (kBmUint4 / 8), s));
+    bm_summary_kernel<<<grid, BM_THREADS, 0, s>>>(ix, bm, bm_sum);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
 }
@@ -1871,35 +2252,18 @@ ScanStats scan_stats_of(const IndexView &ix, int c)
 }
 
 template <int TPW>
-static void launch_filter_or_fused(const IndexView &ix, int nb, int level, int l, QueryState &st,
-                                   const LoopCtl *ctl, bool fused, cudaStream_t s)
+static void launch_fused(const IndexView &ix, int nb, int level, int l, QueryState &st,
+                         const LoopCtl *ctl, cudaStream_t s)
 {
     const int64_t tasks = (int64_t)nb * ((ix.nT + TPW - 1) / TPW);
     const int blocks = (int)std::max<int64_t>(
         1, std::min<int64_t>((tasks + FL_WARPS - 1) / FL_WARPS, 152 * 16));
-    if (fused) {
-        if (ix.m <= 32)
-            bm_fused_kernel<1, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
-        else if (ix.m <= 64)
-            bm_fused_kernel<2, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
-        else
-            bm_fused_kernel<4, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
-    } else {
-        if (ix.m <= 32)
-            bm_filter_kernel<1, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
-        else if (ix.m <= 64)
-            bm_filter_kernel<2, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
-        else
-            bm_filter_kernel<4, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
-    }
-}
-
-static void launch_filter_or_fused(const IndexView &ix, int nb, int level, int l, QueryState &st,
-                                   const LoopCtl *ctl, bool fused, int tpw, cudaStream_t s)
-{
-    if (tpw == 4) launch_filter_or_fused<4>(ix, nb, level, l, st, ctl, fused, s);
-    else if (tpw == 16) launch_filter_or_fused<16>(ix, nb, level, l, st, ctl, fused, s);
-    else launch_filter_or_fused<8>(ix, nb, level, l, st, ctl, fused, s);
+    if (ix.m <= 32)
+        bm_fused_kernel<1, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
+    else if (ix.m <= 64)
+        bm_fused_kernel<2, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
+    else
+        bm_fused_kernel<4, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
 }
 
 qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int64_t Rp, int l,
@@ -1908,35 +2272,41 @@ qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int
 {
     (void)Rp;
     (void)cgrow;
-    if (loads == QW_LOADS_FUSED) {
+    if (loads != QW_LOADS_TMA) {
         if (part != 2) {
-            const int64_t qi = (int64_t)nb * ix.m;
-            bm_bucket_kernel<<<(unsigned)std::max<int64_t>(
-                                   1, std::min<int64_t>((qi + 255) / 256, 152 * 8)),
-                               256, 0, s>>>(ix, level, R, nb, st, ctl);
+            // up to four entries per thread of one block cost less than a launch
+            const int64_t qi = (int64_t)nb * st.bm_mp;
+            const bool one = qi <= 4096;
+            bm_active_kernel<<<1, 1024, 0, s>>>(ix, level, R, nb, st, ctl, one);
             QW_CUDA_TRY(cudaGetLastError());
+            if (!one) {
+                bm_bucket_kernel<<<(unsigned)std::min<int64_t>((qi + 255) / 256, 152 * 8), 256, 0,
+                                   s>>>(ix, level, R, st, ctl);
+                QW_CUDA_TRY(cudaGetLastError());
+            }
         }
         if (part == 1) return QW_OK;
-        launch_filter_or_fused(ix, nb, level, l, st, ctl, true, tpw, s);
-        QW_CUDA_TRY(cudaGetLastError());
-        return QW_OK;
-    }
-    if (loads == QW_LOADS_DIRECT) {
+        if (loads == QW_LOADS_FUSED) {
+            if (tpw == 4) launch_fused<4>(ix, nb, level, l, st, ctl, s);
+            else if (tpw == 16) launch_fused<16>(ix, nb, level, l, st, ctl, s);
+            else launch_fused<8>(ix, nb, level, l, st, ctl, s);
+            QW_CUDA_TRY(cudaGetLastError());
+            return QW_OK;
+        }
         // two passes: filter on the summaries, then count the live groups
-        if (part != 2) {
-            const int64_t qi = (int64_t)nb * ix.m;
-            bm_bucket_kernel<<<(unsigned)std::max<int64_t>(
-                                   1, std::min<int64_t>((qi + 255) / 256, 152 * 8)),
-                               256, 0, s>>>(ix, level, R, nb, st, ctl);
-            QW_CUDA_TRY(cudaGetLastError());
-        }
-        if (part == 1) return QW_OK;
-        launch_filter_or_fused(ix, nb, level, l, st, ctl, false, tpw, s);
+        const int64_t tasks = (int64_t)nb * ((ix.nT + 3) / 4);
+        const unsigned blocks =
+            (unsigned)std::max<int64_t>(1, std::min<int64_t>((tasks + 7) / 8, 152 * 24));
+        bm_filter_kernel<<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, st, ctl);
         QW_CUDA_TRY(cudaGetLastError());
-        bm_count_kernel<<<152 * 8, 256, 0, s>>>(ix, level, l, st, ctl);
+        bm_count_kernel<<<blocks, 256, 0, s>>>(ix, level, l, st, ctl);
         QW_CUDA_TRY(cudaGetLastError());
-        if (st.bm_prof) {
-            bm_prof_kernel<<<1, 1, 0, s>>>(st);
+        // fewer queries than the dense form asks of an average group never take it
+        if (nb >= kDenseMin) {
+            const size_t smem = dense_smem_bytes();
+            QW_CUDA_TRY(cudaFuncSetAttribute(
+                bm_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            bm_dense_kernel<<<2 * 152, DN_THREADS, smem, s>>>(ix, level, R, l, st, ctl);
             QW_CUDA_TRY(cudaGetLastError());
         }
         return QW_OK;
@@ -2010,13 +2380,30 @@ qw_status launch_bm_collect(const IndexView &ix, int nb, int l, int cap, QuerySt
     return QW_OK;
 }
 
+qw_status launch_bm_list(const IndexView &ix, int nb, int l, QueryState &st, bool staged,
+                         cudaStream_t s)
+{
+    if (nb == 0) return QW_OK;
+    if (staged) {
+        const int64_t e = (int64_t)nb * st.bm_mp;
+        bm_final_bucket_kernel<<<(unsigned)std::min<int64_t>((e + 255) / 256, 152 * 8), 256, 0, s>>>(
+            ix, nb, st);
+        QW_CUDA_TRY(cudaGetLastError());
+    }
+    const int64_t tasks = (int64_t)nb * ((ix.nT + 3) / 4);
+    bm_list_kernel<<<(unsigned)std::min<int64_t>((tasks + 7) / 8, 152 * 24), 256, 0, s>>>(ix, l, nb,
+                                                                                        st);
+    QW_CUDA_TRY(cudaGetLastError());
+    return QW_OK;
+}
+
 int bm_reduce_wave(int nT)
 {
     return (int)std::max<int64_t>(1, kRdStoreBytes / ((int64_t)nT * kBmUint4 * kRdStoreWords * 16));
 }
 
 qw_status launch_bm_reduce(const IndexView &ix, int nb, int l, int cap, int cgrow,
-                           QueryState &st, bool tma, int wave_slots, cudaStream_t s)
+                           QueryState &st, int wave_slots, cudaStream_t s)
 {
     if (nb == 0) return QW_OK;
     QW_CUDA_TRY(cudaMemsetAsync(st.rd_ctl, 0, sizeof(int32_t), s));
@@ -2025,12 +2412,12 @@ qw_status launch_bm_reduce(const IndexView &ix, int nb, int l, int cap, int cgro
     QW_CUDA_TRY(cudaGetLastError());
     // one store's worth of slots (wave_slots); queries past it keep the
     // level-path answer
-    const unsigned grid = 152 * 6;
+    const unsigned grid = 152 * 12;
     const unsigned pb = (unsigned)((wave_slots + 127) / 128);
-    rd_count_kernel<<<grid, RD_THREADS, 0, s>>>(ix, l, st, tma, 0, wave_slots);
+    rd_count_kernel<<<grid, RD_THREADS, 0, s>>>(ix, l, st, 0, wave_slots);
     rd_plan_kernel<<<pb, 128, 0, s>>>(l, ix.m, cap, cgrow, st, 0, wave_slots, 0);
-    rd_scan_kernel<<<152 * 4, RD_THREADS, 0, s>>>(ix, st, tma, wave_slots);
-    rd_emit_kernel<<<grid, RD_THREADS, 0, s>>>(ix, st, tma, wave_slots);
+    rd_scan_kernel<<<152 * 4, RD_THREADS, 0, s>>>(ix, st, wave_slots);
+    rd_emit_kernel<<<grid, RD_THREADS, 0, s>>>(ix, st, wave_slots);
     rd_plan_kernel<<<pb, 128, 0, s>>>(l, ix.m, cap, cgrow, st, 0, wave_slots, 2);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;

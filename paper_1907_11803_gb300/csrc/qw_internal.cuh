@@ -115,7 +115,9 @@ struct IndexView {
     // bm_sum holds per bitmap 256 bits, bit g set when 128-id group g has an id.
     const uint4 *bm;
     const int32_t *perm;
-    const uint32_t *bm_sum;
+    const uint32_t *bm_sum;   // rows of 8 words, row bm_base[i] + k * nT + t for bitmap k
+                              // of tile t's block; nT zero rows from row bm_total on
+    int64_t bm_total = 0;     // bitmaps
     const float *Xloc;        // the data in locality order (row j = data id perm[j])
     const int32_t *inv;       // data id -> internal id
     const int64_t *bm_base;
@@ -205,16 +207,12 @@ struct QueryState {
     unsigned long long *level_passes = nullptr;  // profile mode: (query, level) passes run, else null
     uint4 *cbits = nullptr;           // bitmap path: 2 (level parity) x nb x nT candidate bitmaps
     int64_t cb_par = 0;         // uint4 per parity (batch capacity x nT x kBmUint4)
-    // bitmap path: per (level parity, query, tile) the number of candidates
-    // (0: the tile's candidate bitmap was not written at that level)
-    int32_t *clist_n = nullptr;
-    int64_t cln_par = 0;        // entries of clist_n per parity (batch capacity x nT)
-    // bitmap path: per (level parity, query) every candidate of the level as
+    int64_t cln_par = 0;        // (query, tile) pairs per parity (batch capacity x nT)
+    // bitmap path: per query every candidate of its last level as
     // (internal id << 32) | (was a candidate at the previous level << 8) | count,
-    // up to kQCap of them (qbuf_n counts beyond: more means overflow)
+    // up to kQCap of them; per (level parity, query) their number (more: overflow)
     uint64_t *qbuf = nullptr;
     int32_t *qbuf_n = nullptr;
-    int64_t qb_par = 0;         // entries of qbuf per parity (batch capacity x kQCap)
     int64_t qbn_par = 0;        // entries of qbuf_n per parity (batch capacity)
     // bitmap path selection: per query "answer on the level path" flags, and
     // tie lists of kEqCap original ids
@@ -228,25 +226,23 @@ struct QueryState {
     int32_t *rd_hist = nullptr;     // slots x kHistBins: counts of candidates not of C_{R/c}
     int64_t *rd_bq = nullptr;       // slots x 2 x QW_MAX_M: bitmap numbers in tile 0 (L, L - 1)
     uint4 *rd_store = nullptr;      // per slot of a wave, per group: 7 count planes + prev word
-    // bitmap path, two-pass level: item slots (query, tile) with their m bitmap
-    // numbers, and the work list of live (slot << 8 | group) entries
-    int32_t *bm_nitems = nullptr;   // 2 counters: items, work entries (per level)
-    int32_t *bm_nwork = nullptr;
-    int2 *bm_item_qt = nullptr;
-    int64_t *bm_bq = nullptr;       // per (query, projection): bitmap number in tile 0, or -1
-    int32_t *bm_item_bi = nullptr;  // per item, (m + 3) / 4 * 4 bitmap numbers (-1: none)
-    uint32_t *bm_amask = nullptr;   // per (level parity, query, tile): live groups, 8 words
-    int32_t *bm_work = nullptr;
-    // per work entry, (m + 63) / 64 words: the projections whose bucket touches
-    // the group (its summary bit); the others' words are zero and not read
-    unsigned long long *bm_wmask = nullptr;
-    int32_t bm_item_cap = 0;
-    int32_t bm_work_cap = 0;
+    // bitmap path, per (query, projection) of a level, rows of bm_mp entries (m
+    // padded to 16): the bucket's bitmap number in tile 0 (-1: no data), its
+    // summary row, its row in the dense form's table (4 bits each)
+    int32_t bm_mp = 0;
+    int32_t *bm_b0 = nullptr;
+    int32_t *bm_srow = nullptr;
+    uint32_t *bm_rows = nullptr;
+    uint32_t *bm_ctl = nullptr;     // the level's counters (qw_bitmap.cu)
+    int32_t *bm_run = nullptr;      // the queries that run at the level
+    // per (level parity, query, tile), 8 words: the groups with candidates at that
+    // level (before the count pass, and with fused loads: live groups)
+    uint32_t *bm_amask = nullptr;
     unsigned long long *bm_prof = nullptr;  // profile mode: live items, groups, words (summed)
 };
 
 // Candidates per query and level the bitmap path holds (more: the query is
-// answered by the level path).  4 MiB of lists per query (two levels).
+// answered by the level path).  2 MiB of lists per query.
 constexpr int kQCap = 262144;
 // Tie-list capacity per query on the bitmap path (larger tie classes are
 // answered by the level path).
@@ -306,14 +302,18 @@ ScanStats scan_stats_of(const IndexView &ix, int c);
 // staged-copy wait gave up.
 // part (direct and fused loads): 0 every launch of the level, 1 the bucket
 // numbers, 2 the summary filter and the count pass (and the profile counters).
-// tpw: tiles a warp of the filter / fused kernel takes (4, 8 or 16; else 8).
+// tpw: tiles a warp of the fused kernel takes (4, 8 or 16; else 8).
 qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int64_t Rp, int l,
                           int cgrow, QueryState &st, int *err, int loads, cudaStream_t s,
                           const LoopCtl *ctl = nullptr, int part = 0, int tpw = 8);
+// After the level loop: the candidates of every query's last level to its list
+// (staged: the level ran bm_level_tma_kernel).
+qw_status launch_bm_list(const IndexView &ix, int nb, int l, QueryState &st, bool staged,
+                         cudaStream_t s);
 // Rebuild the candidate lists of the queries whose last level overflowed them
-// (kept entries and tie class only); tma: the level ran bm_level_tma_kernel.
+// (kept entries and tie class only).
 qw_status launch_bm_reduce(const IndexView &ix, int nb, int l, int cap, int cgrow,
-                           QueryState &st, bool tma, int wave_slots, cudaStream_t s);
+                           QueryState &st, int wave_slots, cudaStream_t s);
 // Bytes of the rebuild's plane store, and how many slots it holds for an index
 // of nT tiles (more overflowing queries in one batch keep the level-path
 // answer).

@@ -384,7 +384,8 @@ __global__ void decide_kernel(int nb, int level, int64_t R, int cap, QueryState 
     if (st.level_passes) atomicAdd(st.level_passes, 1ull);
     if (!ss.prefix) sl = st.scan_level[q];
     const int32_t before = st.ncand[q];  // |C_R| of the previous level
-    const int32_t nc = st.cross[q];      // |C_R| of this level, summed over tiles
+    // |C_R| of this level (the bitmap path counts its list, the level path sums tiles)
+    const int32_t nc = st.qbuf_n ? st.qbuf_n[(int64_t)(level & 1) * st.qbn_par + q] : st.cross[q];
     st.cross[q] = 0;
     st.scan_full[q] += skipped;
     st.scan_level[q] = 0;
