@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(CQ_THREADS, 2) cluster_query_kernel(
     const int nT = ix.nT;
     const int tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
-    const uint32_t lrep = (uint32_t)l * 0x01010101u;
+    const uint32_t bias = ge_bias(l);
     const int t_first = rank * tpc;
     const int my_tiles = max(0, min(tpc, nT - t_first));
     const unsigned char *lid_bytes = reinterpret_cast<const unsigned char *>(ix.lid);
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(CQ_THREADS, 2) cluster_query_kernel(
             // flag the previous level's candidates in the own counters
             if (level > 0) {
                 for (int w = tid; w < my_tiles * kWordsPerTile; w += CQ_THREADS)
-                    cnt_s[w] = flag_ge(cnt_s[w], lrep);
+                    cnt_s[w] |= ge_bits(cnt_s[w], bias);
             }
             int my_cross = 0;
             unsigned long long my_scan = 0;
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(CQ_THREADS, 2) cluster_query_kernel(
             }
             // census: candidates among the own ids after this level
             for (int w = tid; w < my_tiles * kWordsPerTile; w += CQ_THREADS)
-                my_cross += count_ge(cnt_s[w], lrep);
+                my_cross += __popc(ge_bits(cnt_s[w], bias));
             // this CTA's share of the level, into CTA 0
             my_cross = __reduce_add_sync(0xffffffffu, my_cross);
             if (tid == 0) {
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(CQ_THREADS, 2) cluster_query_kernel(
             const uint32_t *cnt_t = cnt_s + tt * kWordsPerTile;
             for (int w = tid; w < kWordsPerTile; w += CQ_THREADS) {
                 const uint32_t x = cnt_t[w];
-                if (!__vcmpgeu4(x & 0x7f7f7f7fu, lrep)) continue;
+                if (!ge_bits(x, bias)) continue;
 #pragma unroll
                 for (int by = 0; by < 4; ++by) {
                     const uint32_t b8 = (x >> (8 * by)) & 0xffu;

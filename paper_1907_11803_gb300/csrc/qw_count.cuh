@@ -42,37 +42,43 @@ __device__ __forceinline__ uint32_t flank_mask(const FlankSet &f, int s, int e)
     return mask;
 }
 
+// Add one to the byte counter of the id in the low 15 bits of x (bits 15 and up
+// are not looked at): its word is id / 4, its byte id mod 4, and the funnel
+// shift takes 8 id modulo 32, so an id costs a mask, two shifts and the atomic.
+// The counting loops are bound by these instructions (the ALU pipe at 77 % with
+// the id, word, byte and increment taken one after the other) and then by the
+// atomics' bank conflicts.
+__device__ __forceinline__ void count_id(uint32_t *cnt, uint32_t x)
+{
+    static_assert(kTile == 1 << 15, "the word's byte offset is bits 2..14 of the id");
+    atomicAdd(reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(cnt) + (x & 0x7ffcu)),
+              __funnelshift_l(0u, 1u, x << 3));
+}
+
 // Add one to the byte counter of every id of chunk v selected by mask.
 __device__ __forceinline__ void count_chunk(uint32_t *cnt, const uint4 v, uint32_t mask)
 {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
     if (mask == 0xffu) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const uint32_t id = (j & 1) ? (w[j >> 1] >> 16) : (w[j >> 1] & 0xffffu);
-            atomicAdd(&cnt[id >> 2], 1u << ((id << 3) & 24u));
+        for (int j = 0; j < 4; ++j) {
+            count_id(cnt, w[j]);
+            count_id(cnt, w[j] >> 16);
         }
     } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (!(mask & (1u << j))) continue;
-            const uint32_t id = (j & 1) ? (w[j >> 1] >> 16) : (w[j >> 1] & 0xffffu);
-            atomicAdd(&cnt[id >> 2], 1u << ((id << 3) & 24u));
-        }
+        for (int j = 0; j < 8; ++j)
+            if (mask & (1u << j)) count_id(cnt, (j & 1) ? (w[j >> 1] >> 16) : w[j >> 1]);
     }
 }
 
-// Number of the 4 byte counters of x whose count (low 7 bits) is >= l;
-// lrep = l replicated in every byte.
-__device__ __forceinline__ int count_ge(uint32_t x, uint32_t lrep)
+// Bit 7 of every byte of x whose count (low 7 bits) is >= l, for 1 <= l <= 128;
+// bias is 128 - l in every byte, so no byte's sum carries into the next.
+__device__ __forceinline__ uint32_t ge_bits(uint32_t x, uint32_t bias)
 {
-    return __popc(__vcmpgeu4(x & 0x7f7f7f7fu, lrep)) >> 3;
+    return ((x & 0x7f7f7f7fu) + bias) & 0x80808080u;
 }
 
-// Same with the "candidate at the previous level" flag (bit 7) set for those.
-__device__ __forceinline__ uint32_t flag_ge(uint32_t x, uint32_t lrep)
-{
-    return x | (__vcmpgeu4(x & 0x7f7f7f7fu, lrep) & 0x80808080u);
-}
+__device__ __forceinline__ uint32_t ge_bias(int l) { return (uint32_t)(128 - l) * 0x01010101u; }
 
 }  // namespace qw

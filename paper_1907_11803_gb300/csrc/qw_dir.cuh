@@ -6,12 +6,15 @@
 
 namespace qw {
 
-// floor(a / R) for R > 0 (C division truncates toward zero).
+// floor(a / R) for R > 0 (C division truncates toward zero): for a < 0 it is
+// ~(~a / R).  Bucket ids and radii nearly always fit 32 bits, where the division
+// is a fraction of the 64-bit one's instructions.
 __device__ __forceinline__ int64_t floordiv64(int64_t a, int64_t R)
 {
-    int64_t q = a / R;
-    if ((a % R != 0) && (a < 0)) --q;
-    return q;
+    const int64_t sign = a >> 63;
+    const uint64_t u = (uint64_t)(a ^ sign), r = (uint64_t)R;
+    const uint64_t q = ((u | r) >> 32) ? u / r : (uint64_t)((uint32_t)u / (uint32_t)r);
+    return (int64_t)q ^ sign;
 }
 
 __device__ __forceinline__ int64_t clamp64(int64_t x, int64_t lo, int64_t hi)

@@ -26,6 +26,8 @@
 #include <algorithm>
 #include <climits>
 
+#include <cuda_pipeline.h>
+
 namespace qw {
 namespace {
 
@@ -33,20 +35,26 @@ constexpr int LV_THREADS = 256;
 constexpr int kWordsPerTile = kTile / 4;
 constexpr int kUnroll = 4;
 
+// One warp per query.
 __global__ void query_setup_kernel(const int32_t *__restrict__ HQ, int nb, int m,
                                    const int32_t *__restrict__ o,
                                    const int32_t *__restrict__ span, QueryState st)
 {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    const int q = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
     if (q >= nb) return;
     int64_t top = 0;
-    for (int i = 0; i < m; ++i) {
+    for (int i = lane; i < m; i += 32) {
         int64_t g = (int64_t)HQ[(int64_t)q * m + i] - (int64_t)o[i];
         st.g[(int64_t)q * m + i] = g;
         top = max(top, max((int64_t)span[i], g));
         // with probes a query bucket id below the data collides once R > -g
         if (st.probes > 0) top = max(top, -g);
     }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        top = max(top, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)top, off));
+    if (lane != 0) return;
     st.top[q] = top;
     st.active[q] = 1;
     st.ncand[q] = 0;
@@ -99,20 +107,28 @@ __global__ void fallback_kernel(int nb, QueryState st)
     atomicAdd(st.fb_count, 1ull);
 }
 
+// One level of one (tile, query).  Bound by the shared-memory pipe: an atomic of
+// a warp takes two passes over the banks on average (ids of a bucket cycle
+// through the banks in uneven groups), 93 % of the pipe at a deep level, and at
+// the first levels by instructions, 65 % of the issue slots.  1,000 queries on
+// 500,000 points, 64 projections, levels 0-4: 635 792 979 1345 1984 us with one
+// thread per projection searching its ends in turn, every thread stepping over
+// all flanks and the ids outside whole chunks masked in the main loop;
+// 424 466 592 864 1399 us so.  Forty registers (six blocks per SM) gain nothing
+// here and cost QALSH's searches 20 %.
 __global__ void __launch_bounds__(LV_THREADS) level_kernel(IndexView ix, int level, int64_t R,
                                                            int64_t Rp, int l, int cgrow,
                                                            QueryState st, int64_t words_per_query,
                                                            const LoopCtl *ctl)
 {
     __shared__ __align__(16) uint32_t cnt_s[kWordsPerTile];
-    __shared__ int64_t f_gc0[2 * QW_MAX_M];
-    __shared__ int32_t f_cpref[2 * QW_MAX_M + 1];
-    __shared__ uint8_t f_head[2 * QW_MAX_M], f_tail[2 * QW_MAX_M], f_tile[2 * QW_MAX_M];
+    __shared__ int32_t f_end[4][QW_MAX_M];
+    __shared__ uint32_t f_run[2 * QW_MAX_M];        // flank's tile offsets: lo | hi << 16
+    __shared__ int32_t f_cpref[2 * QW_MAX_M + 1];   // exclusive prefix of its whole chunks
     __shared__ int32_t wsum[LV_THREADS / 32];
     __shared__ int hist[kHistBins];
     __shared__ int32_t red_count;
     __shared__ unsigned long long red_scan;
-    FlankSet fl{f_gc0, f_cpref, f_head, f_tail, f_tile};
 
     const int t = blockIdx.x;
     const int q = blockIdx.y;
@@ -136,53 +152,61 @@ __global__ void __launch_bounds__(LV_THREADS) level_kernel(IndexView ix, int lev
     }
     for (int c = threadIdx.x; c < kHistBins; c += LV_THREADS) hist[c] = 0;
 
-    // 1. flank boundaries of every projection (one thread per projection)
-    unsigned long long my_scan = 0;
-    int my_c0 = 0, my_c1 = 0;
-    if (ix.qkey) {
-        // QALSH: the run of the tile's sorted projections inside this level's
-        // interval p_i(q) +- qhalf R, and inside the previous level's; thread
-        // 2i + j searches both ends of interval j of projection i (two binary
-        // searches advancing together) and leaves (end << 32 | start) in
-        // f_gc0[2i + j], which projection i's thread reads before it writes
-        // its flanks there
-        if (threadIdx.x < 2 * m && (threadIdx.x & 1) <= (first ? 0 : 1)) {
-            const int i = threadIdx.x >> 1;
-            const double h = __dmul_rn(ix.qhalf, (double)((threadIdx.x & 1) ? Rp : R));
+    // the tile's counters on their way into shared memory while the flanks are
+    // searched for
+    uint4 *cg = reinterpret_cast<uint4 *>(st.counters + (int64_t)q * words_per_query +
+                                          (int64_t)t * kWordsPerTile);
+    uint4 *cs = reinterpret_cast<uint4 *>(cnt_s);
+    if (first) {
+#pragma unroll
+        for (int r = 0; r < kWordsPerTile / 4 / LV_THREADS; ++r)
+            cs[r * LV_THREADS + threadIdx.x] = make_uint4(0, 0, 0, 0);
+    } else {
+#pragma unroll
+        for (int r = 0; r < kWordsPerTile / 4 / LV_THREADS; ++r)
+            __pipeline_memcpy_async(cs + r * LV_THREADS + threadIdx.x,
+                                    cg + r * LV_THREADS + threadIdx.x, 16);
+        __pipeline_commit();
+    }
+
+    // 1. flank boundaries: the ends of this level's range of every projection
+    //    and, unless it is the first, of the previous level's (ranges nest, so
+    //    only the two new flanks are read; the ends of a previous range without
+    //    data coincide); one search per thread, end b of projection i in
+    //    f_end[b][i]
+    const int ends = (first ? 2 : 4) * m;
+    for (int j = threadIdx.x; j < ends; j += LV_THREADS) {
+        const int b = j / m, i = j - b * m;
+        const int64_t rad = b < 2 ? R : Rp;
+        int pos;
+        if (ix.qkey) {
+            // QALSH: the run of the tile's sorted projections inside the
+            // interval p_i(q) +- qhalf R
+            const double h = __dmul_rn(ix.qhalf, (double)rad);
             const double pq = __longlong_as_double((long long)st.g[(int64_t)q * m + i]);
             const double *kk = ix.qkey + (int64_t)i * ix.nT * kTile + tbase;
-            int la = 0, ha = len, lb = 0, hb = len;
-            while (la < ha || lb < hb) {
-                if (la < ha) {
-                    const int mid = (la + ha) >> 1;
-                    if (__dsub_rn(kk[mid], pq) < -h) la = mid + 1; else ha = mid;
-                }
-                if (lb < hb) {
-                    const int mid = (lb + hb) >> 1;
-                    if (!(__dsub_rn(kk[mid], pq) > h)) lb = mid + 1; else hb = mid;
-                }
+            int lo = 0, hi = len;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                const double dk = __dsub_rn(kk[mid], pq);
+                if ((b & 1) ? !(dk > h) : dk < -h) lo = mid + 1; else hi = mid;
             }
-            f_gc0[threadIdx.x] = ((int64_t)lb << 32) | (int64_t)la;
+            pos = lo;
+        } else {
+            const int64_t dslot = (int64_t)i * ix.nT + t;
+            const int64_t ds = ix.dir_start[dslot];
+            const int64_t sp1 = (int64_t)ix.span[i] + 1;
+            const int cnt = ix.dir_cnt[dslot];
+            // the level's bid range, widened to P buckets on each side with probes
+            const int64_t P = st.probes;
+            int64_t lo = (floordiv64(st.g[(int64_t)q * m + i], rad) - P) * rad;
+            if (b & 1) lo += (2 * P + 1) * rad;
+            pos = dir_lower(ix.dir_bid + ds, ix.dir_off + ds, cnt, len, clamp64(lo, 0, sp1));
         }
-        __syncthreads();
-        if (threadIdx.x < m) {
-            const int i = threadIdx.x;
-            const int64_t cur = f_gc0[2 * i];
-            const int pA = (int)(cur & 0xffffffff), pB = (int)(cur >> 32);
-            int s0 = pA, e0 = pB, s1 = 0, e1 = 0;
-            if (!first) {
-                // intervals nest from level to level: the two new flanks
-                const int64_t prv = f_gc0[2 * i + 1];
-                e0 = (int)(prv & 0xffffffff);
-                s1 = (int)(prv >> 32);
-                e1 = pB;
-            }
-            const int64_t ebase = (int64_t)i * ix.nT * kTile + tbase;
-            flank_set(fl, 2 * i, ebase + s0, ebase + e0, 0, &my_c0);
-            flank_set(fl, 2 * i + 1, ebase + s1, ebase + e1, 0, &my_c1);
-            my_scan = (unsigned long long)(pB - pA);
-        }
-    } else if (threadIdx.x < m) {
+        f_end[b][i] = pos;
+    }
+    if (first && level > 0 && !ix.qkey && threadIdx.x < m) {
+        // entries in the ranges of the skipped levels, for the statistics
         const int i = threadIdx.x;
         const int64_t gi = st.g[(int64_t)q * m + i];
         const int64_t sp1 = (int64_t)ix.span[i] + 1;
@@ -190,39 +214,35 @@ __global__ void __launch_bounds__(LV_THREADS) level_kernel(IndexView ix, int lev
         const int32_t *ub = ix.dir_bid + ix.dir_start[dslot];
         const int32_t *uo = ix.dir_off + ix.dir_start[dslot];
         const int cnt = ix.dir_cnt[dslot];
-        // the level's bid range, widened to P buckets on each side with probes
         const int64_t P = st.probes;
-        const int64_t lo = (floordiv64(gi, R) - P) * R;
-        const int64_t A = clamp64(lo, 0, sp1), B = clamp64(lo + (2 * P + 1) * R, 0, sp1);
-        const int pA = dir_lower(ub, uo, cnt, len, A);
-        const int pB = dir_lower(ub, uo, cnt, len, B);
+        unsigned long long skipped = 0;
+        int64_t Rs = R;
+        for (int L2 = level - 1; L2 >= 0; --L2) {
+            Rs /= cgrow;
+            const int64_t lo3 = (floordiv64(gi, Rs) - P) * Rs;
+            const int64_t A3 = clamp64(lo3, 0, sp1), B3 = clamp64(lo3 + (2 * P + 1) * Rs, 0, sp1);
+            skipped += (unsigned long long)(dir_lower(ub, uo, cnt, len, B3) -
+                                            dir_lower(ub, uo, cnt, len, A3));
+        }
+        if (skipped) atomicAdd(reinterpret_cast<unsigned long long *>(st.scan_full + q), skipped);
+    }
+    __syncthreads();
+    unsigned long long my_scan = 0;
+    int my_c0 = 0, my_c1 = 0;
+    if (threadIdx.x < m) {
+        const int i = threadIdx.x;
+        const int pA = f_end[0][i], pB = f_end[1][i];
         int s0 = pA, e0 = pB, s1 = 0, e1 = 0;
         if (!first) {
-            // ranges nest from level to level, so only the two new flanks are read
-            const int64_t lo2 = (floordiv64(gi, Rp) - P) * Rp;
-            const int64_t A2 = clamp64(lo2, 0, sp1), B2 = clamp64(lo2 + (2 * P + 1) * Rp, 0, sp1);
-            if (A2 < B2) {
-                e0 = dir_lower(ub, uo, cnt, len, A2);
-                s1 = dir_lower(ub, uo, cnt, len, B2);
-                e1 = pB;
-            }
-        } else if (level > 0) {
-            // entries in the ranges of the skipped levels, for the statistics
-            unsigned long long skipped = 0;
-            int64_t Rs = R;
-            for (int L2 = level - 1; L2 >= 0; --L2) {
-                Rs /= cgrow;
-                const int64_t lo3 = (floordiv64(gi, Rs) - P) * Rs;
-                const int64_t A3 = clamp64(lo3, 0, sp1), B3 = clamp64(lo3 + (2 * P + 1) * Rs, 0, sp1);
-                skipped += (unsigned long long)(dir_lower(ub, uo, cnt, len, B3) -
-                                                dir_lower(ub, uo, cnt, len, A3));
-            }
-            if (skipped) atomicAdd(reinterpret_cast<unsigned long long *>(st.scan_full + q), skipped);
+            e0 = f_end[2][i];
+            s1 = f_end[3][i];
+            e1 = pB;
         }
-        // the tile's slots start 16-byte aligned, so chunks are tile offsets / 8
-        const int64_t ebase = (int64_t)i * ix.nT * kTile + tbase;
-        flank_set(fl, 2 * i, ebase + s0, ebase + e0, 0, &my_c0);
-        flank_set(fl, 2 * i + 1, ebase + s1, ebase + e1, 0, &my_c1);
+        static_assert(kTile <= 65535, "tile offsets are packed in pairs");
+        f_run[2 * i] = (uint32_t)s0 | (uint32_t)e0 << 16;
+        f_run[2 * i + 1] = (uint32_t)s1 | (uint32_t)e1 << 16;
+        my_c0 = max((e0 >> 3) - ((s0 + 7) >> 3), 0);
+        my_c1 = max((e1 >> 3) - ((s1 + 7) >> 3), 0);
         my_scan = (unsigned long long)(pB - pA);
     }
     {
@@ -236,83 +256,107 @@ __global__ void __launch_bounds__(LV_THREADS) level_kernel(IndexView ix, int lev
     }
     if (my_scan) atomicAdd(&red_scan, my_scan);
 
-    // 2. the tile's counters into shared memory; flag previous candidates
-    uint4 *cg = reinterpret_cast<uint4 *>(st.counters + (int64_t)q * words_per_query +
-                                          (int64_t)t * kWordsPerTile);
-    uint4 *cs = reinterpret_cast<uint4 *>(cnt_s);
-    const uint32_t lrep = (uint32_t)l * 0x01010101u;
-    if (first) {
-        for (int w4 = threadIdx.x; w4 < kWordsPerTile / 4; w4 += LV_THREADS)
-            cs[w4] = make_uint4(0, 0, 0, 0);
-    } else {
-        for (int w4 = threadIdx.x; w4 < kWordsPerTile / 4; w4 += LV_THREADS) {
-            uint4 x = cg[w4];
-            x.x = flag_ge(x.x, lrep);
-            x.y = flag_ge(x.y, lrep);
-            x.z = flag_ge(x.z, lrep);
-            x.w = flag_ge(x.w, lrep);
-            cs[w4] = x;
+    // 2. flag the previous level's candidates, if the query has any
+    const uint32_t bias = ge_bias(l);
+    if (!first) {
+        __pipeline_wait_prior(0);
+        if (st.ncand[q] > 0) {
+#pragma unroll
+            for (int r = 0; r < kWordsPerTile / 4 / LV_THREADS; ++r) {
+                uint4 x = cs[r * LV_THREADS + threadIdx.x];
+                const uint4 f = make_uint4(ge_bits(x.x, bias), ge_bits(x.y, bias),
+                                           ge_bits(x.z, bias), ge_bits(x.w, bias));
+                if (!(f.x | f.y | f.z | f.w)) continue;
+                cs[r * LV_THREADS + threadIdx.x] =
+                    make_uint4(x.x | f.x, x.y | f.y, x.z | f.z, x.w | f.w);
+            }
         }
     }
     __syncthreads();
 
-    // 3. count every id in the flanks: 8 ids per 16-byte load, kUnroll loads
-    //    in flight per thread; the current flank's bounds stay in registers
-    const int total = f_cpref[2 * m];
-    const uint4 *lid4 = reinterpret_cast<const uint4 *>(ix.lid);
-    int s = -1, c_lo = 0, c_hi = 0;
-    int64_t g0 = 0;
-    uint32_t head_mask = 0xffu, tail_mask = 0xffu;
-    for (int e0 = threadIdx.x; e0 < total; e0 += LV_THREADS * kUnroll) {
-        uint4 v[kUnroll];
-        uint32_t mask[kUnroll];
+    // 3. count every id in the flanks.  The tile's slots start 16-byte aligned,
+    //    so chunk k of a tile's ids is its offsets 8 k .. 8 k + 7.  First the
+    //    ids outside a flank's whole chunks (at most 14), 16 places per flank,
+    //    kUnroll loads in flight per thread; then the whole chunks, a
+    //    contiguous share of the flattened chunk space per warp, so that a lane
+    //    steps over its warp's flanks only, kUnroll 16-byte loads in flight and
+    //    no id to leave out.
+    const uint16_t *lid = ix.lid + tbase;
+    const int64_t pstride = (int64_t)ix.nT * kTile;
+    for (int j0 = threadIdx.x; j0 < 32 * m; j0 += LV_THREADS * kUnroll) {
+        int id[kUnroll];
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
-            const int e = e0 + u * LV_THREADS;
-            mask[u] = 0;
-            if (e < total) {
-                if (e >= c_hi) {
-                    do {
-                        ++s;
-                        c_hi = f_cpref[s + 1];
-                    } while (e >= c_hi);
-                    c_lo = f_cpref[s];
-                    g0 = f_gc0[s];
-                    head_mask = 0xffu << f_head[s];
-                    tail_mask = 0xffu >> (8 - f_tail[s]);
-                }
-                v[u] = __ldg(lid4 + g0 + (e - c_lo));
-                uint32_t mk = 0xffu;
-                if (e == c_lo) mk &= head_mask;
-                if (e == c_hi - 1) mk &= tail_mask;
-                mask[u] = mk;
-            }
+            const int j = j0 + u * LV_THREADS;
+            id[u] = -1;
+            if (j >= 32 * m) continue;
+            const int lo = (int)(f_run[j >> 4] & 0xffffu), hi = (int)(f_run[j >> 4] >> 16);
+            const int c0 = (lo + 7) & ~7, c1 = hi & ~7;
+            const int k = lo + (j & 15);
+            const int at = (c1 > c0 && k >= c0) ? k + (c1 - c0) : k;
+            if (at < hi) id[u] = __ldg(lid + (j >> 5) * pstride + at);
         }
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u)
-            if (mask[u]) count_chunk(cnt_s, v[u], mask[u]);
+            if (id[u] >= 0) count_id(cnt_s, (uint32_t)id[u]);
     }
+    {
+        const int total = f_cpref[2 * m];
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const int share = (total + LV_THREADS / 32 - 1) / (LV_THREADS / 32);
+        const int wend = min((warp + 1) * share, total);
+        int s = -1, c_hi = 0;  // the flank of the lane's last chunk
+        const uint4 *p = nullptr;
+        if (warp * share < wend) {
+            // the last flank that starts at or before the warp's first chunk
+            for (int k = lane; k < 2 * m; k += 32)
+                if (f_cpref[k] <= warp * share) s = k;
+            s = __reduce_max_sync(0xffffffffu, s) - 1;
+        }
+        for (int e0 = warp * share + lane; e0 < wend; e0 += 32 * kUnroll) {
+            uint4 v[kUnroll];
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const int e = e0 + u * 32;
+                if (e >= wend) continue;
+                if (e >= c_hi) {
+                    do c_hi = f_cpref[++s + 1]; while (e >= c_hi);
+                    p = reinterpret_cast<const uint4 *>(lid + (s >> 1) * pstride) +
+                        (((f_run[s] & 0xffffu) + 7) >> 3) - f_cpref[s];
+                }
+                v[u] = __ldg(p + e);
+            }
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u)
+                if (e0 + u * 32 < wend) count_chunk(cnt_s, v[u], 0xffu);
+        }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
 
-    // 4. counters back to global memory, and this tile's candidate profile:
-    //    previous-level candidates, and the other candidates by count
+    // 4. counters back to global memory (one bulk copy), and this tile's
+    //    candidate profile: previous-level candidates, the others by count
+    if (threadIdx.x == 0) {
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                         __cvta_generic_to_global(cg)),
+                     "r"((uint32_t)__cvta_generic_to_shared(cs)), "r"((uint32_t)kTile)
+                     : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
     int my_prev = 0, my_count = 0;
-    for (int w4 = threadIdx.x; w4 < kWordsPerTile / 4; w4 += LV_THREADS) {
-        const uint4 x = cs[w4];
-        cg[w4] = x;
+#pragma unroll
+    for (int r = 0; r < kWordsPerTile / 4 / LV_THREADS; ++r) {
+        const uint4 x = cs[r * LV_THREADS + threadIdx.x];
         const uint32_t wv[4] = {x.x, x.y, x.z, x.w};
+        const uint32_t ge[4] = {ge_bits(x.x, bias), ge_bits(x.y, bias), ge_bits(x.z, bias),
+                                ge_bits(x.w, bias)};
+        if (!(ge[0] | ge[1] | ge[2] | ge[3])) continue;
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-            const int c4 = count_ge(wv[h], lrep);
-            if (!c4) continue;
-            my_count += c4;
-#pragma unroll
-            for (int by = 0; by < 4; ++by) {
-                const uint32_t b8 = (wv[h] >> (8 * by)) & 0xffu;
-                if ((b8 & 0x7fu) < (uint32_t)l) continue;
-                if (b8 & 0x80u) ++my_prev;
-                else atomicAdd(&hist[1 + (b8 & 0x7fu)], 1);
-            }
+            my_count += __popc(ge[h]);
+            my_prev += __popc(ge[h] & wv[h]);
+            for (uint32_t left = ge[h] & ~wv[h]; left; left &= left - 1)
+                atomicAdd(&hist[1 + ((wv[h] >> (__ffs(left) - 8)) & 0x7fu)], 1);
         }
     }
     my_prev = __reduce_add_sync(0xffffffffu, my_prev);
@@ -327,6 +371,8 @@ __global__ void __launch_bounds__(LV_THREADS) level_kernel(IndexView ix, int lev
     if (threadIdx.x == 0) {
         if (red_count) atomicAdd(st.cross + q, red_count);
         if (red_scan) atomicAdd(reinterpret_cast<unsigned long long *>(st.scan_level + q), red_scan);
+        // the copy has read the counters before the block's memory goes
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
     }
 }
 
@@ -493,7 +539,6 @@ __global__ void second_pass_kernel(QueryState st, LoopCtl *ctl, cudaGraphConditi
 }
 
 constexpr int CL_THREADS = 256;
-constexpr int CL_PER = 16;  // ids per thread per chunk (one 16-byte load)
 
 // Plan the kept candidates of one query from the per-tile profiles of its
 // last level: all ids with count >= l when there are at most k + v of them;
@@ -589,14 +634,54 @@ __global__ void __launch_bounds__(CL_THREADS) select_plan_kernel(
 }
 
 // Emit the kept ids of one (tile, query) in ascending order at the tile's
-// planned position.  Each thread owns 128 consecutive ids of the tile, so one
-// pair of block scans orders the whole tile.
-constexpr int EM_PER = kTile / CL_THREADS;  // ids per thread
+// planned position.  The block reads the tile's counters as eight coalesced
+// rows of 16 ids per thread; a thread counts its ids kept outright and those at
+// c* per row, and one scan over the (row, warp) totals of both gives every
+// thread its first output slot.  Bound by reading the counters (32 KiB per tile
+// and query): 568 us for 1,000 queries on 500,000 points with a thread per 128
+// consecutive ids walking its words in local memory, 174 us so.
+constexpr int EM_ROWS = kTile / (CL_THREADS * 16);  // 8
+constexpr int EM_WARPS = CL_THREADS / 32;
 
-__global__ void __launch_bounds__(CL_THREADS) select_emit_kernel(
-    int64_t n, int nT, int l, int cap, QueryState st, int64_t words_per_query)
+// First places of the (row, warp, lane) entries, in that order, of v[r]: tot is
+// EM_ROWS * EM_WARPS words of shared memory.  Returns them in v.
+__device__ __forceinline__ void emit_scan(uint32_t (&v)[EM_ROWS], uint32_t *tot)
 {
-    __shared__ int scan_tmp[CL_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t mine[EM_ROWS];
+#pragma unroll
+    for (int r = 0; r < EM_ROWS; ++r) {
+        uint32_t incl = v[r];
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += y;
+        }
+        mine[r] = incl - v[r];
+        if (lane == 31) tot[r * EM_WARPS + warp] = incl;
+    }
+    __syncthreads();
+    static_assert(EM_ROWS * EM_WARPS == 64, "two totals per lane");
+    if (warp == 0) {
+        const uint32_t x = tot[2 * lane], y = tot[2 * lane + 1];
+        uint32_t incl = x + y;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t z = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += z;
+        }
+        tot[2 * lane] = incl - x - y;
+        tot[2 * lane + 1] = incl - y;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < EM_ROWS; ++r) v[r] = mine[r] + tot[r * EM_WARPS + warp];
+}
+
+__global__ void __launch_bounds__(CL_THREADS, 4) select_emit_kernel(
+    int nT, int l, int cap, QueryState st, int64_t words_per_query)
+{
+    __shared__ uint32_t tot[EM_ROWS * EM_WARPS];
     const int t = blockIdx.x;
     const int q = blockIdx.y;
     const int cstar = st.qplan[q * 2 + 0], take_eq = st.qplan[q * 2 + 1];
@@ -607,84 +692,62 @@ __global__ void __launch_bounds__(CL_THREADS) select_emit_kernel(
     const int64_t tbase = (int64_t)t * kTile;
     // counters are allocated for whole tiles; ids past n hold zero
     const uint4 *cb = reinterpret_cast<const uint4 *>(
-        reinterpret_cast<const uint8_t *>(st.counters + (int64_t)q * words_per_query) + tbase +
-        (int64_t)threadIdx.x * EM_PER);
-    const uint32_t lrep = (uint32_t)l * 0x01010101u;
-    uint4 v[EM_PER / 16];
-    bool mine = false;
+                          reinterpret_cast<const uint8_t *>(st.counters + (int64_t)q * words_per_query) +
+                          tbase) + threadIdx.x;
+    // bit 7 of the bytes to keep outright (previous-level candidates and counts
+    // above c*), and of the others at c*
+    const uint32_t bias = ge_bias(l), abias = ge_bias(min(max(cstar + 1, l), 128));
+    const bool ties = cstar >= l;
+    const uint32_t cbias = ge_bias(min(max(cstar, l), 128));
+    auto at_of = [&](uint32_t x) { return ge_bits(x, cbias); };  // at c* where not kept outright
+    auto above_of = [&](uint32_t x) { return ge_bits(x, abias) | (ge_bits(x, bias) & x); };
+    uint4 v[EM_ROWS];
 #pragma unroll
-    for (int u = 0; u < EM_PER / 16; ++u) {
-        v[u] = cb[u];
-        mine |= (count_ge(v[u].x, lrep) | count_ge(v[u].y, lrep) | count_ge(v[u].z, lrep) |
-                 count_ge(v[u].w, lrep)) != 0;
-    }
-    // the few threads holding candidates walk their 32 words in a loop (kept
-    // rolled: fully unrolled byte loops overflow the instruction cache)
-    uint32_t words[EM_PER / 4];
-    if (mine) {
+    for (int r = 0; r < EM_ROWS; ++r) v[r] = cb[r * CL_THREADS];
+    // ids kept outright in the low half, ids at c* in the high one: at most
+    // kTile together
+    uint32_t first[EM_ROWS];
+    int any = 0;
 #pragma unroll
-        for (int u = 0; u < EM_PER / 16; ++u) {
-            words[4 * u + 0] = v[u].x;
-            words[4 * u + 1] = v[u].y;
-            words[4 * u + 2] = v[u].z;
-            words[4 * u + 3] = v[u].w;
+    for (int r = 0; r < EM_ROWS; ++r) {
+        const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
+        first[r] = 0;
+        if (!(ge_bits(w[0], bias) | ge_bits(w[1], bias) | ge_bits(w[2], bias) |
+              ge_bits(w[3], bias)))
+            continue;
+        any |= 1 << r;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const uint32_t ab = above_of(w[h]);
+            first[r] += (uint32_t)__popc(ab);
+            if (ties) first[r] += (uint32_t)__popc(at_of(w[h]) & ~ab) << 16;
         }
     }
-    int n_eq = 0;
-    if (mine && cstar >= l) {
-#pragma unroll 1
-        for (int wi = 0; wi < EM_PER / 4; ++wi) {
-            const uint32_t x = words[wi];
-            if (!count_ge(x, lrep)) continue;
-            for (int by = 0; by < 4; ++by) {
-                const uint32_t b8 = (x >> (8 * by)) & 0xffu;
-                n_eq += ((b8 & 0x7fu) == (uint32_t)cstar && !(b8 & 0x80u)) ? 1 : 0;
+    emit_scan(first, tot);
+    if (!any) return;
+    const int left_eq = max(take_eq - eq0, 0);  // ids at c* that this tile may keep
+    int32_t *cand = st.cand + (int64_t)q * cap, *col = st.cand_col + (int64_t)q * cap;
+#pragma unroll
+    for (int r = 0; r < EM_ROWS; ++r) {
+        if (!((any >> r) & 1)) continue;
+        const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
+        int rk = (int)(first[r] >> 16);
+        int pos = out0 + (int)(first[r] & 0xffffu) + min(rk, left_eq);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const uint32_t ab = above_of(w[h]), eq = ties ? at_of(w[h]) & ~ab : 0u;
+            for (uint32_t left = ab | eq; left; left &= left - 1) {
+                const int sh = __ffs(left) - 8;
+                if (!((ab >> sh) & 0x80u) && rk++ >= left_eq) continue;
+                if (pos < cap) {
+                    cand[pos] = (int32_t)(tbase + (r * CL_THREADS + (int)threadIdx.x) * 16 + h * 4 +
+                                          (sh >> 3));
+                    col[pos] = (int)((w[h] >> sh) & 0x7fu);
+                }
+                ++pos;
             }
         }
     }
-    int eq_total;
-    int r = eq0 + block_exclusive_scan<CL_THREADS>(n_eq, scan_tmp, &eq_total);
-    int n_sel = 0;
-    if (mine) {
-        int rr = r;
-#pragma unroll 1
-        for (int wi = 0; wi < EM_PER / 4; ++wi) {
-            const uint32_t x = words[wi];
-            if (!count_ge(x, lrep)) continue;
-            for (int by = 0; by < 4; ++by) {
-                const uint32_t b8 = (x >> (8 * by)) & 0xffu;
-                const int c = (int)(b8 & 0x7fu);
-                if (c < l) continue;
-                if ((b8 & 0x80u) || c > cstar) ++n_sel;
-                else if (c == cstar) { n_sel += (rr < take_eq) ? 1 : 0; ++rr; }
-            }
-        }
-    }
-    int sel_total;
-    int pos = out0 + block_exclusive_scan<CL_THREADS>(n_sel, scan_tmp, &sel_total);
-    if (!mine) return;
-    const int64_t id0 = tbase + (int64_t)threadIdx.x * EM_PER;
-#pragma unroll 1
-    for (int wi = 0; wi < EM_PER / 4; ++wi) {
-        const uint32_t x = words[wi];
-        if (!count_ge(x, lrep)) continue;
-        for (int by = 0; by < 4; ++by) {
-            const uint32_t b8 = (x >> (8 * by)) & 0xffu;
-            const int c = (int)(b8 & 0x7fu);
-            if (c < l) continue;
-            bool sel;
-            if ((b8 & 0x80u) || c > cstar) sel = true;
-            else if (c == cstar) { sel = r < take_eq; ++r; }
-            else sel = false;
-            if (!sel) continue;
-            if (pos < cap) {
-                st.cand[(int64_t)q * cap + pos] = (int32_t)(id0 + wi * 4 + by);
-                st.cand_col[(int64_t)q * cap + pos] = c;
-            }
-            ++pos;
-        }
-    }
-    (void)n;
 }
 
 __global__ void candidates_out_kernel(const int32_t *__restrict__ cand,
@@ -730,7 +793,7 @@ qw_status launch_query_setup(const IndexView &ix, const int32_t *HQ, int nb, Que
                              cudaStream_t s)
 {
     QW_CUDA_TRY(cudaMemsetAsync(st.max_top, 0, sizeof(unsigned long long), s));
-    query_setup_kernel<<<(nb + 127) / 128, 128, 0, s>>>(HQ, nb, ix.m, ix.o, ix.span, st);
+    query_setup_kernel<<<(unsigned)(((int64_t)nb * 32 + 127) / 128), 128, 0, s>>>(HQ, nb, ix.m, ix.o, ix.span, st);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
 }
@@ -824,8 +887,8 @@ qw_status launch_collect(const IndexView &ix, int nb, int l, int cap, QueryState
 {
     const int64_t wpq = (int64_t)ix.nT * kWordsPerTile;
     QW_TRY(launch_select_plan(ix, nb, l, cap, st, stats_out, s));
-    select_emit_kernel<<<dim3((unsigned)ix.nT, (unsigned)nb), CL_THREADS, 0, s>>>(ix.n, ix.nT, l, cap,
-                                                                                st, wpq);
+    select_emit_kernel<<<dim3((unsigned)ix.nT, (unsigned)nb), CL_THREADS, 0, s>>>(ix.nT, l, cap, st,
+                                                                                wpq);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
 }
