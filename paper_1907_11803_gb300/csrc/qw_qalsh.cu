@@ -78,6 +78,41 @@ __global__ void __launch_bounds__(PJ_THREADS) fp64_project_kernel(
     }
 }
 
+// The same for few rows (the queries of a batch): one thread per (row,
+// projection), 32 rows and 8 projections per block, the operands of 64
+// coordinates at a time in shared memory as doubles.  64 rows and every
+// projection per block, the form above, gives 500 queries 8 blocks: 576 us, the
+// chains of 16 projections per thread one after the other on one SM's two FP64
+// lanes; 16 us so.
+constexpr int PQ_ROWS = 32, PQ_PROJ = 8, PQ_K = 64;
+
+__global__ void __launch_bounds__(PQ_ROWS *PQ_PROJ) fp64_project_few_kernel(
+    const float *__restrict__ V, int64_t nv, int d, const float *__restrict__ A, int m,
+    double *__restrict__ out, int64_t ld_r, int64_t ld_i)
+{
+    __shared__ double Vs[PQ_K][PQ_ROWS + 1];
+    __shared__ double As[PQ_K][PQ_PROJ];
+    const int64_t r0 = (int64_t)blockIdx.x * PQ_ROWS;
+    const int i0 = blockIdx.y * PQ_PROJ;
+    const int r = threadIdx.x % PQ_ROWS, p = threadIdx.x / PQ_ROWS;
+    double acc = 0.0;
+    for (int j0 = 0; j0 < d; j0 += PQ_K) {
+        const int kc = min(PQ_K, d - j0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < PQ_ROWS * PQ_K; e += PQ_ROWS * PQ_PROJ) {
+            const int rr = e / PQ_K, jj = e % PQ_K;
+            Vs[jj][rr] = (r0 + rr < nv && jj < kc) ? (double)V[(r0 + rr) * d + j0 + jj] : 0.0;
+        }
+        for (int e = threadIdx.x; e < PQ_PROJ * PQ_K; e += PQ_ROWS * PQ_PROJ) {
+            const int ii = e / PQ_K, jj = e % PQ_K;
+            As[jj][ii] = (i0 + ii < m && jj < kc) ? (double)A[(int64_t)(i0 + ii) * d + j0 + jj] : 0.0;
+        }
+        __syncthreads();
+        for (int jj = 0; jj < kc; ++jj) acc = fma(As[jj][p], Vs[jj][r], acc);
+    }
+    if (r0 + r < nv && i0 + p < m) out[(r0 + r) * ld_r + (int64_t)(i0 + p) * ld_i] = acc;
+}
+
 // ---------------------------------------------------------------- order-preserving keys
 // Unsigned 64-bit key with the order of the double (finite values; -0 < +0).
 __device__ __forceinline__ unsigned long long dkey(double x)
@@ -228,20 +263,24 @@ __global__ void __launch_bounds__(QS_THREADS) qalsh_sort_kernel(
 // ---------------------------------------------------------------- per-query setup
 // The query's projections are in st.g (as FP64 bits).  top: one below the
 // first radius R = c^j at which every projection's interval holds the whole
-// data, so that the level loop's "R > top" is the radius rule.
+// data, so that the level loop's "R > top" is the radius rule.  One warp per
+// query, a lane's projections one after the other (one thread per query took
+// 235 us for 500 queries of 64 projections, 6 us so).
 __global__ void qalsh_setup_kernel(int nb, int m, const double *__restrict__ qmin,
                                    const double *__restrict__ qmax, double half_unit, int cgrow,
                                    QueryState st, int *err)
 {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    const int q = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
     if (q >= nb) return;
     int64_t topR = 1;
-    for (int i = 0; i < m; ++i) {
+    for (int i = lane; i < m; i += 32) {
         const double pq = __longlong_as_double((long long)st.g[(int64_t)q * m + i]);
+        const double lo = qmin[i], hi = qmax[i];
         int64_t R = 1;
         for (;;) {
             const double h = __dmul_rn(half_unit, (double)R);
-            if (fabs(__dsub_rn(qmin[i], pq)) <= h && fabs(__dsub_rn(qmax[i], pq)) <= h) break;
+            if (fabs(__dsub_rn(lo, pq)) <= h && fabs(__dsub_rn(hi, pq)) <= h) break;
             if (R > INT64_MAX / cgrow) {
                 atomicOr(err, 2);  // no radius of int64 reaches every object
                 break;
@@ -250,6 +289,10 @@ __global__ void qalsh_setup_kernel(int nb, int m, const double *__restrict__ qmi
         }
         topR = max(topR, R);
     }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        topR = max(topR, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)topR, off));
+    if (lane != 0) return;
     const int64_t top = topR - 1;
     st.top[q] = top;
     st.active[q] = 1;
@@ -275,6 +318,13 @@ qw_status launch_fp64_project(const float *V, int64_t nv, int d, const float *A,
 {
     if (nv == 0) return QW_OK;
     const int64_t blocks = (nv + PJ_ROWS - 1) / PJ_ROWS;
+    if (blocks < 2 * 152) {  // fewer blocks than two per SM
+        const dim3 grid((unsigned)((nv + PQ_ROWS - 1) / PQ_ROWS),
+                        (unsigned)((m + PQ_PROJ - 1) / PQ_PROJ));
+        fp64_project_few_kernel<<<grid, PQ_ROWS * PQ_PROJ, 0, s>>>(V, nv, d, A, m, out, ld_r, ld_i);
+        QW_CUDA_TRY(cudaGetLastError());
+        return QW_OK;
+    }
     fp64_project_kernel<<<(unsigned)blocks, PJ_THREADS, 0, s>>>(V, nv, d, A, m, out, ld_r, ld_i);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
@@ -313,7 +363,7 @@ qw_status launch_qalsh_setup(const IndexView &ix, int nb, QueryState &st, int cg
 {
     QW_CUDA_TRY(cudaMemsetAsync(st.max_top, 0, sizeof(unsigned long long), s));
     if (nb == 0) return QW_OK;
-    qalsh_setup_kernel<<<(nb + 127) / 128, 128, 0, s>>>(nb, ix.m, ix.qmin, ix.qmax, ix.qhalf,
+    qalsh_setup_kernel<<<(unsigned)(((int64_t)nb * 32 + 127) / 128), 128, 0, s>>>(nb, ix.m, ix.qmin, ix.qmax, ix.qhalf,
                                                         cgrow, st, err);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
