@@ -970,7 +970,7 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
         QW_TRY(ix->w_bmsel.ensure((size_t)B * (2 + kEqCap) * sizeof(int32_t) + 256 +
                                   (size_t)B * sizeof(RdPlan) +
                                   (size_t)B * 2 * kHistBins * sizeof(int32_t) +
-                                  (size_t)B * 2 * QW_MAX_M * sizeof(int64_t)));
+                                  (size_t)B * QW_MAX_M * sizeof(int64_t)));
         QW_TRY(ix->w_bmwork.ensure(bm_work_layout(B, ix->nT, m, nullptr)));
         // the overflow rebuild's plane store: one wave of slots
         QW_TRY(ix->w_rdstore.ensure((size_t)std::min<int64_t>(B, bm_reduce_wave(ix->nT)) *
@@ -1270,11 +1270,11 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
                 QW_TRY(host_level_loop(ix, tm, view, nb, cap, learned, use_bitmap, loads, tpw, err,
                                        st, s, &levels_run));
             }
-            QW_TRY(tm.run(QW_K_SELECT, use_bitmap ? (learned ? 5 : 3) : 2, [&] {
+            QW_TRY(tm.run(QW_K_SELECT, use_bitmap ? (learned ? 10 : 8) + (tma_loads ? 1 : 0) : 2, [&] {
                 if (use_bitmap) {
-                    QW_TRY(launch_bm_list(view, nb, ix->l, st, tma_loads, s));
-                    QW_TRY(launch_bm_reduce(view, nb, ix->l, cap, ix->c, st,
-                                            (int)std::min<int64_t>(B, bm_reduce_wave(ix->nT)), s));
+                    const int slots = (int)std::min<int64_t>(B, bm_reduce_wave(ix->nT));
+                    QW_TRY(launch_bm_list(view, nb, ix->l, ix->c, st, tma_loads, slots, s));
+                    QW_TRY(launch_bm_reduce(view, nb, ix->l, cap, ix->c, st, slots, s));
                     if (learned) QW_TRY(launch_bm_recount(view, nb, ix->l, cap, ix->c, st, s));
                     return launch_bm_collect(view, nb, ix->l, cap, st, stats_b, want_cand, s);
                 }
@@ -1285,7 +1285,7 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
                                                late_list, ovf_count, s));
             if (use_bitmap && tm.on) {
                 int32_t h_rd = 0;
-                QW_CUDA_TRY(cudaMemcpyAsync(&h_rd, st.rd_ctl, sizeof(h_rd), cudaMemcpyDeviceToHost, s));
+                QW_CUDA_TRY(cudaMemcpyAsync(&h_rd, st.rd_ctl + 1, sizeof(h_rd), cudaMemcpyDeviceToHost, s));
                 QW_CUDA_TRY(cudaStreamSynchronize(s));
                 ix->prof.bitmap_overflows += h_rd;
             }

@@ -1342,32 +1342,40 @@ __device__ __forceinline__ uint4 rd_word(const QueryState &st, int L, int64_t qt
 }
 
 // Lists the last level's candidates of every query that has at most kQCap of
-// them: the counts of its groups with candidates once more from the bitmaps
+// them and no slot of the list rebuild below: the counts of its groups with candidates once more from the bitmaps
 // (few of the groups counted on the way there), and whether each was a candidate
 // of the previous level (its word there, if the query ran it).  A warp takes
-// four tiles of a query, as bm_count_kernel does.  Listing during the levels
+// four tiles of a query, as bm_count_kernel does; where there are no more than
+// kListQuads of those and the query has more than kListPart candidates (in the
+// locality order they lie in a few tiles), a quarter of their groups.  Listing during the levels
 // instead, every candidate of every level behind a returning atomic, took most
 // of the count pass where candidates are many (606 queries whose last level
 // takes in all 300,000 points: 2.3 ms of a level of 0.17).
-__global__ void __launch_bounds__(256, 3) bm_list_kernel(IndexView ix, int l, int nb, QueryState st)
+constexpr int kListPart = 2048;
+constexpr int64_t kListQuads = 65536;
+
+__global__ void __launch_bounds__(256, 3) bm_list_kernel(IndexView ix, int l, int nb, int parts,
+                                                          QueryState st)
 {
     __shared__ int s_nb[QW_MAX_M + 16];
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     const int m = ix.m, nT = ix.nT, mp = st.bm_mp;
     for (int i = threadIdx.x; i < mp; i += 256) s_nb[i] = i < m ? ix.bm_nb[i] : 0;
     __syncthreads();
-    const int64_t tasks = (int64_t)nb * ((nT + 3) >> 2);
+    const int64_t tasks = (int64_t)nb * ((nT + 3) >> 2) * parts;
     for (int64_t k = (int64_t)blockIdx.x * 8 + wi; k < tasks; k += (int64_t)gridDim.x * 8) {
-        const int q = (int)(k % nb), t0 = (int)(k / nb) * 4;
+        const int q = (int)(k % nb), t0 = (int)(k / nb / parts) * 4, part = (int)(k / nb % parts);
         const int L = st.levels[q] - 1;
         if (L < 0) continue;
         const int n = st.qbuf_n[(int64_t)(L & 1) * st.qbn_par + q];
-        if (n == 0 || n > kQCap) continue;
+        if (n == 0 || n > kQCap || (st.bm_ovf[q] & 8)) continue;
+        if (n <= kListPart && part) continue;  // few candidates: part 0 takes all
         const bool ran_prev = L > st.start[q];
-        const uint32_t x =
+        uint32_t x =
             t0 + (lane >> 3) < nT
                 ? st.bm_amask[((int64_t)(L & 1) * st.cln_par + (int64_t)q * nT + t0) * kSumWords + lane]
                 : 0u;
+        if (n > kListPart && parts > 1) x &= 0xffu << (8 * part);
         if (!__any_sync(0xffffffffu, x != 0)) continue;
         uint64_t *list = st.qbuf + (int64_t)q * kQCap;
         each_set_bit(x, lane, [&](int own, int bit, bool valid, bool four) {
@@ -1429,6 +1437,7 @@ __device__ __forceinline__ void smem_bitonic(uint64_t *keys, int n, int P2)
 // list rebuild below shortens its list and this selection runs again on it (a
 // query whose rebuilt list would still overflow goes to the level path).
 constexpr int SEL_THREADS = 256;
+constexpr int SEL_U = 4;  // list entries in flight per thread
 static_assert(kHistBins <= 256, "count histogram shares the radix histogram");
 
 __global__ void __launch_bounds__(SEL_THREADS) bm_select_kernel(IndexView ix, int l, int cap,
@@ -1463,16 +1472,25 @@ __global__ void __launch_bounds__(SEL_THREADS) bm_select_kernel(IndexView ix, in
     for (int c = threadIdx.x; c < kHistBins; c += SEL_THREADS) hist[c] = 0;
     __syncthreads();
     // counts of the candidates not of the previous level, and how many are
-    for (int j0 = 0; j0 < nl; j0 += SEL_THREADS) {
-        const int j = j0 + threadIdx.x;
-        const uint64_t e = j < nl ? E[j] : 0ull;
-        const bool pf = j < nl && ((e >> 8) & 1u);
-        const bool other = j < nl && !pf;
-        const uint32_t bp = __ballot_sync(0xffffffffu, pf);
-        if (lane == 0 && bp) atomicAdd(&s_np, __popc(bp));
-        const uint32_t bin = other ? 1u + (uint32_t)(e & 0xffu) : 1024u + lane;
-        const uint32_t peers = __match_any_sync(0xffffffffu, bin);
-        if (other && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], __popc(peers));
+    for (int j0 = 0; j0 < nl; j0 += SEL_THREADS * SEL_U) {
+        uint64_t e[SEL_U];
+#pragma unroll
+        for (int u = 0; u < SEL_U; ++u) {
+            const int j = j0 + u * SEL_THREADS + threadIdx.x;
+            e[u] = j < nl ? E[j] : 1ull << 9;  // bit 9: no entry
+        }
+        int n_pf = 0;
+#pragma unroll
+        for (int u = 0; u < SEL_U; ++u) {
+            if (j0 + u * SEL_THREADS >= nl) break;
+            const bool pf = (e[u] >> 8) & 1u;
+            const bool other = !((e[u] >> 8) & 3u);
+            n_pf += __popc(__ballot_sync(0xffffffffu, pf));
+            const uint32_t bin = other ? 1u + (uint32_t)(e[u] & 0xffu) : 1024u;
+            const uint32_t peers = __match_any_sync(0xffffffffu, bin);
+            if (other && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], __popc(peers));
+        }
+        if (lane == 0 && n_pf) atomicAdd(&s_np, n_pf);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1502,34 +1520,52 @@ __global__ void __launch_bounds__(SEL_THREADS) bm_select_kernel(IndexView ix, in
     // kept outright, and the tie class at c* (original ids); one slot
     // reservation per warp
     const int32_t *perm = ix.perm;
-    for (int j0 = 0; j0 < nl; j0 += SEL_THREADS) {
-        const int j = j0 + threadIdx.x;
-        const uint64_t e = j < nl ? E[j] : 0ull;
-        const int c = (int)(e & 0xffu);
-        const bool pf = (e >> 8) & 1u;
-        const bool kp = j < nl && (pf || c > cstar);
-        const bool ti = j < nl && !kp && c == cstar && take > 0;
-        const uint32_t bk = __ballot_sync(0xffffffffu, kp);
-        const uint32_t bt = __ballot_sync(0xffffffffu, ti);
+    for (int j0 = 0; j0 < nl; j0 += SEL_THREADS * SEL_U) {
+        uint64_t e[SEL_U];
+        int32_t orig[SEL_U];
+        uint32_t bk[SEL_U], bt[SEL_U];
+        int nK = 0, nT = 0;
+#pragma unroll
+        for (int u = 0; u < SEL_U; ++u) {
+            const int j = j0 + u * SEL_THREADS + threadIdx.x;
+            e[u] = j < nl ? E[j] : 1ull << 9;
+        }
+#pragma unroll
+        for (int u = 0; u < SEL_U; ++u) {
+            bk[u] = bt[u] = 0u;
+            if (j0 + u * SEL_THREADS >= nl) continue;
+            const int c = (int)(e[u] & 0xffu);
+            const bool in = !((e[u] >> 9) & 1u);
+            const bool kp = in && (((e[u] >> 8) & 1u) || c > cstar);
+            const bool ti = in && !kp && c == cstar && take > 0;
+            if (kp || ti) orig[u] = perm[e[u] >> 32];
+            bk[u] = __ballot_sync(0xffffffffu, kp);
+            bt[u] = __ballot_sync(0xffffffffu, ti);
+            nK += __popc(bk[u]);
+            nT += __popc(bt[u]);
+        }
         int baseK = 0, baseT = 0;
         if (lane == 0) {
-            if (bk) baseK = atomicAdd(&s_nd, __popc(bk));
-            if (bt) baseT = atomicAdd(&s_ne, __popc(bt));
+            if (nK) baseK = atomicAdd(&s_nd, nK);
+            if (nT) baseT = atomicAdd(&s_ne, nT);
         }
         baseK = __shfl_sync(0xffffffffu, baseK, 0);
         baseT = __shfl_sync(0xffffffffu, baseT, 0);
-        if (kp || ti) {
-            const int32_t orig = perm[e >> 32];
-            if (kp) {
-                const int d = baseK + __popc(bk & below);
+#pragma unroll
+        for (int u = 0; u < SEL_U; ++u) {
+            if (j0 + u * SEL_THREADS >= nl) break;
+            if ((bk[u] >> lane) & 1u) {
+                const int d = baseK + __popc(bk[u] & below);
                 if (d < cap) {
-                    cand[d] = orig;
-                    col[d] = c;
+                    cand[d] = orig[u];
+                    col[d] = (int)(e[u] & 0xffu);
                 }
-            } else {
-                const int t = baseT + __popc(bt & below);
-                if (t < kEqCap) eq[t] = orig;
+            } else if ((bt[u] >> lane) & 1u) {
+                const int t = baseT + __popc(bt[u] & below);
+                if (t < kEqCap) eq[t] = orig[u];
             }
+            baseK += __popc(bk[u]);
+            baseT += __popc(bt[u]);
         }
     }
     __syncthreads();
@@ -1627,15 +1663,19 @@ __global__ void __launch_bounds__(SEL_THREADS) bm_select_kernel(IndexView ix, in
 // ---- a last level that overflows the candidate list
 //
 // A query's list holds up to kQCap candidates.  When one doubling of the radius
-// sweeps whole clusters into a query's last level, that level can hold more.  Of
-// them the k + v bound keeps only the previous level's candidates, every
+// sweeps whole clusters into a query's last level, that level can hold more, or
+// so many that listing and selecting from them one by one costs more than counting
+// them twice: from kQDirect on (4,000 queries with 430 million
+// candidates, 325 of them with nearly every point: list, rebuild and selection
+// 2.39 ms with the line at 32,768, 2.44 at 16,384, 2.40 at 65,536, 2.57 without
+// it).  Of them the k + v bound keeps only the previous level's candidates, every
 // candidate whose count is above the boundary count c*, and the smallest
-// original ids of the tie class at c* (Section 3.1, readings R4/R5).  The kernels below rebuild the list of such
-// a query with only those entries, from the candidate words of its last level
+// original ids of the tie class at c* (Section 3.1, readings R4/R5).  The kernels
+// below rebuild the list of such a query with only those entries, from the candidate words of its last level
 // (still in place: a stopped query's tiles are not touched by later levels)
 // and the level bitmaps, each read once:
-//   rd_compact  lists the overflowing queries (slots) and their buckets;
-//   rd_count    one thread per 128-id group holding candidates: the counts
+//   rd_compact  lists the queries (slots) and their buckets;
+//   rd_count    one lane per 128-id group holding candidates: the counts
 //               from the m bitmap words of the last level, the previous
 //               level's candidate word (at a learned first level: their
 //               counts there, from that level's bitmaps), stored as seven bit
@@ -1654,10 +1694,12 @@ __global__ void __launch_bounds__(SEL_THREADS) bm_select_kernel(IndexView ix, in
 // result as from the whole list.  A query whose rebuilt list would still
 // overflow keeps the level-path answer, and so do the slots beyond one
 // store's worth (kRdStoreBytes).
-constexpr int kRdTieList = 4096;   // larger tie classes are cut by the original-id walk
+// candidates listed whole (more, if there is a slot: counted first); above any k + v
+constexpr int kQDirect = 32768;
+static_assert(kQDirect > QW_MAX_CAND, "a slot holds more candidates than are kept");
+constexpr int kRdTieList = kEqCap;  // larger tie classes are cut by the original-id walk
 constexpr int kRdStoreWords = 8;  // uint4 per group: 7 count planes, previous-level word
 constexpr int RD_THREADS = 256;
-static_assert(RD_THREADS == kBmUint4, "one block covers the groups of one tile");
 
 // Count planes of group g of tile t from the bitmaps of one level: bq[i] is
 // the bucket's bitmap in tile 0 (-1: no data), tile t adds t * bm_nb[i].
@@ -1691,120 +1733,155 @@ __device__ __forceinline__ uint32_t count_eq_planes(const Planes &P, int w, int 
     return eq;
 }
 
-__global__ void rd_compact_kernel(IndexView ix, int cgrow, QueryState st, int nb)
+// One warp per query: slots for the queries with more than `over` and at most
+// `upto` candidates, as long as the store has places for those that could also
+// be listed whole.  Marks them (bm_ovf flag 8).
+__global__ void rd_compact_kernel(IndexView ix, int cgrow, QueryState st, int nb, int over,
+                                  int upto, int wave)
 {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    const int q = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
     if (q >= nb) return;
     const int L = st.levels[q] - 1;
-    if (L < 0 || st.qbuf_n[(int64_t)(L & 1) * st.qbn_par + q] <= kQCap) return;
-    const int slot = atomicAdd(st.rd_ctl, 1);
-    RdPlan p;
-    memset(&p, 0, sizeof(p));
-    p.q = q;
-    p.mode = 1;
-    p.prev_recount = (L - 1 < st.start[q] && L > 0) ? 1 : 0;
-    st.rd_plan[slot] = p;
+    if (L < 0) return;
+    const int n = st.qbuf_n[(int64_t)(L & 1) * st.qbn_par + q];
+    if (n <= over || n > upto) return;
+    int slot = 0;
+    if (lane == 0) slot = atomicAdd(st.rd_ctl, 1);
+    slot = __shfl_sync(0xffffffffu, slot, 0);
+    if (n <= kQCap && slot >= wave) return;
+    if (lane == 0) {
+        if (n > kQCap) atomicAdd(st.rd_ctl + 1, 1);
+        st.bm_ovf[q] |= 8;
+        RdPlan p;
+        memset(&p, 0, sizeof(p));
+        p.q = q;
+        p.mode = 1;
+        p.prev_recount = (L - 1 < st.start[q] && L > 0) ? 1 : 0;
+        st.rd_plan[slot] = p;
+    }
     int32_t *h = st.rd_hist + (int64_t)slot * kHistBins;
-    for (int c = 0; c < kHistBins; ++c) h[c] = 0;
+    for (int c = lane; c < kHistBins; c += 32) h[c] = 0;
     const int64_t R = st.finalR[q];
-    int64_t *bq = st.rd_bq + (int64_t)slot * 2 * QW_MAX_M;
-    for (int i = 0; i < ix.m; ++i) {
+    int64_t *bq = st.rd_bq + (int64_t)slot * QW_MAX_M;
+    for (int i = lane; i < ix.m; i += 32) {
         const int64_t gi = st.g[(int64_t)q * ix.m + i];
-        bq[i] = bm_index(ix, i, 0, L, R, floordiv64(gi, R));
-        bq[QW_MAX_M + i] =
-            L > 0 ? bm_index(ix, i, 0, L - 1, R / cgrow, floordiv64(gi, R / cgrow)) : -1;
+        bq[i] = L > 0 ? bm_index(ix, i, 0, L - 1, R / cgrow, floordiv64(gi, R / cgrow)) : -1;
     }
 }
 
-// One block per (slot, tile) at a time, one thread per group.
-__global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, int l,
-                                                                  QueryState st, int s0,
-                                                                  int wave)
+// A warp takes a quarter of the groups with candidates of four tiles of a slot
+// (groups 8 p .. 8 p + 7 of every mask word), as bm_count_kernel takes live
+// groups.  (A thread per group of the index, few of which have candidates of a
+// query: 1,569 us against 1,453 for 1,760 slots of 1,000,000 points.)
+constexpr int kRdParts = 4;
+
+__device__ __forceinline__ uint32_t rd_task(const IndexView &ix, const QueryState &st, int64_t k,
+                                            int lane, int *slot, int *t0, int *q, int *L)
 {
-    __shared__ int sh_hist[kHistBins];
+    const int quads = (ix.nT + 3) >> 2;
+    const int part = (int)(k % kRdParts);
+    *t0 = (int)(k / kRdParts % quads) * 4;
+    *slot = (int)(k / kRdParts / quads);
+    *q = st.rd_plan[*slot].q;
+    *L = st.levels[*q] - 1;
+    const uint32_t x = *t0 + (lane >> 3) < ix.nT
+                           ? st.bm_amask[((int64_t)(*L & 1) * st.cln_par + (int64_t)*q * ix.nT +
+                                          *t0) * kSumWords + lane]
+                           : 0u;
+    return x & (0xffu << (8 * part));
+}
+
+__global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, int l,
+                                                                  QueryState st, int wave)
+{
+    __shared__ int sh_hist[RD_THREADS / 32][kHistBins];
     __shared__ int s_nb[QW_MAX_M + 16];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < st.bm_mp; i += RD_THREADS) s_nb[i] = i < ix.m ? ix.bm_nb[i] : 0;
+    for (int c = lane; c < kHistBins; c += 32) sh_hist[wi][c] = 0;
     __syncthreads();
-    const int nslot = min(st.rd_ctl[0] - s0, wave);
-    const int nT = ix.nT, g = threadIdx.x;
-    for (int64_t it = blockIdx.x; it < (int64_t)max(nslot, 0) * nT; it += gridDim.x) {
-        const int slot = s0 + (int)(it / nT), t = (int)(it % nT);
-        const RdPlan pl = st.rd_plan[slot];
-        const int q = pl.q, L = st.levels[q] - 1;
-        const int64_t qt = (int64_t)q * nT + t;
-        // tiles without candidates (block-uniform)
-        if (!__syncthreads_or(st.bm_amask[((int64_t)(L & 1) * st.cln_par + qt) * kSumWords +
-                                          (threadIdx.x & 7)] != 0))
-            continue;
-        for (int c = threadIdx.x; c < kHistBins; c += RD_THREADS) sh_hist[c] = 0;
-        __syncthreads();
-        const uint4 cw = rd_word(st, L, qt, g);
+    int *hist = sh_hist[wi];
+    const int nT = ix.nT;
+    const int64_t tasks = (int64_t)min(st.rd_ctl[0], wave) * ((nT + 3) >> 2) * kRdParts;
+    for (int64_t k = (int64_t)blockIdx.x * (RD_THREADS / 32) + wi; k < tasks;
+         k += (int64_t)gridDim.x * (RD_THREADS / 32)) {
+        int slot, t0, q, L;
+        const uint32_t x = rd_task(ix, st, k, lane, &slot, &t0, &q, &L);
+        if (!__any_sync(0xffffffffu, x != 0)) continue;
+        const bool recount = st.rd_plan[slot].prev_recount;
         int my_np = 0;
-        Planes P;
-        uint32_t oth[4] = {0, 0, 0, 0};  // candidates not of the previous level
-        int n_oth = 0;
-        if (cw.x | cw.y | cw.z | cw.w) {
-            const int64_t *bq = st.rd_bq + (int64_t)slot * 2 * QW_MAX_M;
+        each_set_bit(x, lane, [&](int own, int bit, bool valid, bool four) {
+            const int t = t0 + (own >> 3), g = (own & 7) * 32 + bit;
+            const int64_t qt = (int64_t)q * nT + t;
             uint4 pw = make_uint4(0, 0, 0, 0);
-            if (pl.prev_recount) {
-                rd_planes(ix, bq + QW_MAX_M, t, g, P);
+            Planes P;
+            if (recount) {
+                rd_planes(ix, st.rd_bq + (int64_t)slot * QW_MAX_M, t, g, P);
                 pw = candidates_of(P, l);
             } else if (L > 0) {
                 pw = rd_word(st, L - 1, qt, g);
             }
-            count_planes(ix, st.bm_b0 + (int64_t)q * st.bm_mp, s_nb, t, g, P);
-            uint4 *store = st.rd_store +
-                           ((int64_t)(slot - s0) * nT * kBmUint4 + (int64_t)t * kBmUint4 + g) *
-                               kRdStoreWords;
+            count_planes(ix, st.bm_b0 + (int64_t)q * st.bm_mp, s_nb, t, g, P, four);
+            const uint4 cw = candidates_of(P, l);
+            uint32_t oth[4] = {0, 0, 0, 0};  // candidates not of the previous level
+            int n_oth = 0;
+            if (valid) {
+                uint4 *store = st.rd_store +
+                               ((int64_t)slot * nT * kBmUint4 + (int64_t)t * kBmUint4 + g) *
+                                   kRdStoreWords;
 #pragma unroll
-            for (int k = 0; k < 7; ++k) store[k] = make_uint4(P.s[k][0], P.s[k][1], P.s[k][2], P.s[k][3]);
-            store[7] = pw;
+                for (int kk = 0; kk < 7; ++kk)
+                    store[kk] = make_uint4(P.s[kk][0], P.s[kk][1], P.s[kk][2], P.s[kk][3]);
+                store[7] = pw;
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                my_np += __popc(word_of(cw, w) & word_of(pw, w));
-                oth[w] = word_of(cw, w) & ~word_of(pw, w);
-                n_oth += __popc(oth[w]);
-            }
-        }
-        // the histogram of their counts: a warp with many of them compares the
-        // planes with every count (one addition per warp and count); adding one
-        // by one meets the same few shared words over and over
-        if (__reduce_add_sync(0xffffffffu, n_oth) > 256) {
-            for (int c = l; c <= ix.m; ++c) {
-                int here = 0;
-#pragma unroll
-                for (int w = 0; w < 4; ++w)
-                    if (oth[w]) here += __popc(count_eq_planes(P, w, c) & oth[w]);
-                here = __reduce_add_sync(0xffffffffu, here);
-                if ((threadIdx.x & 31) == 0 && here) atomicAdd(&sh_hist[c], here);
-            }
-        } else {
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                uint32_t x = oth[w];
-                while (x) {
-                    const int b = __ffs(x) - 1;
-                    x &= x - 1;
-                    atomicAdd(&sh_hist[count_of(P, w, b)], 1);
+                for (int w = 0; w < 4; ++w) {
+                    my_np += __popc(word_of(cw, w) & word_of(pw, w));
+                    oth[w] = word_of(cw, w) & ~word_of(pw, w);
+                    n_oth += __popc(oth[w]);
                 }
             }
-        }
+            // the histogram of their counts: a warp with many of them compares
+            // the planes with every count (one addition per warp and count);
+            // adding one by one meets the same few shared words over and over
+            if (__reduce_add_sync(0xffffffffu, n_oth) > 256) {
+                for (int c = l; c <= ix.m; ++c) {
+                    int here = 0;
+#pragma unroll
+                    for (int w = 0; w < 4; ++w)
+                        if (oth[w]) here += __popc(count_eq_planes(P, w, c) & oth[w]);
+                    here = __reduce_add_sync(0xffffffffu, here);
+                    if (lane == 0 && here) atomicAdd(&hist[c], here);
+                }
+            } else {
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    uint32_t left = oth[w];
+                    while (left) {
+                        const int b = __ffs(left) - 1;
+                        left &= left - 1;
+                        atomicAdd(&hist[count_of(P, w, b)], 1);
+                    }
+                }
+            }
+        });
         my_np = __reduce_add_sync(0xffffffffu, my_np);
-        if ((threadIdx.x & 31) == 0 && my_np) atomicAdd(&st.rd_plan[slot].np, my_np);
-        __syncthreads();
+        if (lane == 0 && my_np) atomicAdd(&st.rd_plan[slot].np, my_np);
+        __syncwarp();
         int32_t *h = st.rd_hist + (int64_t)slot * kHistBins;
-        for (int c = threadIdx.x; c < kHistBins; c += RD_THREADS)
-            if (sh_hist[c]) atomicAdd(h + c, sh_hist[c]);
-        __syncthreads();
+        for (int c = lane; c < kHistBins; c += 32)
+            if (hist[c]) {
+                atomicAdd(h + c, hist[c]);
+                hist[c] = 0;
+            }
+        __syncwarp();
     }
 }
 
-__global__ void rd_plan_kernel(int l, int m, int cap, int cgrow, QueryState st, int s0, int wave,
-                               int stage)
+__global__ void rd_plan_kernel(int l, int m, int cap, int cgrow, QueryState st, int wave, int stage)
 {
-    const int nslot = min(st.rd_ctl[0] - s0, wave);
-    const int slot = s0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (slot >= s0 + nslot) return;
+    const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= min(st.rd_ctl[0], wave)) return;
     RdPlan p = st.rd_plan[slot];
     const int q = p.q;
     const int L = st.levels[q] - 1;
@@ -1829,7 +1906,7 @@ __global__ void rd_plan_kernel(int l, int m, int cap, int cgrow, QueryState st, 
                 acc += h[c];
             }
             if (cstar < 0) {
-                p.mode = 0;  // cannot happen for a list that overflowed
+                p.mode = 0;  // cannot happen with more than k + v candidates
             } else {
                 p.cstar = cstar;
                 p.take = take;
@@ -1837,7 +1914,10 @@ __global__ void rd_plan_kernel(int l, int m, int cap, int cgrow, QueryState st, 
                 p.mode = h[cstar] <= kRdTieList ? 1 : 2;
             }
         }
-    } else if (p.mode != 0) {
+    } else if (p.mode == 0) {
+        // nothing was listed: the selection marks the query
+        st.qbuf_n[(int64_t)(L & 1) * st.qbn_par + q] = kQCap + 1;
+    } else {
         // the rebuilt list (more than kQCap entries: the level path answers)
         st.qbuf_n[(int64_t)(L & 1) * st.qbn_par + q] = p.pos;
         st.bm_ovf[q] |= 4;
@@ -1866,72 +1946,69 @@ __device__ __forceinline__ void rd_stored(const QueryState &st, int slot, int nT
     pw = store[7];
 }
 
-// The kept entries of every rebuilt slot, one thread per group: previous-level
-// candidates, counts above c*, and (a short tie class) the tie class.
-__global__ void __launch_bounds__(RD_THREADS, 3) rd_emit_kernel(IndexView ix, QueryState st,
+// The kept entries of every rebuilt slot, warps as in rd_count_kernel:
+// previous-level candidates, counts above c*, and (a short tie class) the tie
+// class.
+__global__ void __launch_bounds__(RD_THREADS, 3) rd_emit_kernel(IndexView ix, int l, QueryState st,
                                                                  int wave)
 {
-    const int nslot = min(st.rd_ctl[0], wave);
-    const int m = ix.m, nT = ix.nT, g = threadIdx.x;
-    for (int64_t it = blockIdx.x; it < (int64_t)nslot * nT; it += gridDim.x) {
-        const int slot = (int)(it / nT), t = (int)(it % nT);
-        const RdPlan pl = st.rd_plan[slot];
-        if (pl.mode == 0) continue;
-        const int q = pl.q, L = st.levels[q] - 1;
-        const int64_t qt = (int64_t)q * nT + t;
-        const uint4 cw = rd_word(st, L, qt, g);
-        if (!(cw.x | cw.y | cw.z | cw.w)) continue;
-        Planes P;
-        uint4 pw;
-        rd_stored(st, slot, nT, t, g, P, pw);
-        uint4 keep;
-        int my_n = 0;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            const uint32_t c_w = word_of(cw, w), p_w = word_of(pw, w);
-            const uint32_t oth = c_w & ~p_w;
-            uint32_t kw = (c_w & p_w) | (pl.cstar < m ? count_ge_planes(P, w, pl.cstar + 1) & oth : 0u);
-            if (pl.mode == 1) kw |= count_eq_planes(P, w, pl.cstar) & oth;
-            if (w == 0) keep.x = kw;
-            else if (w == 1) keep.y = kw;
-            else if (w == 2) keep.z = kw;
-            else keep.w = kw;
-            my_n += __popc(kw);
-        }
-        if (my_n) {
-            uint64_t *E = st.qbuf + (int64_t)q * kQCap;
-            int pos = atomicAdd(&st.rd_plan[slot].pos, my_n);
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int m = ix.m, nT = ix.nT;
+    const int64_t tasks = (int64_t)min(st.rd_ctl[0], wave) * ((nT + 3) >> 2) * kRdParts;
+    for (int64_t k = (int64_t)blockIdx.x * (RD_THREADS / 32) + wi; k < tasks;
+         k += (int64_t)gridDim.x * (RD_THREADS / 32)) {
+        int slot, t0, q, L;
+        const uint32_t x = rd_task(ix, st, k, lane, &slot, &t0, &q, &L);
+        if (!__any_sync(0xffffffffu, x != 0)) continue;
+        const int mode = st.rd_plan[slot].mode, cstar = st.rd_plan[slot].cstar;
+        if (mode == 0) continue;
+        uint64_t *E = st.qbuf + (int64_t)q * kQCap;
+        each_set_bit(x, lane, [&](int own, int bit, bool valid, bool) {
+            const int t = t0 + (own >> 3), g = (own & 7) * 32 + bit;
+            Planes P;
+            uint4 pw;
+            rd_stored(st, slot, nT, t, g, P, pw);
+            uint32_t kw[4];
+            int my_n = 0;
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
-                uint32_t x = word_of(keep, w);
-                const uint32_t p_w = word_of(pw, w);
-                while (x) {
-                    const int b = __ffs(x) - 1;
-                    x &= x - 1;
-                    const int64_t iid = (int64_t)t * kTile + (int64_t)g * 128 + w * 32 + b;
-                    if (pos < kQCap)
-                        E[pos] = ((uint64_t)iid << 32) | ((uint64_t)((p_w >> b) & 1u) << 8) |
-                                 (uint64_t)count_of(P, w, b);
-                    ++pos;
-                }
+                const uint32_t c_w = count_ge_planes(P, w, l), p_w = word_of(pw, w);
+                const uint32_t oth = c_w & ~p_w;
+                kw[w] = (c_w & p_w) | (cstar < m ? count_ge_planes(P, w, cstar + 1) & oth : 0u);
+                if (mode == 1) kw[w] |= count_eq_planes(P, w, cstar) & oth;
+                if (!valid) kw[w] = 0u;
+                my_n += __popc(kw[w]);
             }
-        }
+            int incl = my_n;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
+            }
+            int pos = 0;
+            if (lane == 31 && incl) pos = atomicAdd(&st.rd_plan[slot].pos, incl);
+            pos = __shfl_sync(0xffffffffu, pos, 31) + incl - my_n;
+            if (my_n)
+                append_candidates(P, make_uint4(kw[0], kw[1], kw[2], kw[3]), pw, E, pos,
+                                  (int64_t)t * kTile + (int64_t)g * 128);
+        });
     }
 }
 
 // One block per slot with a long tie class: data ids 0, 1, 2, ... are tested
-// kScanPer * 256 at a time (thread t takes ids o0 + u * 256 + t, so the loads
+// kScanPer * RS_THREADS at a time (thread t takes ids o0 + u * RS_THREADS + t, so the loads
 // of each u are coalesced and the kScanPer chains of dependent reads are in
 // flight together; tie member: a candidate of the last level, not of the
 // previous one, with count c*) until `take` members are found; those are the
 // take smallest original ids of the tie class (reading R5), listed with count
 // c*.  The walk reads about take * n / (tie class size) ids.
 constexpr int kScanPer = 4;
+constexpr int RS_THREADS = 1024;
 
-__global__ void __launch_bounds__(RD_THREADS) rd_scan_kernel(IndexView ix, QueryState st,
+__global__ void __launch_bounds__(RS_THREADS) rd_scan_kernel(IndexView ix, QueryState st,
                                                               int wave)
 {
-    constexpr int NW = RD_THREADS / 32;
+    constexpr int NW = RS_THREADS / 32;
     __shared__ int s_wc[kScanPer][NW];
     __shared__ int s_base;
     const int nslot = min(st.rd_ctl[0], wave);
@@ -1946,11 +2023,11 @@ __global__ void __launch_bounds__(RD_THREADS) rd_scan_kernel(IndexView ix, Query
         __syncthreads();
         const int base = s_base;
         int found = 0;
-        for (int64_t o0 = 0; o0 < ix.n && found < pl.take; o0 += RD_THREADS * kScanPer) {
+        for (int64_t o0 = 0; o0 < ix.n && found < pl.take; o0 += RS_THREADS * kScanPer) {
             int64_t iid[kScanPer];
 #pragma unroll
             for (int u = 0; u < kScanPer; ++u) {
-                const int64_t o = o0 + u * RD_THREADS + threadIdx.x;
+                const int64_t o = o0 + u * RS_THREADS + threadIdx.x;
                 iid[u] = o < ix.n ? (int64_t)ix.inv[o] : -1;
             }
             uint4 cw[kScanPer];
@@ -2380,8 +2457,8 @@ qw_status launch_bm_collect(const IndexView &ix, int nb, int l, int cap, QuerySt
     return QW_OK;
 }
 
-qw_status launch_bm_list(const IndexView &ix, int nb, int l, QueryState &st, bool staged,
-                         cudaStream_t s)
+qw_status launch_bm_list(const IndexView &ix, int nb, int l, int cgrow, QueryState &st,
+                         bool staged, int wave_slots, cudaStream_t s)
 {
     if (nb == 0) return QW_OK;
     if (staged) {
@@ -2390,9 +2467,18 @@ qw_status launch_bm_list(const IndexView &ix, int nb, int l, QueryState &st, boo
             ix, nb, st);
         QW_CUDA_TRY(cudaGetLastError());
     }
-    const int64_t tasks = (int64_t)nb * ((ix.nT + 3) / 4);
-    bm_list_kernel<<<(unsigned)std::min<int64_t>((tasks + 7) / 8, 152 * 24), 256, 0, s>>>(ix, l, nb,
-                                                                                        st);
+    // slots of the rebuild: the lists that would overflow and the long ones; where
+    // the store (wave_slots) has no place for every query, the former first
+    const unsigned qb = (unsigned)(((int64_t)nb * 32 + 127) / 128);
+    QW_CUDA_TRY(cudaMemsetAsync(st.rd_ctl, 0, 2 * sizeof(int32_t), s));
+    rd_compact_kernel<<<qb, 128, 0, s>>>(ix, cgrow, st, nb, nb <= wave_slots ? kQDirect : kQCap,
+                                         INT32_MAX, wave_slots);
+    if (nb > wave_slots)
+        rd_compact_kernel<<<qb, 128, 0, s>>>(ix, cgrow, st, nb, kQDirect, kQCap, wave_slots);
+    const int64_t quads = (int64_t)nb * ((ix.nT + 3) / 4);
+    const int parts = quads <= kListQuads ? 4 : 1;
+    bm_list_kernel<<<(unsigned)std::min<int64_t>((quads * parts + 7) / 8, 152 * 24), 256, 0, s>>>(
+        ix, l, nb, parts, st);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
 }
@@ -2406,19 +2492,15 @@ qw_status launch_bm_reduce(const IndexView &ix, int nb, int l, int cap, int cgro
                            QueryState &st, int wave_slots, cudaStream_t s)
 {
     if (nb == 0) return QW_OK;
-    QW_CUDA_TRY(cudaMemsetAsync(st.rd_ctl, 0, sizeof(int32_t), s));
-    const unsigned qb = (unsigned)((nb + 127) / 128);
-    rd_compact_kernel<<<qb, 128, 0, s>>>(ix, cgrow, st, nb);
-    QW_CUDA_TRY(cudaGetLastError());
     // one store's worth of slots (wave_slots); queries past it keep the
     // level-path answer
     const unsigned grid = 152 * 12;
     const unsigned pb = (unsigned)((wave_slots + 127) / 128);
-    rd_count_kernel<<<grid, RD_THREADS, 0, s>>>(ix, l, st, 0, wave_slots);
-    rd_plan_kernel<<<pb, 128, 0, s>>>(l, ix.m, cap, cgrow, st, 0, wave_slots, 0);
-    rd_scan_kernel<<<152 * 4, RD_THREADS, 0, s>>>(ix, st, wave_slots);
-    rd_emit_kernel<<<grid, RD_THREADS, 0, s>>>(ix, st, wave_slots);
-    rd_plan_kernel<<<pb, 128, 0, s>>>(l, ix.m, cap, cgrow, st, 0, wave_slots, 2);
+    rd_count_kernel<<<grid, RD_THREADS, 0, s>>>(ix, l, st, wave_slots);
+    rd_plan_kernel<<<pb, 128, 0, s>>>(l, ix.m, cap, cgrow, st, wave_slots, 0);
+    rd_scan_kernel<<<152 * 2, RS_THREADS, 0, s>>>(ix, st, wave_slots);
+    rd_emit_kernel<<<grid, RD_THREADS, 0, s>>>(ix, l, st, wave_slots);
+    rd_plan_kernel<<<pb, 128, 0, s>>>(l, ix.m, cap, cgrow, st, wave_slots, 2);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
 }

@@ -221,10 +221,10 @@ struct QueryState {
     int32_t *recount = nullptr;     // per query: stopped at its learned first level (bitmap path)
     // bitmap path, last levels whose candidates overflowed the list: the
     // number of such queries, per slot its plan and its count histogram
-    int32_t *rd_ctl = nullptr;      // [0]: slots
+    int32_t *rd_ctl = nullptr;      // [0]: slots, [1]: of them with more than kQCap
     struct RdPlan *rd_plan = nullptr;
     int32_t *rd_hist = nullptr;     // slots x kHistBins: counts of candidates not of C_{R/c}
-    int64_t *rd_bq = nullptr;       // slots x 2 x QW_MAX_M: bitmap numbers in tile 0 (L, L - 1)
+    int64_t *rd_bq = nullptr;       // slots x QW_MAX_M: bitmap numbers in tile 0 at L - 1
     uint4 *rd_store = nullptr;      // per slot of a wave, per group: 7 count planes + prev word
     // bitmap path, per (query, projection) of a level, rows of bm_mp entries (m
     // padded to 16): the bucket's bitmap number in tile 0 (-1: no data), its
@@ -308,8 +308,8 @@ qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int
                           const LoopCtl *ctl = nullptr, int part = 0, int tpw = 8);
 // After the level loop: the candidates of every query's last level to its list
 // (staged: the level ran bm_level_tma_kernel).
-qw_status launch_bm_list(const IndexView &ix, int nb, int l, QueryState &st, bool staged,
-                         cudaStream_t s);
+qw_status launch_bm_list(const IndexView &ix, int nb, int l, int cgrow, QueryState &st,
+                         bool staged, int wave_slots, cudaStream_t s);
 // Rebuild the candidate lists of the queries whose last level overflowed them
 // (kept entries and tie class only).
 qw_status launch_bm_reduce(const IndexView &ix, int nb, int l, int cap, int cgrow,

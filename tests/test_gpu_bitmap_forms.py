@@ -31,3 +31,30 @@ def test_count_forms(qwlib, cuda, n, nq, m, c, scale):
         for x, y in zip(got, want):
             assert torch.equal(x, y)
     index.free()
+
+
+@pytest.mark.parametrize("k,v", [(10, 500), (10, 4086)])
+@pytest.mark.parametrize("graph", [False, True])
+def test_long_lists(qwlib, cuda, k, v, graph):
+    """Last levels of a few to 100,000 candidates (listed whole, or counted first
+    and listed as far as they are kept), tie classes of a few ids and of
+    thousands."""
+    import torch
+    g = torch.Generator(device=cuda).manual_seed(7)
+    n, d, m = 100_000, 6, 12
+    size = torch.tensor([35_000, 33_000, 20_000, 9_000, 2_900, 100], device=cuda)
+    lab = torch.repeat_interleave(torch.arange(6, device=cuda), size)
+    lab = lab[torch.randperm(n, generator=g, device=cuda)]
+    centres = torch.randn((6, d), generator=g, device=cuda) * 30
+    X = (centres[lab] + torch.randn((n, d), generator=g, device=cuda) * 0.5).contiguous()
+    Q = X[torch.randint(0, n, (300,), generator=g, device=cuda)]
+    Q = (Q + torch.randn(Q.shape, generator=g, device=cuda) * 0.2).contiguous()
+    A = torch.randn((m, d), generator=g, device=cuda)
+    b = torch.rand((m,), generator=g, device=cuda)
+    index = qwlib.Index(X, A, b, w=1.0, c=2, v=v, l=9, bitmaps=True)
+    want = index.candidates(Q, k, path="levels")
+    assert (want[2][:, 2] > 32_768).any()
+    got = index.candidates(Q, k, path="bitmap", loads="direct", graph=graph)
+    for x, y in zip(got, want):
+        assert torch.equal(x, y)
+    index.free()
