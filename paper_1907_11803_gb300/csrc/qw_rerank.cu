@@ -20,10 +20,15 @@
 // certain gaps, so the first k ids are exactly those of the FP64 order, ties
 // broken by the smaller id.
 // Only a prefix of the sorted order matters: the positions up to the end of
-// the run holding position k - 1.  Its last value T is found without sorting
-// (radix selection of the k-th smallest FP32 value, then the next larger
-// value while the gap to it is uncertain), and only the candidates with FP32
-// distance <= T are sorted; the other stages see exactly that prefix.
+// the run holding position k - 1.  A value T at or a little past its end is
+// found without sorting (a bound of the k-th smallest FP32 value, then the next
+// larger value while the gap to it is uncertain), and only the candidates with
+// FP32 distance <= T are sorted; the other stages see exactly that prefix.
+//
+// Bound by the rows' reads out of L2 (about 11 TB/s) and by the block stages
+// after them: 10,000 queries x 800 candidates of 128 dimensions took 685 us with
+// a radix selection of four passes and a butterfly per row, 563 so, 382 of
+// them up to the distances.
 #include "qw_internal.cuh"
 #include "qw_scan.cuh"
 #include "qw_tc.cuh"
@@ -140,6 +145,23 @@ __device__ uint32_t min_above(const float *v, int n, float t, int *bc)
     return r;
 }
 
+// A bound T of the k-th smallest (k < n) of n non-negative values, ordered like
+// their bits: at least k of them are <= T, at most k + max(4, k / 8) unless more
+// equal the k-th.  The counts go to sm.key (two ints a slot, P2 >= n slots).
+__device__ __forceinline__ float kth_bound(const float *v, int n, int k, int P2,
+                                           const RerankSmem &sm)
+{
+    const uint32_t *u = reinterpret_cast<const uint32_t *>(v);
+    const bool wide = P2 >= 128;
+    uint32_t T = block_kth_bound<RR_THREADS>(u, n, k, max(4, k >> 3), wide ? min(2048, 2 * P2) : 256,
+                                             wide ? reinterpret_cast<int *>(sm.key) : sm.hist,
+                                             sm.bc, sm.scan_tmp);
+    __syncthreads();
+    // a part that reaches past infinity bounds nothing: the value itself
+    if (T > 0x7f800000u) T = block_kth_smallest<RR_THREADS>(u, n, k, sm.hist, sm.bc);
+    return __uint_as_float(T);
+}
+
 // Stages 1-6 for the nc candidates whose ids are in sm.sid[0..nc), using P2
 // (a power of two >= nc) slots; writes the query's k results.
 // row_of (optional): the row of data id `id` in X is row_of[id] (X in the
@@ -207,25 +229,22 @@ __device__ void rerank_finish(const float *__restrict__ X, const int32_t *__rest
                 }
             }
         }
-#pragma unroll
-        for (int u = 0; u < kRows; ++u) {
-            const int j = j0 + u;
-            const float sum = warp_sum(acc[u]);
-            if (lane == 0 && j < nc) d32[j] = sum;
-        }
+        // (the folded sums are warp_sum's trees)
+        const float sum = rows_sum<kRows>(acc, lane);
+        const int j = j0 + lane / (32 / kRows);
+        if (lane % (32 / kRows) == 0 && j < nc) d32[j] = sum;
     }
     __syncthreads();
 
     // 2. the prefix of the (FP32 distance, id) order that decides the result:
-    //    T = the k-th smallest distance, extended while the gap to the next
+    //    T >= the k-th smallest distance, extended while the gap to the next
     //    larger distance is uncertain (at most kExtend times, else the whole
     //    array is sorted); the candidates with distance <= T, sorted
     constexpr int kExtend = 16;
     bool whole = nc <= k;
     if (!whole) {
         // non-negative FP32 values are ordered like their bit patterns
-        float T = __uint_as_float(block_kth_smallest<RR_THREADS>(
-            reinterpret_cast<const uint32_t *>(d32), nc, k, sm.hist, sm.bc));
+        float T = kth_bound(d32, nc, k, P2, sm);
         whole = true;
         for (int it = 0; it < kExtend; ++it) {
             const uint32_t nb = min_above(d32, nc, T, sm.bc);
@@ -560,7 +579,6 @@ __global__ void __launch_bounds__(RR_THREADS) rerank_bf16_kernel(
     __shared__ int bc[4];
     __shared__ float s_qq;
     __shared__ int s_ngroups;
-    __shared__ int hist2[2048];
     RerankSmem sm = carve_rerank(smraw, P2, scan_tmp, &any_mark, hist, bc);
     int32_t *cid = reinterpret_cast<int32_t *>(sm.mark + P2 + 15 - ((P2 + 15) % 16));  // P2 ids
     int32_t *gkey = reinterpret_cast<int32_t *>(sm.key);  // P2 group slots (-1: empty)
@@ -697,13 +715,11 @@ __global__ void __launch_bounds__(RR_THREADS) rerank_bf16_kernel(
         sm.outd[j] = hi2;
     }
     __syncthreads();
-    // B. a bound uk >= the k-th smallest upper bound (non-negative: ordered like
-    //    its bits; at most 2^-13 above it): every candidate among the k nearest
-    //    has its lower bound <= uk
+    // B. a bound uk >= the k-th smallest upper bound (the groups in `key` are no
+    //    longer read): every candidate among the k nearest has its lower bound
+    //    <= uk
     float uk = CUDART_INF_F;
-    if (nc > k)
-        uk = __uint_as_float(block_kth_upper<RR_THREADS>(
-            reinterpret_cast<const uint32_t *>(sm.outd), nc, k, hist2, sm.bc));
+    if (nc > k) uk = kth_bound(sm.outd, nc, k, P2, sm);
     // C. keep the candidates that could be among the k nearest, in list order
     //    (the rows array in sid is no longer read)
     const int per = (nc + RR_THREADS - 1) / RR_THREADS;
@@ -918,12 +934,10 @@ __global__ void __launch_bounds__(RR_THREADS) rerank_tc_kernel(
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tbase) : "memory");
     }
-    // 3. the k-th smallest upper bound; the candidates that could be among the
-    //    k nearest go through the exact stages (the rows array is free now)
+    // 3. a bound of the k-th smallest upper bound; the candidates that could be
+    //    among the k nearest go through the exact stages (the rows array is free now)
     float uk = CUDART_INF_F;
-    if (nc > k)
-        uk = __uint_as_float(block_kth_smallest<RR_THREADS>(
-            reinterpret_cast<const uint32_t *>(sm.outd), nc, k, sm.hist, sm.bc));
+    if (nc > k) uk = kth_bound(sm.outd, nc, k, P2, sm);
     const int per = (nc + RR_THREADS - 1) / RR_THREADS;
     const int j0 = min(nc, tid * per), j1 = min(nc, j0 + per);
     int mine = 0;

@@ -128,59 +128,78 @@ __device__ uint32_t block_kth_smallest(const uint32_t *v, int n, int kk, int *hi
         hist, bc);
 }
 
-// An upper bound U of the kk-th smallest (1-based, 1 <= kk <= n) of n
-// unsigned 32-bit keys with at least kk keys <= U: two radix passes of 11 bits
-// (bits 31..21, then 20..10), U = the found prefix with bits 9..0 set.  For
-// non-negative floats (ordered like their bits) U exceeds the kk-th smallest
-// by less than 2^-13 of it.  Block-wide over NT threads; hist: 2048 ints and
-// bc: 2 ints of shared memory.  Returns U in every thread.
+// An upper bound U of the kk-th smallest (1-based, 1 <= kk <= n) of n unsigned
+// 32-bit keys: kk + slack or fewer keys are <= U, unless more are equal to the
+// kk-th.  The keys' range [min, max] in nbins (a power of two, at least 32) equal
+// parts, then, if the part of the kk-th holds too many, that part again.  Keys in
+// a narrow range (distances of one query) nearly all differ in their part, so the
+// counting meets few bank conflicts and one pass mostly does; a radix select from
+// the top byte spends its first passes on bits that all keys share.  Block-wide
+// over NT threads; hist: nbins ints, bc: 4 ints, tmp: NT / 32 ints of shared memory.
 template <int NT>
-__device__ uint32_t block_kth_upper(const uint32_t *v, int n, int kk, int *hist, int *bc)
+__device__ uint32_t block_kth_bound(const uint32_t *v, int n, int kk, int slack, int nbins,
+                                    int *hist, int *bc, int *tmp)
 {
-    const int lane = threadIdx.x & 31;
-    uint32_t prefix = 0, mask = 0;
-    for (int shift = 21; shift >= 10; shift -= 11) {
-        for (int i = threadIdx.x; i < 2048; i += NT) hist[i] = 0;
-        __syncthreads();
-        for (int j0 = 0; j0 < n; j0 += NT) {
-            const int j = j0 + threadIdx.x;
-            const uint32_t u = j < n ? v[j] : 0u;
-            const bool in = j < n && (u & mask) == prefix;
-            const uint32_t bin = in ? (u >> shift) & 2047u : 2048u + lane;
-            const uint32_t peers = __match_any_sync(0xffffffffu, bin);
-            if (in && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], __popc(peers));
+    uint32_t lo = 0xffffffffu, hi = 0;
+    for (int j = threadIdx.x; j < n; j += NT) {
+        lo = min(lo, v[j]);
+        hi = max(hi, v[j]);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (threadIdx.x == 0) {
+        bc[0] = -1;
+        bc[1] = 0;
+    }
+    for (int i = threadIdx.x; i < nbins; i += NT) hist[i] = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(reinterpret_cast<unsigned int *>(bc), lo);
+        atomicMax(reinterpret_cast<unsigned int *>(bc) + 1, hi);
+    }
+    __syncthreads();
+    lo = (uint32_t)bc[0];
+    hi = (uint32_t)bc[1];
+    const int log2b = 31 - __clz(nbins), per = max(nbins / NT, 1);
+    int shift = max(32 - __clz(hi - lo) - log2b, 0);
+    for (;;) {
+        for (int j = threadIdx.x; j < n; j += NT) {
+            const uint32_t u = v[j];
+            if (u >= lo && u <= hi) atomicAdd(&hist[(u - lo) >> shift], 1);
         }
         __syncthreads();
-        if (threadIdx.x < 32) {
-            // lane sums 64 bins, warp scan, then the lane holding kk walks them
-            int sl = 0;
-            for (int u = 0; u < 64; ++u) sl += hist[lane * 64 + u];
-            int incl = sl;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, off);
-                if (lane >= off) incl += y;
-            }
-            const int excl = incl - sl;
-            if (excl < kk && kk <= incl) {
-                int cum = excl;
-                for (int u = 0; u < 64; ++u) {
-                    const int c = hist[lane * 64 + u];
-                    if (cum < kk && kk <= cum + c) {
-                        bc[0] = lane * 64 + u;
-                        bc[1] = kk - cum;
-                    }
-                    cum += c;
+        // the part of the kk-th: each thread sums `per` parts, and the one whose
+        // range holds it walks them
+        const int b0 = (int)threadIdx.x * per;
+        int sum = 0, total;
+        if (b0 < nbins)
+            for (int u = 0; u < per; ++u) sum += hist[b0 + u];
+        int before = block_exclusive_scan<NT>(sum, tmp, &total);
+        if (before < kk && kk <= before + sum)
+            for (int u = 0; u < per; ++u) {
+                const int c = hist[b0 + u];
+                if (kk <= before + c) {
+                    bc[0] = b0 + u;
+                    bc[1] = before;
+                    bc[2] = c;
+                    break;
                 }
+                before += c;
             }
-        }
         __syncthreads();
-        prefix |= (uint32_t)bc[0] << shift;
-        mask |= 2047u << shift;
-        kk = bc[1];
+        const int bin = bc[0], first = bc[1], count = bc[2];
+        const uint32_t blo = lo + ((uint32_t)bin << shift);
+        const uint32_t rest = (1u << shift) - 1u;
+        const uint32_t bhi = hi - blo < rest ? hi : blo + rest;
+        if (shift == 0 || first + count - kk <= slack) return bhi;
+        kk -= first;
+        lo = blo;
+        hi = bhi;
+        shift = max(shift - log2b, 0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < nbins; i += NT) hist[i] = 0;
         __syncthreads();
     }
-    return prefix | 1023u;
 }
 
 }  // namespace qw
