@@ -1448,6 +1448,7 @@ __global__ void __launch_bounds__(SEL_THREADS) bm_select_kernel(IndexView ix, in
     extern __shared__ uint64_t keys[];
     __shared__ int hist[256];
     __shared__ int bc[4];
+    __shared__ int tmp[SEL_THREADS / 32];
     __shared__ int s_np, s_nd, s_ne, s_nt, s_cstar, s_take, s_keep;
     const int q = blockIdx.x;
     const int m = ix.m;
@@ -1611,8 +1612,9 @@ __global__ void __launch_bounds__(SEL_THREADS) bm_select_kernel(IndexView ix, in
     } else if (take > 0) {
         // the take smallest ids of the tie class: those <= its take-th smallest
         // (ids are distinct, so exactly take of them)
-        const uint32_t T = take < ne ? block_kth_smallest<SEL_THREADS>(
-                                           reinterpret_cast<const uint32_t *>(eq), ne, take, hist, bc)
+        const uint32_t T = take < ne ? block_kth_bound<SEL_THREADS>(
+                                           reinterpret_cast<const uint32_t *>(eq), ne, take, 0, 256,
+                                           hist, bc, tmp)
                                      : 0xffffffffu;
         for (int j0 = 0; j0 < ne; j0 += SEL_THREADS) {
             const int j = j0 + threadIdx.x;
@@ -2106,13 +2108,19 @@ __global__ void __launch_bounds__(RS_THREADS) rd_scan_kernel(IndexView ix, Query
 // with k + v.
 constexpr int RC_THREADS = 128;
 constexpr int kRcSplits = 8;
+constexpr int kRcPer = 8;  // candidates per thread of a piece
 constexpr int kRcChunks = (QW_MAX_M * 4 + 15) / 16;  // 16-byte pieces of the widest row
 
 // Ids of a 32-bit word within [lo, hi] (element-wise, inclusive).
 template <typename T> __device__ __forceinline__ int in_range(uint32_t h, uint32_t lo, uint32_t hi);
 template <> __device__ __forceinline__ int in_range<uint8_t>(uint32_t h, uint32_t lo, uint32_t hi)
 {
-    return __popc(__vcmpgeu4(h, lo) & __vcmpleu4(h, hi)) >> 3;
+    // a >= b per byte in its bit 7: the difference of the low bits borrows from
+    // bit 7 unless they are >=, and bit 7 itself decides where the two differ
+    const uint32_t top = 0x80808080u;
+    const uint32_t d0 = (h | top) - (lo & ~top), d1 = (hi | top) - (h & ~top);
+    const uint32_t ge = (h & ~lo) | (~(h ^ lo) & d0), le = (hi & ~h) | (~(hi ^ h) & d1);
+    return __popc(ge & le & top);
 }
 template <> __device__ __forceinline__ int in_range<uint16_t>(uint32_t h, uint32_t lo, uint32_t hi)
 {
@@ -2138,6 +2146,7 @@ __global__ void __launch_bounds__(RC_THREADS) bm_recount_kernel(IndexView ix, in
     const int n = st.qbuf_n[(int64_t)(L & 1) * st.qbn_par + q];
     uint64_t *E = st.qbuf + (int64_t)q * kQCap;
     if (n > kQCap) return;  // the selection marks the query for the level path
+    if (split > 0 && split * RC_THREADS * kRcPer >= n) return;
     if (R > st.top[q]) {
         // the plain path stops at level L - 1 by radius: not this answer
         if (threadIdx.x == 0 && split == 0) atomicOr(st.bm_ovf + q, 2);
@@ -2165,7 +2174,11 @@ __global__ void __launch_bounds__(RC_THREADS) bm_recount_kernel(IndexView ix, in
     __syncthreads();
     const char *H = static_cast<const char *>(ix.hloc);
     int mine = 0;
-    for (int j = split * RC_THREADS + threadIdx.x; j < n; j += nsplit * RC_THREADS) {
+    // the splits take pieces of kRcPer candidates per thread in turn
+    const int piece = RC_THREADS * kRcPer;
+    for (int i = threadIdx.x;; i += RC_THREADS) {
+        const int j = (i / piece * nsplit + split) * piece + i % piece;
+        if (j >= n) break;
         const uint64_t e = E[j];
         const uint4 *row = reinterpret_cast<const uint4 *>(H + (int64_t)(e >> 32) * ix.hloc_stride);
         int c = 0;

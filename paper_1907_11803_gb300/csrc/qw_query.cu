@@ -427,20 +427,21 @@ __global__ void decide_kernel(int nb, int level, int64_t R, int cap, QueryState 
         }
     }
     if (lane != 0) return;
-    if (st.level_passes) atomicAdd(st.level_passes, 1ull);
+    // all reads before the first write: one latency instead of one each
     if (!ss.prefix) sl = st.scan_level[q];
     const int32_t before = st.ncand[q];  // |C_R| of the previous level
     // |C_R| of this level (the bitmap path counts its list, the level path sums tiles)
     const int32_t nc = st.qbuf_n ? st.qbuf_n[(int64_t)(level & 1) * st.qbn_par + q] : st.cross[q];
+    const int64_t full = st.scan_full[q], top = st.top[q];
+    if (st.level_passes) atomicAdd(st.level_passes, 1ull);
     st.cross[q] = 0;
-    st.scan_full[q] += skipped;
     st.scan_level[q] = 0;
     st.scan_last[q] = sl;
-    st.scan_full[q] += sl;
+    st.scan_full[q] = full + skipped + sl;
     st.levels[q] = level + 1;
     st.finalR[q] = R;
     const bool enough = nc >= cap;        // the k + v bound (Section 3.1)
-    const bool past = R > st.top[q];      // no further level can change C_R
+    const bool past = R > top;            // no further level can change C_R
     if ((enough || past) && first && level > 0) {
         if (ss.recount_first) {
             // bitmap path: stop here; the previous level's candidates are
