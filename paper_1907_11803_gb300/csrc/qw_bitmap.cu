@@ -343,7 +343,7 @@ __device__ __forceinline__ bool dense_level(const IndexView &ix, const QueryStat
 // Buckets of projection i at a level (one past the last stored level).
 __device__ __forceinline__ int buckets_at(const IndexView &ix, int i, int level, int64_t R)
 {
-    return level > ix.bm_J[i] ? 1 : (int)((int64_t)ix.span[i] / R + 1);
+    return level > ix.bm_J[i] ? 1 : (int)(floordiv64(ix.span[i], R) + 1);
 }
 
 // 16-byte words of a group's table (odd: the groups start in different banks).
@@ -397,10 +397,16 @@ __global__ void __launch_bounds__(1024) bm_active_kernel(IndexView ix, int level
     int run = 0;
     for (int q0 = 0; q0 < nb; q0 += 1024 * E) {
         const int q1 = q0 + (int)threadIdx.x * E;
+        int act[E], first[E];  // all of a thread's loads in flight
+#pragma unroll
+        for (int u = 0; u < E; ++u) {
+            act[u] = q1 + u < nb ? st.active[q1 + u] : 0;
+            first[u] = q1 + u < nb ? st.start[q1 + u] : 0;
+        }
         uint32_t on = 0;
 #pragma unroll
         for (int u = 0; u < E; ++u)
-            if (q1 + u < nb && st.active[q1 + u] && level >= st.start[q1 + u]) on |= 1u << u;
+            if (act[u] && level >= first[u]) on |= 1u << u;
         int total;
         int at = run + block_exclusive_scan<1024>(__popc(on), tmp, &total);
 #pragma unroll
@@ -1772,29 +1778,31 @@ __global__ void rd_compact_kernel(IndexView ix, int cgrow, QueryState st, int nb
     }
 }
 
-// A warp takes a quarter of the groups with candidates of four tiles of a slot
-// (groups 8 p .. 8 p + 7 of every mask word), as bm_count_kernel takes live
-// groups.  (A thread per group of the index, few of which have candidates of a
-// query: 1,569 us against 1,453 for 1,760 slots of 1,000,000 points.)
-constexpr int kRdParts = 4;
+// A warp takes an eighth of the groups with candidates of four tiles of a slot
+// (groups 4 p .. 4 p + 3 of every mask word), as bm_count_kernel takes live
+// groups; the slots' tasks alternate, so that after the first of a slot most
+// counts are known to lie below its c* and stay out of the histogram.  4,000
+// queries, 1,000,000 points, 1,100 slots: 1,283 us in quarters, slot by slot and
+// with the whole histogram, 1,164 so; 262 slots with all of 3,000,000 points 986
+// and 935 us; 606 with all of 300,000 290 and 223.
+constexpr int kRdParts = 8;
 
 __device__ __forceinline__ uint32_t rd_task(const IndexView &ix, const QueryState &st, int64_t k,
-                                            int lane, int *slot, int *t0, int *q, int *L)
+                                            int nslot, int lane, int *slot, int *t0, int *q, int *L)
 {
-    const int quads = (ix.nT + 3) >> 2;
-    const int part = (int)(k % kRdParts);
-    *t0 = (int)(k / kRdParts % quads) * 4;
-    *slot = (int)(k / kRdParts / quads);
+    const int part = (int)(k / nslot % kRdParts);
+    *t0 = (int)(k / nslot / kRdParts) * 4;
+    *slot = (int)(k % nslot);
     *q = st.rd_plan[*slot].q;
     *L = st.levels[*q] - 1;
     const uint32_t x = *t0 + (lane >> 3) < ix.nT
                            ? st.bm_amask[((int64_t)(*L & 1) * st.cln_par + (int64_t)*q * ix.nT +
                                           *t0) * kSumWords + lane]
                            : 0u;
-    return x & (0xffu << (8 * part));
+    return x & (0xffffffffu >> (32 - 32 / kRdParts) << (32 / kRdParts * part));
 }
 
-__global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, int l,
+__global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, int l, int cap,
                                                                   QueryState st, int wave)
 {
     __shared__ int sh_hist[RD_THREADS / 32][kHistBins];
@@ -1805,13 +1813,15 @@ __global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, i
     __syncthreads();
     int *hist = sh_hist[wi];
     const int nT = ix.nT;
-    const int64_t tasks = (int64_t)min(st.rd_ctl[0], wave) * ((nT + 3) >> 2) * kRdParts;
+    const int nslot = min(st.rd_ctl[0], wave);
+    const int64_t tasks = (int64_t)nslot * ((nT + 3) >> 2) * kRdParts;
     for (int64_t k = (int64_t)blockIdx.x * (RD_THREADS / 32) + wi; k < tasks;
          k += (int64_t)gridDim.x * (RD_THREADS / 32)) {
         int slot, t0, q, L;
-        const uint32_t x = rd_task(ix, st, k, lane, &slot, &t0, &q, &L);
+        const uint32_t x = rd_task(ix, st, k, nslot, lane, &slot, &t0, &q, &L);
         if (!__any_sync(0xffffffffu, x != 0)) continue;
         const bool recount = st.rd_plan[slot].prev_recount;
+        const int floor = max(l, __ldcg(&st.rd_plan[slot].floor));
         int my_np = 0;
         each_set_bit(x, lane, [&](int own, int bit, bool valid, bool four) {
             const int t = t0 + (own >> 3), g = (own & 7) * 32 + bit;
@@ -1840,6 +1850,7 @@ __global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, i
                 for (int w = 0; w < 4; ++w) {
                     my_np += __popc(word_of(cw, w) & word_of(pw, w));
                     oth[w] = word_of(cw, w) & ~word_of(pw, w);
+                    if (floor > l) oth[w] &= count_ge_planes(P, w, floor);
                     n_oth += __popc(oth[w]);
                 }
             }
@@ -1847,7 +1858,7 @@ __global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, i
             // the planes with every count (one addition per warp and count);
             // adding one by one meets the same few shared words over and over
             if (__reduce_add_sync(0xffffffffu, n_oth) > 256) {
-                for (int c = l; c <= ix.m; ++c) {
+                for (int c = floor; c <= ix.m; ++c) {
                     int here = 0;
 #pragma unroll
                     for (int w = 0; w < 4; ++w)
@@ -1877,6 +1888,20 @@ __global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, i
                 hist[c] = 0;
             }
         __syncwarp();
+        // k + v or more of them with at least c so far: c* is no lower
+        int above = 0, c = 0;
+        for (int c0 = ix.m; c0 >= floor && c == 0; c0 -= 32) {
+            int incl = c0 - lane >= floor ? __ldcg(h + c0 - lane) : 0;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
+            }
+            const uint32_t full = __ballot_sync(0xffffffffu, above + incl >= cap);
+            if (full) c = c0 - (__ffs(full) - 1);
+            above += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0 && c > floor) atomicMax(&st.rd_plan[slot].floor, c);
     }
 }
 
@@ -1956,11 +1981,12 @@ __global__ void __launch_bounds__(RD_THREADS, 3) rd_emit_kernel(IndexView ix, in
 {
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     const int m = ix.m, nT = ix.nT;
-    const int64_t tasks = (int64_t)min(st.rd_ctl[0], wave) * ((nT + 3) >> 2) * kRdParts;
+    const int nslot = min(st.rd_ctl[0], wave);
+    const int64_t tasks = (int64_t)nslot * ((nT + 3) >> 2) * kRdParts;
     for (int64_t k = (int64_t)blockIdx.x * (RD_THREADS / 32) + wi; k < tasks;
          k += (int64_t)gridDim.x * (RD_THREADS / 32)) {
         int slot, t0, q, L;
-        const uint32_t x = rd_task(ix, st, k, lane, &slot, &t0, &q, &L);
+        const uint32_t x = rd_task(ix, st, k, nslot, lane, &slot, &t0, &q, &L);
         if (!__any_sync(0xffffffffu, x != 0)) continue;
         const int mode = st.rd_plan[slot].mode, cstar = st.rd_plan[slot].cstar;
         if (mode == 0) continue;
@@ -2509,7 +2535,7 @@ qw_status launch_bm_reduce(const IndexView &ix, int nb, int l, int cap, int cgro
     // level-path answer
     const unsigned grid = 152 * 12;
     const unsigned pb = (unsigned)((wave_slots + 127) / 128);
-    rd_count_kernel<<<grid, RD_THREADS, 0, s>>>(ix, l, st, wave_slots);
+    rd_count_kernel<<<grid, RD_THREADS, 0, s>>>(ix, l, cap, st, wave_slots);
     rd_plan_kernel<<<pb, 128, 0, s>>>(l, ix.m, cap, cgrow, st, wave_slots, 0);
     rd_scan_kernel<<<152 * 2, RS_THREADS, 0, s>>>(ix, st, wave_slots);
     rd_emit_kernel<<<grid, RD_THREADS, 0, s>>>(ix, l, st, wave_slots);

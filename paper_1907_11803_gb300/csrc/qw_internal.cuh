@@ -173,6 +173,7 @@ struct RdPlan {
     int32_t pos;    // entries of the rebuilt list
     int32_t prev_recount;  // learned first level: previous level from its bitmaps
     int32_t pad[8];
+    int32_t floor;      // c* is at least this (counts below are not in the histogram)
 };
 
 // Per-batch query state, all device arrays of length nb (or nb x m).

@@ -116,29 +116,80 @@ __device__ __forceinline__ float norm_bound(float sumsq, int d)
     return sqrtf(sumsq + (float)d * ((float)d * 1.4e-45f)) * 1.01f;
 }
 
-// Bucket id of entry (r, i) from its dot product as a pair and S >= sum_j
-// |a_j v_j| (W(a) W(v), whose weights are at least 1).  With L terms per lane every one of the 2 L additions to the low
-// part, and of the 6 of the lanes' sums, rounds a value of at most
-// u (L + 4) S: 2 (L + 4)^2 u^2 S in all; the FP64 definition is within
-// d 2^-53 S + 2^-51 |u| w of the real value, and so is u below.  Returns true
-// when the FP64 sequence had to decide.
-__device__ bool settle_entry(const HashArgs &h, int64_t r, int i, float2 t, double S)
+// Whether u, within rel S / w + 2^-50 |u| or so of the definition's value, may lie
+// in another bucket than that.
+__device__ __forceinline__ bool open_at(double u, double rel, double S, double w, int d)
 {
-    const double w = (double)h.w;
-    double u = __ddiv_rn(__dadd_rn(__dadd_rn((double)t.x, (double)t.y), (double)h.b[i]), w);
-    double f = floor(u);
-    const double L = (double)(h.d / 8 + 8);
-    const double rel = 2.0 * L * L * 3.552713678800501e-15 + (double)h.d * 1.1102230246251565e-16;
-    const double E = 1.05 * (rel * S + (double)h.d * 1e-44) / w + fabs(u) * 8.9e-16;
-    const double frac = u - f;
-    const bool exact = !(fmin(frac, 1.0 - frac) > E);
-    if (exact) {
-        const float *vr = h.V + r * (int64_t)h.d, *ar = h.A + (int64_t)i * h.d;
-        double s = 0.0;
-        for (int j = 0; j < h.d; ++j) s = __dadd_rn(s, __dmul_rn((double)ar[j], (double)vr[j]));
-        u = __ddiv_rn(__dadd_rn(s, (double)h.b[i]), w);
-        f = floor(u);
+    const double E = 1.05 * (rel * S + (double)d * 1e-44) / w + fabs(u) * 8.9e-16;
+    const double frac = u - floor(u);
+    return !(fmin(frac, 1.0 - frac) > E);
+}
+
+// (v . a + bias) / w of each open lane's rows v and a, as far as its bucket needs
+// it (see settle_entry; apart from it so that its registers are not the callers').
+__device__ __noinline__ double open_value(const float *v, const float *a, int d, double bias,
+                                          double w, double S, bool open)
+{
+    const int lane = threadIdx.x & 31;
+    double u = 0.0;
+    uint32_t mask = __ballot_sync(0xffffffffu, open);
+    if (__popc(mask) <= 8) {
+        for (; mask; mask &= mask - 1) {
+            const int src = __ffs(mask) - 1;
+            const float *vr = reinterpret_cast<const float *>(
+                __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(v), src));
+            const float *ar = reinterpret_cast<const float *>(
+                __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(a), src));
+            double s = 0.0;
+#pragma unroll 4
+            for (int j = lane; j < d; j += 32) s = fma((double)__ldg(ar + j), (double)__ldg(vr + j), s);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1)
+                s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, off));
+            if (lane == src) {
+                u = __ddiv_rn(__dadd_rn(s, bias), w);
+                open = open_at(u, (double)(d + d / 32 + 8) * 1.1102230246251565e-16, S, w, d);
+            }
+        }
     }
+    if (open) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int j = 0; j < d; ++j)
+            s = __dadd_rn(s, __dmul_rn((double)__ldg(a + j), (double)__ldg(v + j)));
+        u = __ddiv_rn(__dadd_rn(s, bias), w);
+    }
+    return u;
+}
+
+// Bucket id of each lane's entry (r, i) from its dot product as a pair and S >=
+// sum_j |a_j v_j| (W(a) W(v), whose weights are at least 1); every lane of the
+// warp calls it, those without an entry with valid = false.  With L terms per lane
+// every one of the 2 L additions to the low part, and of the 6 of the lanes' sums,
+// rounds a value of at most u (L + 4) S: 2 (L + 4)^2 u^2 S in all; the FP64
+// definition is within d 2^-53 S + 2^-51 |u| w of the real value, and so is u
+// below.  An entry that this leaves open is summed in FP64 by the warp (d / 32
+// fused steps per lane and five sums: (d / 32 + 8) 2^-53 S), and only one that is
+// open then takes the definition's own sequence, d dependent additions (67 us at
+// d = 512).  At d = 512 one entry in 50,000 is open after the pairs, so a call met
+// the sequence in some block: 2,000 rows x 64 took 107 us, 40
+// so.  Where more than eight lanes are open they take the sequence side by side
+// at once.  Returns true when the pair did not decide.
+__device__ __forceinline__ bool settle_entry(const HashArgs &h, int64_t r, int i, float2 t,
+                                             double S, bool valid)
+{
+    const double w = (double)h.w, bias = valid ? (double)h.b[i] : 0.0;
+    double u = __ddiv_rn(__dadd_rn(__dadd_rn((double)t.x, (double)t.y), bias), w);
+    const double L = (double)(h.d / 8 + 8);
+    const bool open = valid && open_at(u, 2.0 * L * L * 3.552713678800501e-15 +
+                                              (double)h.d * 1.1102230246251565e-16, S, w, h.d);
+    if (__any_sync(0xffffffffu, open)) {
+        const double x = open_value(h.V + r * (int64_t)h.d, h.A + (int64_t)i * h.d, h.d, bias, w,
+                                    S, open);
+        if (open) u = x;
+    }
+    if (!valid) return false;
+    const double f = floor(u);
     int32_t *hp = h.H + r * h.ld_row + (int64_t)i * h.ld_col;
     if (!(f >= -2147483647.0 && f <= 2147483646.0)) {
         atomicOr(h.err, 2);
@@ -146,7 +197,7 @@ __device__ bool settle_entry(const HashArgs &h, int64_t r, int i, float2 t, doub
     } else {
         *hp = (int32_t)f;
     }
-    return exact;
+    return open;
 }
 
 // Pass 2 of a block: its `count` listed entries (local row << 7 | local
@@ -167,10 +218,11 @@ __device__ void settle_listed(const HashArgs &h, const uint16_t *list, int count
             if (valid && lane8 == 0) sums[s] = t;
         }
         __syncthreads();
-        if ((int)threadIdx.x < nn) {
-            const int e = list[base + threadIdx.x];
-            const double S = (double)vn[e >> 7] * (double)an[e & 127];
-            settle_entry(h, row0 + (e >> 7), col0 + (e & 127), sums[threadIdx.x], S);
+        if ((int)(threadIdx.x & ~31u) < nn) {  // whole warps
+            const bool valid = (int)threadIdx.x < nn;
+            const int e = list[base + (valid ? (int)threadIdx.x : 0)];
+            settle_entry(h, row0 + (e >> 7), col0 + (e & 127), sums[valid ? threadIdx.x : 0],
+                         (double)vn[e >> 7] * (double)an[e & 127], valid);
         }
         __syncthreads();
     }
@@ -203,10 +255,8 @@ __global__ void __launch_bounds__(NT) project_rows_kernel(HashArgs h)
         sv += __shfl_xor_sync(0xffffffffu, sv, off);
         sa += __shfl_xor_sync(0xffffffffu, sa, off);
     }
-    if (valid && lane8 == 0) {
-        const double S = (double)norm_bound(sv, h.d) * (double)norm_bound(sa, h.d);
-        if (settle_entry(h, r, i, t, S) && h.fixups) atomicAdd(h.fixups, 1ull);
-    }
+    const double S = (double)norm_bound(sv, h.d) * (double)norm_bound(sa, h.d);
+    if (settle_entry(h, r, i, t, S, valid && lane8 == 0) && h.fixups) atomicAdd(h.fixups, 1ull);
 }
 
 // A (32 TM) x (8 TN) tile of entries per block, TM x TN per thread, the operands

@@ -29,3 +29,20 @@ def test_hash_tile_edges(orc, qwlib, cuda, n, d, m, tc):
     H, fix = qwlib.hash(*(torch.from_numpy(x).to(cuda) for x in (X, A, b)), 4.0, tensor_cores=tc)
     assert np.array_equal(H.cpu().numpy(), want)
     assert 0 <= fix <= want.size
+
+
+@pytest.mark.parametrize("rows", [[0], [3, 40, 41], list(range(70))])
+@pytest.mark.parametrize("n,d", [(70, 512), (70, 33), (300, 513)])
+def test_entries_on_an_edge(orc, qwlib, cuda, n, d, rows):
+    """Rows of integers whose projections fall exactly on a bucket's edge (summed
+    in FP64 by a warp, or side by side, and then in the definition's order), among
+    rows that the first sums decide."""
+    import torch
+    rng = np.random.default_rng(d)
+    m = 9
+    V = rng.standard_normal((n, d)).astype(np.float32)
+    V[rows] = rng.integers(-3, 4, size=(len(rows), d))
+    A = rng.integers(-2, 3, size=(m, d)).astype(np.float32)
+    b = np.zeros(m, np.float32)
+    got, _ = qwlib.hash(*(torch.from_numpy(x).to(cuda) for x in (V, A, b)), 1.0)
+    assert np.array_equal(got.cpu().numpy(), orc.hash(V, A, b, 1.0))
