@@ -469,7 +469,8 @@ __device__ __forceinline__ void add8_word(uint32_t (&p)[7], const uint32_t (&x)[
 // the compare gives the word's live groups.  Issue bound: about 6.5
 // instructions per projection and four tiles.  (One warp per tile with a bit
 // transpose of every word, for each group's own list of projections, issued
-// about 30: 2,638 us per call on 3 million points and 10,000 queries, 584 so.)
+// about 30: 2,638 us per call on 3 million points and 10,000 queries; 584 so with
+// the reads of 16 projections in flight, 545 with 32.)
 __global__ void __launch_bounds__(FL_WARPS * 32) bm_filter_kernel(IndexView ix, int level, int l,
                                                                   QueryState st, const LoopCtl *ctl)
 {
@@ -490,7 +491,7 @@ __global__ void __launch_bounds__(FL_WARPS * 32) bm_filter_kernel(IndexView ix, 
         const int4 *rows = reinterpret_cast<const int4 *>(st.bm_srow + (int64_t)q * mp);
         const uint32_t *sum = ix.bm_sum + (int64_t)t0 * kSumWords + in_row;
         uint32_t P[7] = {0, 0, 0, 0, 0, 0, 0};
-#pragma unroll 2
+#pragma unroll 4
         for (int i = 0; i < mp; i += 8) {
             const int4 ra = __ldg(rows + (i >> 2)), rb = __ldg(rows + (i >> 2) + 1);
             const int32_t r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
