@@ -394,8 +394,13 @@ __device__ __forceinline__ RerankSmem carve_rerank(unsigned char *base, int P2, 
     return r;
 }
 
-template <int kRows>
-__global__ void __launch_bounds__(RR_THREADS) rerank_kernel(
+// kBlocks: blocks per SM that the registers leave room for.  Rows of up to 128
+// coordinates are one read per lane, and many warps hide it best (0: the compiler
+// takes 40 registers); longer rows want registers for a row's next reads (4: 64).
+// 10,000 queries x 800 rows of 128: 563 us with 0, 651 with 4; 4,000 x 4,096 of
+// 256: 4,631 and 2,579; 2,000 x 1,050 of 512: 838 and 655.
+template <int kRows, int kBlocks>
+__global__ void __launch_bounds__(RR_THREADS, kBlocks) rerank_kernel(
     const float *__restrict__ X, const int32_t *__restrict__ row_of, int d,
     const float *__restrict__ Qb, int k, int cap, int P2,
     const int32_t *__restrict__ cand, const int32_t *__restrict__ nkeep,
@@ -1045,15 +1050,21 @@ qw_status launch_rerank(const IndexView &ix, const float *Qb, int nb, int k, int
     int P2 = 2;
     while (P2 < cap) P2 <<= 1;
     const size_t smem = (size_t)P2 * (sizeof(double) + 2 * sizeof(float) + sizeof(int32_t) + 1);
-    const void *fn = rows == 2 ? (const void *)rerank_kernel<2>
-                     : rows == 8 ? (const void *)rerank_kernel<8> : (const void *)rerank_kernel<4>;
-    QW_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // 16-byte row loads need d % 4 == 0 and 16-byte aligned bases
     const bool vec = (ix.d % 4 == 0) && ((uintptr_t)Qb % 16 == 0) && ((uintptr_t)X % 16 == 0);
-    QW_RERANK_ROWS_DISPATCH(rows, rerank_kernel, <<<nb, RR_THREADS, smem, s>>>(
-        X, row_of, ix.d, Qb, k, cap, P2, st.cand, st.nkeep, ids_out, dists_out, vec))
-    QW_CUDA_TRY(cudaGetLastError());
-    return QW_OK;
+    auto launch = [&](auto kernel) -> qw_status {
+        QW_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem));
+        kernel<<<nb, RR_THREADS, smem, s>>>(X, row_of, ix.d, Qb, k, cap, P2, st.cand, st.nkeep,
+                                            ids_out, dists_out, vec);
+        QW_CUDA_TRY(cudaGetLastError());
+        return QW_OK;
+    };
+    if (ix.d > 128)
+        return rows == 2 ? launch(rerank_kernel<2, 4>)
+             : rows == 8 ? launch(rerank_kernel<8, 4>) : launch(rerank_kernel<4, 4>);
+    return rows == 2 ? launch(rerank_kernel<2, 0>)
+         : rows == 8 ? launch(rerank_kernel<8, 0>) : launch(rerank_kernel<4, 0>);
 }
 
 }  // namespace qw
