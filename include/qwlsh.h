@@ -317,7 +317,7 @@ typedef struct {
     int32_t tile;          /* ids per index tile (entries are grouped by id / tile) */
     int32_t n_tiles;
     int32_t span_max;      /* largest anchored bucket id over all projections */
-    int64_t n_fixups;      /* data projections recomputed in FP64 at build time */
+    int64_t n_fixups;      /* data projections near an edge, summed again at build time */
     int64_t device_bytes;  /* device memory held by the index (excluding workspace) */
     int64_t bitmap_bytes;  /* the level bitmaps (0 without them), in device memory unless
                               host_bitmaps */
