@@ -410,17 +410,14 @@ qw_status launch_tile_sort(const int32_t *Ht, int64_t n, int m, int nT, const in
 {
     if (span_max < kCountBids) {
         const int nb = span_max + 1;
-        const size_t smem = count_sort_smem(nb);
-        QW_CUDA_TRY(cudaFuncSetAttribute(tile_count_sort_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        tile_count_sort_kernel<<<dim3((unsigned)nT, (unsigned)m), SORT_THREADS, smem, s>>>(
-            Ht, n, o, lid, dir_bid, dir_off, dir_start, dir_cnt, nT, nb);
+        QW_TRY(allow_smem(tile_count_sort_kernel, count_sort_smem(kCountBids)));
+        tile_count_sort_kernel<<<dim3((unsigned)nT, (unsigned)m), SORT_THREADS, count_sort_smem(nb),
+                                 s>>>(Ht, n, o, lid, dir_bid, dir_off, dir_start, dir_cnt, nT, nb);
         QW_CUDA_TRY(cudaGetLastError());
         return QW_OK;
     }
     const size_t smem = (size_t)kTile * (sizeof(int32_t) + sizeof(uint16_t) + sizeof(uint8_t));
-    QW_CUDA_TRY(cudaFuncSetAttribute(tile_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+    QW_TRY(allow_smem(tile_sort_kernel, smem));
     tile_sort_kernel<<<dim3((unsigned)nT, (unsigned)m), SORT_THREADS, smem, s>>>(
         Ht, n, o, lid, dir_bid, dir_off, dir_start, dir_cnt, nT);
     QW_CUDA_TRY(cudaGetLastError());

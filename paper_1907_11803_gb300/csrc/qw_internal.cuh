@@ -55,6 +55,18 @@ struct DevBuf {
     template <class T> T *as() const { return reinterpret_cast<T *>(p); }
 };
 
+// Allow launches of `kernel` `most` bytes of dynamic shared memory: the most that
+// any launch of it asks for.  The limit belongs to the function and not to a
+// launch, so a call that set it to its own size could find a smaller one set by
+// another thread's call between here and its launch, which would then fail.
+template <class K>
+inline qw_status allow_smem(K *kernel, size_t most)
+{
+    QW_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)most));
+    return QW_OK;
+}
+
 // ---------------------------------------------------------------- projection
 // H[r * ld_row + i * ld_col] = floor((a_i . V_r + b_i) / w), FP32 with a
 // recomputation (pairs of floats, then FP64) of every entry near a bucket
