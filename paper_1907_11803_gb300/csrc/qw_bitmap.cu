@@ -2421,8 +2421,7 @@ qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int
         // fewer queries than the dense form asks of an average group never take it
         if (nb >= kDenseMin) {
             const size_t smem = dense_smem_bytes();
-            QW_CUDA_TRY(cudaFuncSetAttribute(
-                bm_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            QW_TRY(allow_smem(bm_dense_kernel, smem));
             bm_dense_kernel<<<2 * 152, DN_THREADS, smem, s>>>(ix, level, R, l, st, ctl);
             QW_CUDA_TRY(cudaGetLastError());
         }
@@ -2432,8 +2431,7 @@ qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int
     QW_CUDA_TRY(cudaGetDevice(&dev));
     QW_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
     const size_t smem = tma_smem_bytes();
-    QW_CUDA_TRY(cudaFuncSetAttribute(bm_level_tma_kernel,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QW_TRY(allow_smem(bm_level_tma_kernel, smem));
     const int64_t items = (int64_t)nb * ix.nT;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(n_sm, items));
     bm_level_tma_kernel<<<grid, TMA_THREADS, smem, s>>>(ix, level, R, l, nb, st, ctl, err);
@@ -2489,9 +2487,9 @@ qw_status launch_bm_collect(const IndexView &ix, int nb, int l, int cap, QuerySt
 {
     int P2 = 2;
     while (P2 < cap) P2 <<= 1;
+    // (within the 48 KiB that every launch may have)
+    static_assert(QW_MAX_CAND * sizeof(uint64_t) + 2048 <= 48 << 10, "keys and the block's counts");
     const size_t smem = sorted ? (size_t)P2 * sizeof(uint64_t) : 0;
-    QW_CUDA_TRY(cudaFuncSetAttribute(bm_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
     bm_select_kernel<<<nb, SEL_THREADS, smem, s>>>(ix, l, cap, st, stats_out, sorted);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;

@@ -74,6 +74,10 @@ __host__ __device__ inline size_t cluster_smem_bytes(int tpc, int m)
            3 * nseg + 16;
 }
 
+// Dynamic shared memory that every launch may have: what a block's static part
+// leaves (five tiles take at most 207 KiB, six never fit).
+constexpr size_t kClusterSmem = kMaxBlockSmem - sizeof(ClusterShared) - 1024;
+
 __global__ void __launch_bounds__(CQ_THREADS, 2) cluster_query_kernel(
     IndexView ix, const int32_t *__restrict__ HQ, int nq, int l, int cgrow, int cap, int tpc,
     QueryState st, int *__restrict__ queue, int64_t *__restrict__ stats_out, int *__restrict__ err)
@@ -490,9 +494,11 @@ static cudaLaunchConfig_t cluster_config(int cluster_size, int tpc, int m, cudaS
 // the shape cannot be launched).
 static int cluster_capacity(int cluster_size, int tpc, int m)
 {
-    const int smem = (int)cluster_smem_bytes(tpc, m);
+    // (an index's own size as the limit could be lowered by another thread's call
+    // before the launch)
+    if (cluster_smem_bytes(tpc, m) > kClusterSmem) return 0;
     if (cudaFuncSetAttribute(cluster_query_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem) != cudaSuccess) {
+                             (int)kClusterSmem) != cudaSuccess) {
         (void)cudaGetLastError();
         return 0;
     }

@@ -66,6 +66,8 @@ inline qw_status allow_smem(K *kernel, size_t most)
                                      (int)most));
     return QW_OK;
 }
+// What a block may have in all, static and dynamic (sm_103a).
+constexpr size_t kMaxBlockSmem = (size_t)227 << 10;
 
 // ---------------------------------------------------------------- projection
 // H[r * ld_row + i * ld_col] = floor((a_i . V_r + b_i) / w), FP32 with a

@@ -996,10 +996,12 @@ static qw_status launch_mlp_tc(qw_mlp *mp, const float *X, const float *Q, const
     if (n == 0) return QW_OK;
     const int K0 = mp->n_in, Ka = std::max(K0, mp->H);
     // at least 120 KiB, so one CTA per SM: each holds all 512 TMEM columns
-    const size_t smem = std::max<size_t>((size_t)TC_ROWS * Ka * 2 + (size_t)TC_MAXN * TC_KC * 2,
-                                         (size_t)120 << 10);
-    QW_CUDA_TRY(cudaFuncSetAttribute(mlp_forward_tc_kernel,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    auto smem_of = [](int K) {
+        return std::max<size_t>((size_t)TC_ROWS * K * 2 + (size_t)TC_MAXN * TC_KC * 2,
+                                (size_t)120 << 10);
+    };
+    const size_t smem = smem_of(Ka);
+    QW_TRY(allow_smem(mlp_forward_tc_kernel, smem_of(TC_MAXK)));
     const __half *h = mp->p16.as<__half>();
     const float *p = mp->p32.as<float>();
     // rows per CTA: enough CTAs for every SM (one CTA per SM), 16 to 128
@@ -1036,8 +1038,7 @@ qw_status launch_start_model(qw_mlp *mp, const float *Q, const int32_t *HQ, int 
         mp->t_version = mp->version;
     }
     const size_t smem = (size_t)SM_RB * ((size_t)nin + 2 * (size_t)H + (size_t)C) * sizeof(float);
-    QW_CUDA_TRY(cudaFuncSetAttribute(start_model_kernel,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QW_TRY(allow_smem(start_model_kernel, kMaxBlockSmem));  // (no static shared memory)
     const __half *t = mp->p16t.as<__half>();
     const float *p = mp->p32.as<float>();
     start_model_kernel<<<(nq + SM_RB - 1) / SM_RB, SM_THREADS, smem, s>>>(

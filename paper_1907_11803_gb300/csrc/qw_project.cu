@@ -687,13 +687,12 @@ qw_status launch_hash(const float *V, int64_t nv, int d, const float *A, const f
         while (ncols < (uint32_t)(3 * N)) ncols <<= 1;
         // shared memory sized so that the CTAs resident on an SM never ask
         // for more than its 512 TMEM columns (no allocation waits)
-        const size_t per = (size_t)(2 * PT_ROWS + 2 * 128) * PT_KC * 2;
-        static_assert((size_t)(2 * PT_ROWS + 2 * 128) * PT_KC * 2 >=
-                          PT_ROWS * 128 * sizeof(uint16_t) + PT_ROWS * sizeof(float2),
+        constexpr size_t per = (size_t)(2 * PT_ROWS + 2 * 128) * PT_KC * 2;
+        static_assert(per >= PT_ROWS * 128 * sizeof(uint16_t) + PT_ROWS * sizeof(float2),
                       "the list of open entries fits the operand tiles");
-        const size_t smem = std::max<size_t>(per, ncols > 256 ? (size_t)120 << 10 : (size_t)80 << 10);
-        QW_CUDA_TRY(cudaFuncSetAttribute(project_tc_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        static_assert(per <= (size_t)80 << 10, "the operand tiles fit the smaller size");
+        const size_t smem = ncols > 256 ? (size_t)120 << 10 : (size_t)80 << 10;
+        QW_TRY(allow_smem(project_tc_kernel, (size_t)120 << 10));
         const int64_t blocks = (nv + PT_ROWS - 1) / PT_ROWS;
         if (blocks > 2147483647LL) return QW_ERR_ARG;
         project_tc_kernel<<<(unsigned)blocks, PT_ROWS, smem, s>>>(h, ncols);

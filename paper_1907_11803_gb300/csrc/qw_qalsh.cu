@@ -350,8 +350,7 @@ qw_status launch_qalsh_sort(double *P, int64_t n, int m, int nT, uint16_t *tlid,
                             uint16_t *lid, cudaStream_t s)
 {
     const size_t smem = (size_t)QS_HALF * (sizeof(unsigned long long) + sizeof(uint16_t));
-    QW_CUDA_TRY(cudaFuncSetAttribute(qalsh_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+    QW_TRY(allow_smem(qalsh_sort_kernel, smem));
     qalsh_sort_kernel<<<dim3((unsigned)nT, (unsigned)m), QS_THREADS, smem, s>>>(P, n, nT, tlid,
                                                                              qkey, lid);
     QW_CUDA_TRY(cudaGetLastError());

@@ -961,6 +961,15 @@ __global__ void __launch_bounds__(RR_THREADS) rerank_tc_kernel(
                      dists_out + (int64_t)q * k, vec);
 }
 
+// Shared memory of P2 candidate slots (a power of two): the FP32 form's arrays, and
+// with the pre-filters' candidate ids.
+static_assert((QW_MAX_CAND & (QW_MAX_CAND - 1)) == 0, "the most slots");
+size_t rerank_smem(int P2)
+{
+    return (size_t)P2 * (sizeof(double) + 2 * sizeof(float) + sizeof(int32_t) + 1);
+}
+size_t prefilter_smem(int P2) { return rerank_smem(P2) + 16 + (size_t)P2 * sizeof(int32_t); }
+
 }  // namespace
 
 // Rows a warp takes at a time: 2, 4 (default) or 8.
@@ -979,12 +988,11 @@ qw_status launch_rerank_bf16(const IndexView &ix, const void *Rb, const float *r
     if (nb == 0) return QW_OK;
     int P2 = 2;
     while (P2 < cap) P2 <<= 1;
-    const size_t smem = (size_t)P2 * (sizeof(double) + 2 * sizeof(float) + sizeof(int32_t) + 1) +
-                        16 + (size_t)P2 * sizeof(int32_t);
-    const void *fn = rows == 2 ? (const void *)rerank_bf16_kernel<2>
-                     : rows == 8 ? (const void *)rerank_bf16_kernel<8>
-                                 : (const void *)rerank_bf16_kernel<4>;
-    QW_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = prefilter_smem(P2);
+    QW_TRY(allow_smem(rows == 2   ? rerank_bf16_kernel<2>
+                      : rows == 8 ? rerank_bf16_kernel<8>
+                                  : rerank_bf16_kernel<4>,
+                      prefilter_smem(QW_MAX_CAND)));
     // rows in the locality order when the index has them (the copy's order)
     const float *Xr = ix.Xloc ? ix.Xloc : ix.X;
     const int32_t *row_of = ix.Xloc ? ix.inv : nullptr;
@@ -1016,15 +1024,13 @@ qw_status launch_rerank_tc(const IndexView &ix, const void *Rb, const float *rno
     const int dk = (d + 15) & ~15;
     const int KC = dk < TR_KC ? dk : TR_KC;
     const size_t smem = (size_t)TR_STAGES * TR_ROWS * KC * 2 + (size_t)TR_N * dk * 2 +
-                        (size_t)P2 * (sizeof(double) + 2 * sizeof(float) + sizeof(int32_t) + 1) +
-                        16 + (size_t)P2 * sizeof(int32_t);
-    if (smem + 2048 > 227 * 1024) {
+                        prefilter_smem(P2);
+    if (smem + 2048 > kMaxBlockSmem) {
         set_error("qw_run_workload: QW_RERANK_BF16_TC needs (k + v) and d small enough for its "
                   "shared-memory tiles");
         return QW_ERR_ARG;
     }
-    QW_CUDA_TRY(cudaFuncSetAttribute(rerank_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+    QW_TRY(allow_smem(rerank_tc_kernel, kMaxBlockSmem - 2048));
     const float *Xr = ix.Xloc ? ix.Xloc : ix.X;
     const int32_t *row_of = ix.Xloc ? ix.inv : nullptr;
     const bool vec = (d % 4 == 0) && ((uintptr_t)Qb % 16 == 0) && ((uintptr_t)Xr % 16 == 0);
@@ -1049,12 +1055,11 @@ qw_status launch_rerank(const IndexView &ix, const float *Qb, int nb, int k, int
     const float *X = Xrows ? Xrows : ix.X;
     int P2 = 2;
     while (P2 < cap) P2 <<= 1;
-    const size_t smem = (size_t)P2 * (sizeof(double) + 2 * sizeof(float) + sizeof(int32_t) + 1);
+    const size_t smem = rerank_smem(P2);
     // 16-byte row loads need d % 4 == 0 and 16-byte aligned bases
     const bool vec = (ix.d % 4 == 0) && ((uintptr_t)Qb % 16 == 0) && ((uintptr_t)X % 16 == 0);
     auto launch = [&](auto kernel) -> qw_status {
-        QW_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem));
+        QW_TRY(allow_smem(kernel, rerank_smem(QW_MAX_CAND)));
         kernel<<<nb, RR_THREADS, smem, s>>>(X, row_of, ix.d, Qb, k, cap, P2, st.cand, st.nkeep,
                                             ids_out, dists_out, vec);
         QW_CUDA_TRY(cudaGetLastError());
