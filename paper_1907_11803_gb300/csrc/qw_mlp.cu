@@ -272,43 +272,50 @@ __global__ void features_kernel(const float *__restrict__ Q, const int32_t *__re
     }
 }
 
-// Sum of squares: each thread in a pair of floats (every square and every sum
-// split into its rounded value and the exact error, the errors summed apart:
-// about 2^-44 of the sum), the threads' sums in FP64.  FP64 throughout runs at
-// two lanes a clock and SM: 483 us for 1,000,000 x 128, 122 us so.
+// Sum of squares: each thread in pairs of floats (every square and every sum split
+// into its rounded value and the exact error, the errors summed apart), 128 squares
+// at a time, the pairs added in FP64.  The pieces' errors are below 2^-33 of the sum
+// (2 L^2 2^-48 with L = 128), about 2^-42 as they fall; a piece whose sum is below
+// 2^-80 (the squares' errors would be lost below 2^-149) or past FP32 is summed
+// again in FP64.  FP64 throughout runs at two lanes a clock and SM: 483 us for
+// 1,000,000 x 128, 122 us so.
+constexpr int kSumPieces = 32;  // 16-byte words per piece and thread
+
 __global__ void __launch_bounds__(256) sumsq_kernel(const float *__restrict__ X, int64_t count,
                                                     double *__restrict__ out)
 {
-    float hi = 0.0f, lo = 0.0f;
-    auto add = [&](float x) {
-        const float p = __fmul_rn(x, x);
-        const float pe = fmaf(x, x, -p);
-        const float s = __fadd_rn(hi, p);
-        const float z = __fsub_rn(s, hi);
-        const float se = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, z)), __fsub_rn(p, z));
-        hi = s;
-        lo = __fadd_rn(lo, __fadd_rn(se, pe));
-    };
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t n4 = (reinterpret_cast<uintptr_t>(X) & 15) == 0 ? count / 4 : 0;
-    for (int64_t i = i0; i < n4; i += step) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(X) + i);
-        add(v.x);
-        add(v.y);
-        add(v.z);
-        add(v.w);
+    double s = 0.0;
+    for (int64_t p0 = i0; p0 < n4; p0 += kSumPieces * step) {
+        const int64_t p1 = min(n4, p0 + kSumPieces * step);
+        float hi = 0.0f, lo = 0.0f;
+        auto add = [&](float x) {
+            const float p = __fmul_rn(x, x);
+            const float pe = fmaf(x, x, -p);
+            const float t = __fadd_rn(hi, p);
+            const float z = __fsub_rn(t, hi);
+            const float te = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z));
+            hi = t;
+            lo = __fadd_rn(lo, __fadd_rn(te, pe));
+        };
+#pragma unroll 4
+        for (int64_t i = p0; i < p1; i += step) {
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(X) + i);
+            add(v.x);
+            add(v.y);
+            add(v.z);
+            add(v.w);
+        }
+        if (hi >= 0x1p-80f && hi <= 3.4e38f && fabsf(lo) <= 3.4e38f) {
+            s += (double)hi + (double)lo;
+        } else {
+            for (int64_t i = p0; i < p1; i += step)
+                for (int64_t e = 4 * i; e < 4 * i + 4; ++e) s += (double)X[e] * (double)X[e];
+        }
     }
-    for (int64_t i = 4 * n4 + i0; i < count; i += step) add(__ldg(X + i));
-    double s;
-    if (hi <= 3.4e38f && fabsf(lo) <= 3.4e38f) {
-        s = (double)hi + (double)lo;
-    } else {  // squares beyond FP32: this thread's share again in FP64
-        s = 0.0;
-        for (int64_t i = i0; i < n4; i += step)
-            for (int64_t e = 4 * i; e < 4 * i + 4; ++e) s += (double)X[e] * (double)X[e];
-        for (int64_t i = 4 * n4 + i0; i < count; i += step) s += (double)X[i] * (double)X[i];
-    }
+    for (int64_t i = 4 * n4 + i0; i < count; i += step) s += (double)X[i] * (double)X[i];
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
 }
