@@ -361,8 +361,9 @@ int32_t qw_qalsh_collision_threshold(int32_t m, float w, int32_t c, int64_t n, i
  * lies within a proven error bound (and at least 1e-5 w) of a bucket boundary
  * is recomputed in pairs of floats, and where those leave the floor open in
  * FP64 with the dot product summed in index order, so H equals the FP64
- * result.  *n_fixups (optional, host) receives how many were
- * recomputed; passing it makes the call wait for the stream.
+ * result.  *n_fixups (optional, host) receives how many lie that close to a
+ * boundary (in blocks of up to 256 rows, which are summed in pairs of floats at
+ * once, too); passing it makes the call wait for the stream.
  * Errors: QW_ERR_ARG (null pointer, nv < 0, d < 1, m < 1, w <= 0),
  * QW_ERR_RANGE (a bucket id outside int32; H is then unspecified),
  * QW_ERR_CUDA. */

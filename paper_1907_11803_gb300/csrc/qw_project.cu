@@ -174,8 +174,8 @@ __device__ __noinline__ double open_value(const float *v, const float *a, int d,
 // d = 512).  At d = 512 one entry in 50,000 is open after the pairs, so a call met
 // the sequence in some block: 2,000 rows x 64 took 107 us, 40
 // so.  Where more than eight lanes are open they take the sequence side by side
-// at once.  Returns true when the pair did not decide.
-__device__ __forceinline__ bool settle_entry(const HashArgs &h, int64_t r, int i, float2 t,
+// at once.
+__device__ __forceinline__ void settle_entry(const HashArgs &h, int64_t r, int i, float2 t,
                                              double S, bool valid)
 {
     const double w = (double)h.w, bias = valid ? (double)h.b[i] : 0.0;
@@ -188,7 +188,7 @@ __device__ __forceinline__ bool settle_entry(const HashArgs &h, int64_t r, int i
                                     S, open);
         if (open) u = x;
     }
-    if (!valid) return false;
+    if (!valid) return;
     const double f = floor(u);
     int32_t *hp = h.H + r * h.ld_row + (int64_t)i * h.ld_col;
     if (!(f >= -2147483647.0 && f <= 2147483646.0)) {
@@ -197,7 +197,21 @@ __device__ __forceinline__ bool settle_entry(const HashArgs &h, int64_t r, int i
     } else {
         *hp = (int32_t)f;
     }
-    return open;
+}
+
+// Pass 1's error of t per unit of W(a) W(v), over w.
+__device__ __forceinline__ float sum_unit(int d, float w)
+{
+    return kU * (1.0f + 4.0f * (float)d * kU) * 1.01f / w;
+}
+
+// Whether floor(u) of pass 1 is taken for u = (t + b) / w, E the error of t over w:
+// not near an edge, not out of int32, not a NaN.
+__device__ __forceinline__ bool sure_at(float u, float f, float E)
+{
+    const float frac = u - f;                       // exact
+    const float eps = fmaxf(E + 4.0f * kU * (fabsf(u) + 1.0f), 1e-5f);
+    return fminf(frac, 1.0f - frac) > eps && f >= -2147483520.0f && f <= 2147483520.0f;
 }
 
 // Pass 2 of a block: its `count` listed entries (local row << 7 | local
@@ -233,6 +247,7 @@ __device__ void settle_listed(const HashArgs &h, const uint16_t *list, int count
 // entries per block.  The tiled kernel gives at most one block per 64 rows,
 // whose dependent chunks take 11.5 us at d = 128 whatever the rows; this form
 // takes 5.6 us for 16 rows of 64 projections and 15.8 for 300, hence the limit.
+// The entries counted are those that the tiled kernel would list.
 __global__ void __launch_bounds__(NT) project_rows_kernel(HashArgs h)
 {
     const int64_t e = (int64_t)blockIdx.x * (NT / 8) + (threadIdx.x >> 3);
@@ -255,8 +270,15 @@ __global__ void __launch_bounds__(NT) project_rows_kernel(HashArgs h)
         sv += __shfl_xor_sync(0xffffffffu, sv, off);
         sa += __shfl_xor_sync(0xffffffffu, sa, off);
     }
-    const double S = (double)norm_bound(sv, h.d) * (double)norm_bound(sa, h.d);
-    if (settle_entry(h, r, i, t, S, valid && lane8 == 0) && h.fixups) atomicAdd(h.fixups, 1ull);
+    const float wv = norm_bound(sv, h.d), wa = norm_bound(sa, h.d);
+    const bool mine = valid && lane8 == 0;
+    if (h.fixups) {
+        const float u = __fmul_rn(__fadd_rn(t.x, valid ? __ldg(h.b + i) : 0.0f), __frcp_rn(h.w));
+        const uint32_t near = __ballot_sync(
+            0xffffffffu, mine && !sure_at(u, floorf(u), wa * sum_unit(h.d, h.w) * wv));
+        if (near && (threadIdx.x & 31) == 0) atomicAdd(h.fixups, (unsigned long long)__popc(near));
+    }
+    settle_entry(h, r, i, t, (double)wv * (double)wa, mine);
 }
 
 // A (32 TM) x (8 TN) tile of entries per block, TM x TN per thread, the operands
@@ -407,8 +429,7 @@ __global__ void __launch_bounds__(NT, 2) project_fp32_kernel(HashArgs h)
     // dividing by w as a product with its reciprocal: one more rounding, 3 u |u|
     // in all (a reciprocal below the normal range is off by less than the 1e-5)
     const float rw = __frcp_rn(w);
-    // error of t per unit of W(a) W(v), over w
-    const float unit = kU * (1.0f + 4.0f * (float)d * kU) * 1.01f / w;
+    const float unit = sum_unit(d, w);
     const bool out_rows = h.ld_col == 1 && (h.ld_row & 3) == 0 && (m & 3) == 0 &&
                           (reinterpret_cast<uintptr_t>(h.H) & 15) == 0;
     const bool out_cols = TM == 8 && h.ld_row == 1 && (h.ld_col & 3) == 0 && row0 + BM <= h.nv &&
@@ -430,11 +451,7 @@ __global__ void __launch_bounds__(NT, 2) project_fp32_kernel(HashArgs h)
             const int lc = col_of(j);
             const float u = __fmul_rn(__fadd_rn(acc[i][j], bias[j]), rw);
             const float f = floorf(u);
-            const float frac = u - f;                       // exact
-            const float eps = fmaxf(na[j] * wv + 4.0f * kU * (fabsf(u) + 1.0f), 1e-5f);
-            // near an edge, out of int32 or NaN: the second pass decides
-            const bool sure = fminf(frac, 1.0f - frac) > eps && f >= -2147483520.0f &&
-                              f <= 2147483520.0f;
+            const bool sure = sure_at(u, f, na[j] * wv);  // else the second pass decides
             acc[i][j] = __int_as_float(sure ? (int32_t)f : 0);
             if (!sure && row0 + lr < h.nv && col0 + lc < m)
                 sm.fix.list[atomicAdd(&n_list, 1)] = (uint16_t)(lr << 7 | lc);
