@@ -10,14 +10,21 @@
 // inside one leaf of nearby points.  A node all of whose points fall on one
 // side (copies of one point) is cut in the middle, and so is every node after
 // kMaxUneven levels, which bounds the depth.  The order only decides which ids
-// share a group: no result depends on it, so FP32 sums serve.
+// share a group: no result depends on it, only how many groups the bitmap path has
+// to count.  FP32 sums serve where they are taken of what tells a node's points
+// apart: every coordinate is read as its difference from the node's first point
+// (exact to a rounding, so that an offset common to the data costs nothing), and a
+// hyperplane's normal is scaled to a largest component of 1 (only the side and the
+// order of distances count), so that no product leaves the range that the
+// coordinates themselves fit.  Sums of a chunk's differences stay below FP32's
+// largest number for coordinates up to about 1e33.
 //
 // All nodes of a level are split together.  A node's points are cut in chunks
 // of whole blocks (256 rows, more for large nodes: at most kMaxChunks chunks
 // per node); the kernels of a level work on chunks, those that combine a
 // node's chunks (in chunk order: the tree is the same for every build) on
-// nodes.  What bounds it is reading the rows five times a level: 20 ms at
-// 1,000,000 x 128 (21 levels; 11 ms of it the side sums), against more than a
+// nodes.  What bounds it is reading the rows five times a level: 18 ms at
+// 1,000,000 x 128 (21 levels; 8.4 ms of it the side sums), against more than a
 // second on 16 host cores in FP64, beside copying the data there.  The host
 // only launches: it reads three counters per level.
 #include "qw_internal.cuh"
@@ -46,11 +53,13 @@ struct Tree {
     int32_t *perm, *perm2;   // the order, and the split nodes' next one
     float *t;                // signed distance to the node's hyperplane (times |v|)
     int32_t *lo, *hi, *c0;   // nodes of the level: range, first chunk
-    int32_t *lo2, *hi2, *c02;
+    int32_t *o;              // ... and data id of the first point
+    int32_t *lo2, *hi2, *c02, *o2;
     int32_t *cut;            // per node, points of the first child
     int32_t *node, *node2;   // per chunk, its node
-    float *v;                // per node, c2 - c1 (d), then the threshold
-    float *part;             // per chunk, coordinate sums of both sides (2 d)
+    float *v;                // per node, c2 - c1 scaled (d), then the threshold
+    float *part;             // per chunk, coordinate sums of both sides (2 d), of the
+                             // differences from the node's first point
     int32_t *below;          // per chunk, points of the first side
     unsigned long long *kmin, *kmax;  // per chunk, smallest and largest (key, position)
     int32_t *ctl;            // next level: nodes, chunks, longest node
@@ -78,11 +87,17 @@ __device__ __forceinline__ void chunk_range(const Tree &T, int chunk, int &u, in
     e = min(T.hi[u], b + cs);
 }
 
-// f(position, row . w) for the rows at positions [b, e) of the order, a warp
+// The node's first point: what its coordinates are taken relative to.
+__device__ __forceinline__ const float *node_origin(const Tree &T, int u)
+{
+    return T.X + (int64_t)T.o[u] * T.d;
+}
+
+// f(position, (row - o) . w) for the rows at positions [b, e) of the order, a warp
 // four rows at a time (their loads in flight together); every lane calls f.
 template <class F>
-__device__ __forceinline__ void rows_dot(const Tree &T, const float *__restrict__ w, int b, int e,
-                                         F &&f)
+__device__ __forceinline__ void rows_dot(const Tree &T, const float *__restrict__ w,
+                                         const float *__restrict__ o, int b, int e, F &&f)
 {
     constexpr int R = 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, d = T.d;
@@ -95,21 +110,24 @@ __device__ __forceinline__ void rows_dot(const Tree &T, const float *__restrict_
             acc[r] = 0.0f;
         }
         if (T.vec) {
+#pragma unroll 1  // (the rows' loads are in flight together; more registers cost blocks)
             for (int c = 4 * lane; c < d; c += 128) {
                 const float4 y = *reinterpret_cast<const float4 *>(w + c);
+                const float4 q = __ldg(reinterpret_cast<const float4 *>(o + c));
                 float4 z[R];
 #pragma unroll
                 for (int r = 0; r < R; ++r) z[r] = __ldg(reinterpret_cast<const float4 *>(x[r] + c));
 #pragma unroll
                 for (int r = 0; r < R; ++r)
-                    acc[r] = fmaf(z[r].x, y.x, fmaf(z[r].y, y.y, fmaf(z[r].z, y.z,
-                                                                     fmaf(z[r].w, y.w, acc[r]))));
+                    acc[r] = fmaf(z[r].x - q.x, y.x,
+                                  fmaf(z[r].y - q.y, y.y,
+                                       fmaf(z[r].z - q.z, y.z, fmaf(z[r].w - q.w, y.w, acc[r]))));
             }
         } else {
             for (int c = lane; c < d; c += 32) {
-                const float y = w[c];
+                const float y = w[c], q = __ldg(o + c);
 #pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] = fmaf(__ldg(x[r] + c), y, acc[r]);
+                for (int r = 0; r < R; ++r) acc[r] = fmaf(__ldg(x[r] + c) - q, y, acc[r]);
             }
         }
 #pragma unroll
@@ -130,6 +148,7 @@ __global__ void tree_init_kernel(Tree T)
         T.lo[0] = 0;
         T.hi[0] = (int)T.n;
         T.c0[0] = 0;
+        T.o[0] = 0;
     }
     const int cs = chunk_rows((int)T.n);
     if (j0 < ((int)T.n + cs - 1) / cs) T.node[j0] = 0;
@@ -137,13 +156,13 @@ __global__ void tree_init_kernel(Tree T)
 
 // Per chunk, the positions of the smallest and largest projection on direction
 // `dir` (ties: the first position).
-__global__ void __launch_bounds__(TR_ROWS) tree_seed_kernel(Tree T, int dir)
+__global__ void __launch_bounds__(TR_ROWS, 4) tree_seed_kernel(Tree T, int dir)
 {
     __shared__ unsigned long long smin[TR_ROWS / 32], smax[TR_ROWS / 32];
     int u, b, e;
     chunk_range(T, blockIdx.x, u, b, e);
     unsigned long long mn = ~0ull, mx = 0ull;
-    rows_dot(T, T.A + (int64_t)dir * T.d, b, e, [&](int j, float t) {
+    rows_dot(T, T.A + (int64_t)dir * T.d, node_origin(T, u), b, e, [&](int j, float t) {
         const unsigned long long k = (unsigned long long)fkey(t) << 32;
         mn = min(mn, k | (uint32_t)j);
         mx = max(mx, k | (0xffffffffu - (uint32_t)j));
@@ -163,22 +182,25 @@ __global__ void __launch_bounds__(TR_ROWS) tree_seed_kernel(Tree T, int dir)
     }
 }
 
-// Block-wide sum of one float per thread.
-__device__ __forceinline__ float block_sum(float x, float *tmp)
+// Block-wide sum (or largest) of one float per thread.
+template <bool MAX>
+__device__ __forceinline__ float block_reduce(float x, float *tmp)
 {
+    auto both = [](float a, float b) { return MAX ? fmaxf(a, b) : a + b; };
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    for (int off = 16; off > 0; off >>= 1) x = both(x, __shfl_xor_sync(0xffffffffu, x, off));
     __syncthreads();
     if ((threadIdx.x & 31) == 0) tmp[threadIdx.x >> 5] = x;
     __syncthreads();
-    float s = 0.0f;
-    for (int w = 0; w < TR_ROWS / 32; ++w) s += tmp[w];
+    float s = tmp[0];
+    for (int w = 1; w < TR_ROWS / 32; ++w) s = both(s, tmp[w]);
     return s;
 }
 
-// Per node: the hyperplane between two centroids, v = c2 - c1 and the
-// threshold (|c2|^2 - |c1|^2) / 2, from the seeds (round 0) or from the sums of
-// the chunks' sides.  A side without points leaves the hyperplane as it is.
+// Per node: the hyperplane between two centroids, v = c2 - c1 over its largest
+// component and the threshold v . (c1 + c2) / 2, from the seeds (round 0) or from
+// the sums of the chunks' sides.  A side without points leaves the hyperplane as it
+// is.
 __global__ void __launch_bounds__(TR_ROWS) tree_plane_kernel(Tree T, int n_chunks, int n_nodes,
                                                              bool seeds)
 {
@@ -189,7 +211,9 @@ __global__ void __launch_bounds__(TR_ROWS) tree_plane_kernel(Tree T, int n_chunk
     const int k0 = T.c0[u], k1 = u + 1 < n_nodes ? T.c0[u + 1] : n_chunks;
     const int len = T.hi[u] - T.lo[u];
     float *v = T.v + (int64_t)u * T.dv;
-    float q = 0.0f;
+    // the centroids, relative to the node's first point
+    const float *x1 = nullptr, *x2 = nullptr, *o = node_origin(T, u);
+    float r1 = 0.0f, r2 = 0.0f;
     if (seeds) {
         if (threadIdx.x == 0) {
             s_mn = ~0ull;
@@ -201,13 +225,8 @@ __global__ void __launch_bounds__(TR_ROWS) tree_plane_kernel(Tree T, int n_chunk
             atomicMax(&s_mx, T.kmax[k]);
         }
         __syncthreads();
-        const float *x1 = T.X + (int64_t)T.perm[(uint32_t)s_mn] * d;
-        const float *x2 = T.X + (int64_t)T.perm[0xffffffffu - (uint32_t)s_mx] * d;
-        for (int c = threadIdx.x; c < d; c += TR_ROWS) {
-            const float a = x1[c], b = x2[c];
-            v[c] = b - a;
-            q += (b - a) * (b + a);
-        }
+        x1 = T.X + (int64_t)T.perm[(uint32_t)s_mn] * d;
+        x2 = T.X + (int64_t)T.perm[0xffffffffu - (uint32_t)s_mx] * d;
     } else {
         if (threadIdx.x == 0) s_below = 0;
         __syncthreads();
@@ -217,29 +236,50 @@ __global__ void __launch_bounds__(TR_ROWS) tree_plane_kernel(Tree T, int n_chunk
         __syncthreads();
         const int n1 = s_below, n2 = len - n1;
         if (n1 == 0 || n2 == 0) return;
-        const float r1 = 1.0f / (float)n1, r2 = 1.0f / (float)n2;
-        for (int c = threadIdx.x; c < d; c += TR_ROWS) {
-            float a = 0.0f, b = 0.0f;
+        r1 = 1.0f / (float)n1;
+        r2 = 1.0f / (float)n2;
+    }
+    auto centroids = [&](int c, float &a, float &b) {
+        if (seeds) {
+            a = x1[c] - o[c];
+            b = x2[c] - o[c];
+        } else {
+            a = b = 0.0f;
 #pragma unroll 8
             for (int k = k0; k < k1; ++k) {
-                a += T.part[(int64_t)k * 2 * d + c];
-                b += T.part[(int64_t)k * 2 * d + d + c];
+                a = fmaf(T.part[(int64_t)k * 2 * d + c], r1, a);
+                b = fmaf(T.part[(int64_t)k * 2 * d + d + c], r2, b);
             }
-            a *= r1;
-            b *= r2;
-            v[c] = b - a;
-            q += (b - a) * (b + a);
         }
+    };
+    // the centroids' middle takes the place of the sums of the node's first chunk (a
+    // coordinate's sums are read by its thread alone)
+    float *mid = T.part + (int64_t)k0 * 2 * d;
+    float most = 0.0f;
+    for (int c = threadIdx.x; c < d; c += TR_ROWS) {
+        float a, b;
+        centroids(c, a, b);
+        mid[c] = 0.5f * a + 0.5f * b;
+        v[c] = b - a;
+        most = fmaxf(most, fabsf(b - a));
     }
-    q = block_sum(q, tmp);
-    if (threadIdx.x == 0) v[d] = 0.5f * q;
+    most = block_reduce<true>(most, tmp);
+    float q = 0.0f;
+    for (int c = threadIdx.x; c < d; c += TR_ROWS) {
+        const float w = most > 0.0f ? v[c] / most : 0.0f;
+        v[c] = w;
+        q += w * mid[c];
+    }
+    q = block_reduce<false>(q, tmp);
+    if (threadIdx.x == 0) v[d] = q;
 }
 
 // Per chunk: each row's side of its node's hyperplane, and the coordinate sums
 // of both sides.  A block takes 256 rows at a time: warps form the rows'
 // projections, then threads own coordinates (256 / d threads share one, each a
-// part of the rows) and add the rows, now in L1, side by side.
-__global__ void __launch_bounds__(TR_ROWS) tree_assign_kernel(Tree T, bool in_smem)
+// part of the rows) and add the rows, now in L1, side by side.  Five blocks per SM
+// hide its loads: 12.0 ms at 300,000 x 512 (three with 80 registers: 26).
+__global__ void __launch_bounds__(TR_ROWS, 5) tree_assign_kernel(Tree T, bool in_smem)
 {
     extern __shared__ float sums_s[];
     __shared__ uint8_t side[TR_ROWS];
@@ -247,7 +287,7 @@ __global__ void __launch_bounds__(TR_ROWS) tree_assign_kernel(Tree T, bool in_sm
     int u, b, e;
     chunk_range(T, blockIdx.x, u, b, e);
     const int d = T.d;
-    const float *v = T.v + (int64_t)u * T.dv;
+    const float *v = T.v + (int64_t)u * T.dv, *o = node_origin(T, u);
     const float thr = v[d];
     float *out = T.part + (int64_t)blockIdx.x * 2 * d;
     const int G = in_smem && d < TR_ROWS ? TR_ROWS / d : 1;   // threads per coordinate
@@ -257,7 +297,7 @@ __global__ void __launch_bounds__(TR_ROWS) tree_assign_kernel(Tree T, bool in_sm
     __syncthreads();
     for (int r0 = b; r0 < e; r0 += TR_ROWS) {
         const int r1 = min(e, r0 + TR_ROWS);
-        rows_dot(T, v, r0, r1, [&](int j, float t) {
+        rows_dot(T, v, o, r0, r1, [&](int j, float t) {
             if ((threadIdx.x & 31) == 0) side[j - r0] = t < thr ? 0 : 1;
         });
         __syncthreads();
@@ -266,9 +306,10 @@ __global__ void __launch_bounds__(TR_ROWS) tree_assign_kernel(Tree T, bool in_sm
         const int g = G > 1 ? threadIdx.x / d : 0;
         for (int c = G > 1 ? threadIdx.x % d : threadIdx.x; c < d && g < G; c += TR_ROWS) {
             float s0 = sums[g * 2 * d + c], s1 = sums[g * 2 * d + d + c];
+            const float oc = __ldg(o + c);
 #pragma unroll 8
             for (int j = r0 + g; j < r1; j += G) {
-                const float x = __ldg(T.X + (int64_t)T.perm[j] * d + c);
+                const float x = __ldg(T.X + (int64_t)T.perm[j] * d + c) - oc;
                 const bool second = side[j - r0] != 0;
                 s0 += second ? 0.0f : x;
                 s1 += second ? x : 0.0f;
@@ -289,7 +330,7 @@ __global__ void __launch_bounds__(TR_ROWS) tree_assign_kernel(Tree T, bool in_sm
 }
 
 // Per chunk: the rows' signed distances and how many are below zero.
-__global__ void __launch_bounds__(TR_ROWS) tree_side_kernel(Tree T)
+__global__ void __launch_bounds__(TR_ROWS, 4) tree_side_kernel(Tree T)
 {
     __shared__ int s_below;
     int u, b, e;
@@ -299,7 +340,7 @@ __global__ void __launch_bounds__(TR_ROWS) tree_side_kernel(Tree T)
     if (threadIdx.x == 0) s_below = 0;
     __syncthreads();
     int mine = 0;
-    rows_dot(T, v, b, e, [&](int j, float t) {
+    rows_dot(T, v, node_origin(T, u), b, e, [&](int j, float t) {
         t -= thr;
         // keep an order where sums overflow
         if (!(fabsf(t) <= FLT_MAX)) t = t < 0.0f ? -FLT_MAX : FLT_MAX;
@@ -475,6 +516,7 @@ __global__ void __launch_bounds__(1024) tree_next_kernel(Tree T, int n_nodes)
             T.lo2[at] = lo[x];
             T.hi2[at] = hi[x];
             T.c02[at] = ct;
+            T.o2[at] = T.perm[lo[x]];
             const int k = (len + chunk_rows(len) - 1) / chunk_rows(len);
             for (int y = 0; y < k; ++y) T.node2[ct + y] = at;
             ct += k;
@@ -525,7 +567,7 @@ qw_status locality_order(const float *X, int64_t n, int d, const float *A, int m
     };
     const size_t o_perm2 = take((size_t)n * 4), o_t = take((size_t)n * 4);
     const size_t o_node = take((size_t)max_chunks * 4), o_node2 = take((size_t)max_chunks * 4);
-    size_t o_n[7];
+    size_t o_n[9];
     for (size_t &o : o_n) o = take((size_t)(max_nodes + 1) * 4);
     const size_t o_v = take((size_t)max_nodes * T.dv * 4);
     const size_t o_part = take((size_t)max_chunks * 2 * d * 4);
@@ -540,8 +582,8 @@ qw_status locality_order(const float *X, int64_t n, int d, const float *A, int m
     T.t = reinterpret_cast<float *>(p + o_t);
     T.node = reinterpret_cast<int32_t *>(p + o_node);
     T.node2 = reinterpret_cast<int32_t *>(p + o_node2);
-    int32_t **nodes[7] = {&T.lo, &T.hi, &T.c0, &T.lo2, &T.hi2, &T.c02, &T.cut};
-    for (int k = 0; k < 7; ++k) *nodes[k] = reinterpret_cast<int32_t *>(p + o_n[k]);
+    int32_t **nodes[9] = {&T.lo, &T.hi, &T.c0, &T.o, &T.lo2, &T.hi2, &T.c02, &T.o2, &T.cut};
+    for (int k = 0; k < 9; ++k) *nodes[k] = reinterpret_cast<int32_t *>(p + o_n[k]);
     T.v = reinterpret_cast<float *>(p + o_v);
     T.part = reinterpret_cast<float *>(p + o_part);
     T.below = reinterpret_cast<int32_t *>(p + o_below);
@@ -578,6 +620,7 @@ qw_status locality_order(const float *X, int64_t n, int d, const float *A, int m
         std::swap(T.lo, T.lo2);
         std::swap(T.hi, T.hi2);
         std::swap(T.c0, T.c02);
+        std::swap(T.o, T.o2);
         std::swap(T.node, T.node2);
     }
     QW_CUDA_TRY(cudaStreamSynchronize(s));  // mem is freed on return
