@@ -288,7 +288,13 @@ __global__ void __launch_bounds__(NT) project_rows_kernel(HashArgs h)
 // 8 x 8 (16 clocks of reads against 16 of products per warp and coordinate;
 // 8 x 4 measured 654 us on 1,000,000 x 128 x 64, the first form with 4 x 4 and
 // 4-byte reads 1,055 us, this one 459 us).  TM = 2 serves row counts
-// that would leave SMs without a block of 256 rows.
+// that would leave SMs without a block of 256 rows; where its blocks of 64 rows leave
+// SMs without one too, gridDim.z blocks form the same tile and each settles and
+// writes its share of the rows: on data far from the origin, where the first pass
+// leaves most entries open, a block's second pass takes far longer than its first.
+// 300 rows of 512 coordinates about 0, 1,000 and 100,000 (w = 4): 32, 253 and 1,788
+// us with a block per tile, 32, 42 and 145 so; 2,000 rows of 128: 12, 39 and 135, now
+// 12, 20 and 56.
 template <int TM, int TN>
 __global__ void __launch_bounds__(NT, 2) project_fp32_kernel(HashArgs h)
 {
@@ -445,6 +451,7 @@ __global__ void __launch_bounds__(NT, 2) project_fp32_kernel(HashArgs h)
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int lr = row_of(i);
+        if (TM == 2 && lr % gridDim.z != blockIdx.z) continue;  // another block's share
         const float wv = vn[lr];
 #pragma unroll
         for (int j = 0; j < TN; ++j) {
@@ -515,6 +522,8 @@ __global__ void __launch_bounds__(NT, 2) project_fp32_kernel(HashArgs h)
 constexpr int PT_ROWS = 128;  // rows per CTA (the MMA's M)
 constexpr int PT_KC = 64;     // input coordinates per staged chunk
 
+// gridDim.y blocks form the same 128 rows and each settles and writes its share (as
+// above, where the rows give few blocks).
 __global__ void __launch_bounds__(PT_ROWS, 1) project_tc_kernel(HashArgs h, uint32_t ncols)
 {
     const float *__restrict__ V = h.V, *__restrict__ A = h.A, *__restrict__ b = h.b;
@@ -642,7 +651,7 @@ __global__ void __launch_bounds__(PT_ROWS, 1) project_tc_kernel(HashArgs h, uint
         tc_ld16(tbase + lane_base + (uint32_t)n0, hh);
         tc_ld16(tbase + lane_base + (uint32_t)(N + n0), hl);
         tc_ld16(tbase + lane_base + (uint32_t)(2 * N + n0), lh);
-        if (r >= nv) continue;
+        if (r >= nv || tid % gridDim.y != blockIdx.y) continue;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
             const int i = n0 + j;
@@ -698,6 +707,10 @@ qw_status launch_hash(const float *V, int64_t nv, int d, const float *A, const f
     h.err = err;
     h.fixups = fixups;
     h.vec = d % 4 == 0 && ((uintptr_t)V | (uintptr_t)A) % 16 == 0;
+    // blocks of one tile: one per SM in all, at least two rows each
+    auto shares = [](int64_t tiles) {
+        return std::max<int64_t>(1, std::min<int64_t>(32, 152 / tiles));
+    };
     if (tensor_cores && m <= 128) {
         const int N = (m + 15) & ~15;
         uint32_t ncols = 32;
@@ -712,7 +725,8 @@ qw_status launch_hash(const float *V, int64_t nv, int d, const float *A, const f
         QW_TRY(allow_smem(project_tc_kernel, (size_t)120 << 10));
         const int64_t blocks = (nv + PT_ROWS - 1) / PT_ROWS;
         if (blocks > 2147483647LL) return QW_ERR_ARG;
-        project_tc_kernel<<<(unsigned)blocks, PT_ROWS, smem, s>>>(h, ncols);
+        const dim3 grid((unsigned)blocks, (unsigned)shares(blocks));
+        project_tc_kernel<<<grid, PT_ROWS, smem, s>>>(h, ncols);
     } else if (nv <= kFewRows && nv * m <= kFewEntries) {
         project_rows_kernel<<<(unsigned)((nv * m + NT / 8 - 1) / (NT / 8)), NT, 0, s>>>(h);
     } else {
@@ -722,7 +736,7 @@ qw_status launch_hash(const float *V, int64_t nv, int d, const float *A, const f
         const bool wide = (nv + 255) / 256 * cb >= 2 * 152;
         const int64_t rb = wide ? (nv + 255) / 256 : (nv + 63) / 64;
         if (rb > 2147483647LL) return QW_ERR_ARG;
-        const dim3 grid((unsigned)rb, (unsigned)cb);
+        const dim3 grid((unsigned)rb, (unsigned)cb, wide ? 1u : (unsigned)shares(rb * cb));
         if (bn == 32 && wide) project_fp32_kernel<8, 4><<<grid, NT, 0, s>>>(h);
         else if (bn == 32) project_fp32_kernel<2, 4><<<grid, NT, 0, s>>>(h);
         else if (wide) project_fp32_kernel<8, 8><<<grid, NT, 0, s>>>(h);
