@@ -259,11 +259,11 @@ typedef struct {
 #define QW_PATH_BITMAP 3
 
 /* Kernel classes of the query path, for qw_profile. */
-#define QW_K_PROJECT 0   /* query projection + FP64 boundary pass */
+#define QW_K_PROJECT 0   /* query projection, entries near a bucket edge included */
 #define QW_K_SETUP 1     /* per-query state */
-#define QW_K_LEVEL 2     /* bucket-range search + collision counting, one launch per level
-                            (bitmap path with direct loads and a host-driven loop: the
-                            summary filter and the count pass only, see QW_K_BUCKET) */
+#define QW_K_LEVEL 2     /* collision counting: with the bucket-range search one launch per
+                            level (bitmap path: the summary filter and its one or two count
+                            passes, or the fused or staged kernel; see QW_K_BUCKET) */
 #define QW_K_DECIDE 3    /* per-level termination test */
 #define QW_K_SELECT 4    /* candidate selection under the k + v bound */
 #define QW_K_RERANK 5    /* candidate distances + top-k */
@@ -271,9 +271,9 @@ typedef struct {
                             query in one persistent launch */
 #define QW_K_ORDER 7     /* workload ordering: signature sort, gather, scatter of results */
 #define QW_K_START 8     /* learned start levels: features + network forward */
-#define QW_K_BUCKET 9    /* bitmap path, direct loads, host-driven loop: the bitmap numbers of
-                            the query's buckets before each level's filter (in graph mode they
-                            are part of QW_K_LEVEL) */
+#define QW_K_BUCKET 9    /* bitmap path, direct and fused loads, host-driven loop: the running
+                            queries and their buckets' bitmap numbers before each level's
+                            counts, one or two launches (in graph mode part of QW_K_LEVEL) */
 #define QW_K_COUNT 10
 
 /* Launch counts and (profile mode) summed kernel times of qw_run_workload /

@@ -790,12 +790,11 @@ static qw_status host_level_loop(qw_index *ix, LaunchTimer &tm, const IndexView 
             if (bitmap && loads != QW_LOADS_TMA) {
                 // the bucket numbers apart, so that QW_K_LEVEL times the filter
                 // and count passes alone
-                QW_TRY(tm.run(QW_K_BUCKET, 2, [&] {
+                QW_TRY(tm.run(QW_K_BUCKET, bm_level_launches(nb, st.bm_mp, loads, 1), [&] {
                     return launch_bm_level(view, nb, level, R, Rp, ix->l, ix->c, st, err, loads,
                                            s, nullptr, 1, tpw);
                 }));
-                const int nl = loads == QW_LOADS_FUSED ? 1 : 3;
-                QW_TRY(tm.run(QW_K_LEVEL, nl, [&] {
+                QW_TRY(tm.run(QW_K_LEVEL, bm_level_launches(nb, st.bm_mp, loads, 2), [&] {
                     return launch_bm_level(view, nb, level, R, Rp, ix->l, ix->c, st, err, loads,
                                            s, nullptr, 2, tpw);
                 }));
@@ -1145,7 +1144,7 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
     int32_t *HQall = ix->w_hq.as<int32_t>();
     QW_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
     if (!qalsh)
-        QW_TRY(tm.run(QW_K_PROJECT, 2, [&] {
+        QW_TRY(tm.run(QW_K_PROJECT, 1, [&] {
             return launch_hash(Qall, nq, d, ix->A.as<float>(), ix->b.as<float>(), m, ix->w, HQall,
                                m, 1, err, nullptr, s, qp && qp->projection == QW_PROJ_TENSOR);
         }));
@@ -1270,19 +1269,20 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
                 QW_TRY(host_level_loop(ix, tm, view, nb, cap, learned, use_bitmap, loads, tpw, err,
                                        st, s, &levels_run));
             }
-            QW_TRY(tm.run(QW_K_SELECT, use_bitmap ? (learned ? 10 : 8) + (tma_loads ? 1 : 0) : 2, [&] {
+            const int slots = (int)std::min<int64_t>(B, bm_reduce_wave(ix->nT));
+            const int n_select =
+                use_bitmap ? bm_select_launches(nb, tma_loads, slots, learned) : 2;
+            QW_TRY(tm.run(QW_K_SELECT, n_select, [&] {
                 if (use_bitmap) {
-                    const int slots = (int)std::min<int64_t>(B, bm_reduce_wave(ix->nT));
                     QW_TRY(launch_bm_list(view, nb, ix->l, ix->c, st, tma_loads, slots, s));
                     QW_TRY(launch_bm_reduce(view, nb, ix->l, cap, ix->c, st, slots, s));
                     if (learned) QW_TRY(launch_bm_recount(view, nb, ix->l, cap, ix->c, st, s));
-                    return launch_bm_collect(view, nb, ix->l, cap, st, stats_b, want_cand, s);
+                    QW_TRY(launch_bm_collect(view, nb, ix->l, cap, st, stats_b, want_cand, s));
+                    return launch_bm_overflow_list(st, nb, order ? perm : nullptr, b0, ovf_list,
+                                                   late_list, ovf_count, s);
                 }
                 return launch_collect(view, nb, ix->l, cap, st, stats_b, s);
             }));
-            if (use_bitmap)
-                QW_TRY(launch_bm_overflow_list(st, nb, order ? perm : nullptr, b0, ovf_list,
-                                               late_list, ovf_count, s));
             if (use_bitmap && tm.on) {
                 int32_t h_rd = 0;
                 QW_CUDA_TRY(cudaMemcpyAsync(&h_rd, st.rd_ctl + 1, sizeof(h_rd), cudaMemcpyDeviceToHost, s));
@@ -1360,13 +1360,11 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
             set_error("qw_run_workload: a staged-copy wait in the bitmap kernel gave up");
             return QW_ERR_TIMEOUT;
         }
-        // per level: the bucket numbers, filter and both counts (bitmap path, direct
-        // loads), else one counting launch
-        ix->prof.launches[QW_K_LEVEL] +=
-            (int64_t)h_ctl.iters *
-            (use_bitmap && loads == QW_LOADS_DIRECT ? 5 : (use_bitmap && loads == QW_LOADS_FUSED ? 3 : 1));
+        // per level the decision and the loop's step; per batch the loop's three
+        // first kernels, and the two that begin a second pass
+        ix->prof.launches[QW_K_LEVEL] += (int64_t)h_ctl.kernels;
         levels_run = (int)h_ctl.iters;
-        ix->prof.launches[QW_K_DECIDE] += 2 * (int64_t)h_ctl.iters + n_batches * (learned ? 3 : 1);
+        ix->prof.launches[QW_K_DECIDE] += 2 * (int64_t)h_ctl.iters + n_batches * (learned ? 5 : 3);
         if (learned) {
             ix->prof.start_fallbacks += (int64_t)h_ctl.fb_total;
             ix->prof.start_levels_skipped += (int64_t)h_ctl.skipped_total;

@@ -2383,6 +2383,18 @@ static void launch_fused(const IndexView &ix, int nb, int level, int l, QuerySta
         bm_fused_kernel<4, TPW><<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, nb, st, ctl);
 }
 
+// Up to four (query, projection) entries per thread of one block cost less than a
+// launch.
+static bool buckets_in_one_block(int nb, int mp) { return (int64_t)nb * mp <= 4096; }
+
+int bm_level_launches(int nb, int mp, int loads, int part)
+{
+    if (loads == QW_LOADS_TMA) return 1;
+    const int buckets = part == 2 ? 0 : buckets_in_one_block(nb, mp) ? 1 : 2;
+    const int counts = part == 1 ? 0 : loads == QW_LOADS_FUSED ? 1 : nb >= kDenseMin ? 3 : 2;
+    return buckets + counts;
+}
+
 qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int64_t Rp, int l,
                           int cgrow, QueryState &st, int *err, int loads, cudaStream_t s,
                           const LoopCtl *ctl, int part, int tpw)
@@ -2391,9 +2403,8 @@ qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int
     (void)cgrow;
     if (loads != QW_LOADS_TMA) {
         if (part != 2) {
-            // up to four entries per thread of one block cost less than a launch
             const int64_t qi = (int64_t)nb * st.bm_mp;
-            const bool one = qi <= 4096;
+            const bool one = buckets_in_one_block(nb, st.bm_mp);
             bm_active_kernel<<<1, 1024, 0, s>>>(ix, level, R, nb, st, ctl, one);
             QW_CUDA_TRY(cudaGetLastError());
             if (!one) {
@@ -2493,6 +2504,13 @@ qw_status launch_bm_collect(const IndexView &ix, int nb, int l, int cap, QuerySt
     bm_select_kernel<<<nb, SEL_THREADS, smem, s>>>(ix, l, cap, st, stats_out, sorted);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
+}
+
+// (the final buckets, one or two passes for slots, the listing; the rebuild's five;
+// the selection and the list of queries to answer again)
+int bm_select_launches(int nb, bool staged, int wave_slots, bool learned)
+{
+    return (staged ? 1 : 0) + (nb > wave_slots ? 2 : 1) + 1 + 5 + (learned ? 2 : 0) + 2;
 }
 
 qw_status launch_bm_list(const IndexView &ix, int nb, int l, int cgrow, QueryState &st,

@@ -170,7 +170,8 @@ qw_status build(LevelGraphCache *c, const GraphKey &key, const IndexView &ix, in
             ScanStats ss = bitmap ? scan_stats_of(ix, cgrow) : ScanStats();
             ss.recount_first = bitmap && learned;
             QW_TRY(launch_decide(nb, 0, 1, cap, st, cs, ctl, ss));
-            return launch_loop_ctl(ctl, st.max_top, cgrow, h, err, cs);
+            const int kernels = bitmap ? bm_level_launches(nb, st.bm_mp, loads, 0) : 1;
+            return launch_loop_ctl(ctl, st.max_top, cgrow, kernels, h, err, cs);
         };
     };
     if ((s = capture_into(cs, body, nullptr, 0, level_body(h1))) != QW_OK) return fail(s);

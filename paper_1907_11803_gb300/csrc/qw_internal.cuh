@@ -272,6 +272,7 @@ struct LoopCtl {
     int32_t level;
     int32_t pass;                 // 0, then 1 for the recomputed queries (learned start)
     unsigned long long iters;     // level passes run, summed over the call's batches
+    unsigned long long kernels;   // counting kernels they launched
     unsigned long long fb_total;  // learned start: queries recomputed, summed over batches
     unsigned long long skipped_total;  // learned start: levels skipped, summed over batches
     int32_t min_start;            // smallest first level of the batch's queries
@@ -321,6 +322,11 @@ ScanStats scan_stats_of(const IndexView &ix, int c);
 qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int64_t Rp, int l,
                           int cgrow, QueryState &st, int *err, int loads, cudaStream_t s,
                           const LoopCtl *ctl = nullptr, int part = 0, int tpw = 8);
+// Kernels that launch_bm_level launches, and those of a batch after its level loop
+// (launch_bm_list, launch_bm_reduce, launch_bm_recount for learned starts,
+// launch_bm_collect, launch_bm_overflow_list).
+int bm_level_launches(int nb, int mp, int loads, int part);
+int bm_select_launches(int nb, bool staged, int wave_slots, bool learned);
 // After the level loop: the candidates of every query's last level to its list
 // (staged: the level ran bm_level_tma_kernel).
 qw_status launch_bm_list(const IndexView &ix, int nb, int l, int cgrow, QueryState &st,
@@ -348,7 +354,8 @@ qw_status launch_bm_overflow_list(const QueryState &st, int nb, const int32_t *o
 
 // Device-driven loop control (qw_graph.cu builds the graphs that use them).
 qw_status launch_loop_init(LoopCtl *ctl, const QueryState &st, int nb, int cgrow, cudaStream_t s);
-qw_status launch_loop_ctl(LoopCtl *ctl, const unsigned long long *max_top, int cgrow,
+// kernels: launched per level by the counting
+qw_status launch_loop_ctl(LoopCtl *ctl, const unsigned long long *max_top, int cgrow, int kernels,
                           cudaGraphConditionalHandle h, int *err, cudaStream_t s);
 qw_status launch_fallback_graph(int nb, QueryState &st, LoopCtl *ctl,
                                 cudaGraphConditionalHandle h, cudaStream_t s);

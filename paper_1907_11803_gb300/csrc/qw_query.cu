@@ -505,13 +505,14 @@ __global__ void loop_init_kernel(LoopCtl *ctl, int cgrow)
 // next level.  Mirrors the host loop; level 63 would overflow R and is an
 // error (flag 8).
 __global__ void loop_ctl_kernel(LoopCtl *ctl, const unsigned long long *max_top, int cgrow,
-                                cudaGraphConditionalHandle h, int *err)
+                                int kernels, cudaGraphConditionalHandle h, int *err)
 {
     const int64_t R = ctl->R;
     // stop once R exceeds every useful radius, or no query is left to run
     bool more = (unsigned long long)R <= *max_top && ctl->active > 0;
     ctl->active = 0;
     ctl->iters += 1;
+    ctl->kernels += (unsigned long long)kernels;
     if (more && ctl->level > 62) {
         atomicOr(err, 8);
         more = false;
@@ -841,10 +842,10 @@ qw_status launch_loop_init(LoopCtl *ctl, const QueryState &st, int nb, int cgrow
     return QW_OK;
 }
 
-qw_status launch_loop_ctl(LoopCtl *ctl, const unsigned long long *max_top, int cgrow,
+qw_status launch_loop_ctl(LoopCtl *ctl, const unsigned long long *max_top, int cgrow, int kernels,
                           cudaGraphConditionalHandle h, int *err, cudaStream_t s)
 {
-    loop_ctl_kernel<<<1, 1, 0, s>>>(ctl, max_top, cgrow, h, err);
+    loop_ctl_kernel<<<1, 1, 0, s>>>(ctl, max_top, cgrow, kernels, h, err);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
 }
