@@ -655,29 +655,53 @@ __device__ __forceinline__ void count_planes(const IndexView &ix, const int32_t 
     }
 }
 
+constexpr int kCountWarps = 152 * 3 * 8;  // resident at once, of blocks that count groups
+
+// The bits of every word that part p of `parts` (a power of two up to 32) takes.
+__device__ __forceinline__ uint32_t part_bits(int p, int parts)
+{
+    const int bits = 32 / parts;
+    return (0xffffffffu >> (32 - bits)) << (bits * p);
+}
+
 // Few queries per group.  A warp takes the live bits of one query's four tiles
 // (a word per lane), and its lanes the set bits, 32 at a time: a lane reads its
 // group's word of each of the query's m bitmaps and sums them into bit planes.
 // Bound by the latency of those 16-byte reads (about 20 sectors a request): see
 // bm_dense_kernel for levels where many queries share a group.
+// Where the queries that run give the resident warps less than a task each, a task is
+// cut in up to 32 parts (equal runs of bits of every word): most groups are live
+// where the data has few clusters or a query lies far from them, and 1,024 groups
+// in one warp are 32 rounds of reads one after the other.  One query on 1,000,000
+// points of one Gaussian, 64 dimensions, a whole call: 1,054 us with whole tasks,
+// 400 so; 16 queries 1,634 and 711.
 __global__ void __launch_bounds__(256, 3) bm_count_kernel(IndexView ix, int level, int l,
                                                           QueryState st, const LoopCtl *ctl)
 {
     __shared__ int s_nb[QW_MAX_M + 16];
     __shared__ uint32_t s_keep[8][32];
+    __shared__ int s_whole, s_parts;
     if (dense_level(ix, st)) return;
     if (ctl) level = ctl->level;
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     const int m = ix.m, nT = ix.nT, mp = st.bm_mp;
     for (int i = threadIdx.x; i < mp; i += 256) s_nb[i] = i < m ? ix.bm_nb[i] : 0;
+    if (threadIdx.x == 0) {
+        const int whole = (int)st.bm_ctl[kCtlRun] * ((nT + 3) >> 2);  // (at most 2^23)
+        int parts = 1;
+        while (parts < 32 && whole * parts * 2 <= kCountWarps) parts *= 2;
+        s_whole = whole;
+        s_parts = parts;
+    }
     __syncthreads();
     const int run = (int)st.bm_ctl[kCtlRun];
-    const int64_t tasks = (int64_t)run * ((nT + 3) >> 2);
-    for (int64_t k = (int64_t)blockIdx.x * 8 + wi; k < tasks; k += (int64_t)gridDim.x * 8) {
-        const int q = st.bm_run[k % run], t0 = (int)(k / run) * 4;
+    for (int k = blockIdx.x * 8 + wi; k < s_whole * s_parts; k += gridDim.x * 8) {
+        const int task = k % s_whole;
+        const int q = st.bm_run[task % run], t0 = task / run * 4;
         uint32_t *am = st.bm_amask +
                        ((int64_t)(level & 1) * st.cln_par + (int64_t)q * nT + t0) * kSumWords + lane;
-        const uint32_t x = t0 + (lane >> 3) < nT ? *am : 0u;
+        uint32_t x = t0 + (lane >> 3) < nT ? *am : 0u;
+        if (s_parts > 1) x &= part_bits(k / s_whole, s_parts);
         if (!__any_sync(0xffffffffu, x != 0)) continue;
         s_keep[wi][lane] = x;
         __syncwarp();
@@ -694,7 +718,10 @@ __global__ void __launch_bounds__(256, 3) bm_count_kernel(IndexView ix, int leve
         });
         __syncwarp();
         const uint32_t keep = s_keep[wi][lane];
-        if (keep != x) *am = keep;
+        if (keep != x) {
+            if (s_parts == 1) *am = keep;
+            else atomicAnd(am, keep | ~x);  // (the other bits are other warps')
+        }
         __syncwarp();
     }
 }
@@ -1352,37 +1379,40 @@ __device__ __forceinline__ uint4 rd_word(const QueryState &st, int L, int64_t qt
 // them and no slot of the list rebuild below: the counts of its groups with candidates once more from the bitmaps
 // (few of the groups counted on the way there), and whether each was a candidate
 // of the previous level (its word there, if the query ran it).  A warp takes
-// four tiles of a query, as bm_count_kernel does; where there are no more than
-// kListQuads of those and the query has more than kListPart candidates (in the
-// locality order they lie in a few tiles), a quarter of their groups.  Listing during the levels
+// four tiles of a query, as bm_count_kernel does, or one of `parts` parts of their
+// groups where the query has more than kListPart candidates, or where they are more
+// than 32 and there are warps to spare (else part 0 takes them all).  Listing during the levels
 // instead, every candidate of every level behind a returning atomic, took most
 // of the count pass where candidates are many (606 queries whose last level
 // takes in all 300,000 points: 2.3 ms of a level of 0.17).
 constexpr int kListPart = 2048;
-constexpr int64_t kListQuads = 65536;
 
 __global__ void __launch_bounds__(256, 3) bm_list_kernel(IndexView ix, int l, int nb, int parts,
-                                                          QueryState st)
+                                                          bool spare, QueryState st)
 {
     __shared__ int s_nb[QW_MAX_M + 16];
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     const int m = ix.m, nT = ix.nT, mp = st.bm_mp;
     for (int i = threadIdx.x; i < mp; i += 256) s_nb[i] = i < m ? ix.bm_nb[i] : 0;
     __syncthreads();
-    const int64_t tasks = (int64_t)nb * ((nT + 3) >> 2) * parts;
-    for (int64_t k = (int64_t)blockIdx.x * 8 + wi; k < tasks; k += (int64_t)gridDim.x * 8) {
-        const int q = (int)(k % nb), t0 = (int)(k / nb / parts) * 4, part = (int)(k / nb % parts);
+    const int tasks = nb * ((nT + 3) >> 2) * parts;
+    for (int k = blockIdx.x * 8 + wi; k < tasks; k += gridDim.x * 8) {
+        const int q = k % nb, t0 = k / nb / parts * 4, part = k / nb % parts;
         const int L = st.levels[q] - 1;
         if (L < 0) continue;
         const int n = st.qbuf_n[(int64_t)(L & 1) * st.qbn_par + q];
         if (n == 0 || n > kQCap || (st.bm_ovf[q] & 8)) continue;
-        if (n <= kListPart && part) continue;  // few candidates: part 0 takes all
         const bool ran_prev = L > st.start[q];
         uint32_t x =
             t0 + (lane >> 3) < nT
                 ? st.bm_amask[((int64_t)(L & 1) * st.cln_par + (int64_t)q * nT + t0) * kSumWords + lane]
                 : 0u;
-        if (n > kListPart && parts > 1) x &= 0xffu << (8 * part);
+        if (parts > 1) {
+            if (n > kListPart || (spare && __reduce_add_sync(0xffffffffu, __popc(x)) > 32))
+                x &= part_bits(part, parts);
+            else if (part)
+                continue;
+        }
         if (!__any_sync(0xffffffffu, x != 0)) continue;
         uint64_t *list = st.qbuf + (int64_t)q * kQCap;
         each_set_bit(x, lane, [&](int own, int bit, bool valid, bool four) {
@@ -1800,7 +1830,7 @@ __device__ __forceinline__ uint32_t rd_task(const IndexView &ix, const QueryStat
                            ? st.bm_amask[((int64_t)(*L & 1) * st.cln_par + (int64_t)*q * ix.nT +
                                           *t0) * kSumWords + lane]
                            : 0u;
-    return x & (0xffffffffu >> (32 - 32 / kRdParts) << (32 / kRdParts * part));
+    return x & part_bits(part, kRdParts);
 }
 
 __global__ void __launch_bounds__(RD_THREADS, 3) rd_count_kernel(IndexView ix, int l, int cap,
@@ -2423,11 +2453,12 @@ qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int
         }
         // two passes: filter on the summaries, then count the live groups
         const int64_t tasks = (int64_t)nb * ((ix.nT + 3) / 4);
-        const unsigned blocks =
-            (unsigned)std::max<int64_t>(1, std::min<int64_t>((tasks + 7) / 8, 152 * 24));
-        bm_filter_kernel<<<blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, st, ctl);
+        const int64_t blocks =
+            std::max<int64_t>(1, std::min<int64_t>((tasks + 7) / 8, 152 * 24));
+        bm_filter_kernel<<<(unsigned)blocks, FL_WARPS * 32, 0, s>>>(ix, level, l, st, ctl);
         QW_CUDA_TRY(cudaGetLastError());
-        bm_count_kernel<<<blocks, 256, 0, s>>>(ix, level, l, st, ctl);
+        const int64_t cblocks = std::max(blocks, std::min<int64_t>(tasks * 4, kCountWarps / 8));
+        bm_count_kernel<<<(unsigned)cblocks, 256, 0, s>>>(ix, level, l, st, ctl);
         QW_CUDA_TRY(cudaGetLastError());
         // fewer queries than the dense form asks of an average group never take it
         if (nb >= kDenseMin) {
@@ -2532,9 +2563,10 @@ qw_status launch_bm_list(const IndexView &ix, int nb, int l, int cgrow, QuerySta
     if (nb > wave_slots)
         rd_compact_kernel<<<qb, 128, 0, s>>>(ix, cgrow, st, nb, kQDirect, kQCap, wave_slots);
     const int64_t quads = (int64_t)nb * ((ix.nT + 3) / 4);
-    const int parts = quads <= kListQuads ? 4 : 1;
+    int parts = quads <= 65536 ? 4 : 1;
+    while (parts < 32 && quads * parts * 2 <= kCountWarps) parts *= 2;
     bm_list_kernel<<<(unsigned)std::min<int64_t>((quads * parts + 7) / 8, 152 * 24), 256, 0, s>>>(
-        ix, l, nb, parts, st);
+        ix, l, nb, parts, quads * parts <= kCountWarps, st);
     QW_CUDA_TRY(cudaGetLastError());
     return QW_OK;
 }
