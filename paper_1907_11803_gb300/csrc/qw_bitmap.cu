@@ -324,20 +324,42 @@ constexpr int kSumWords = kBmUint4 / 32;      // summary words per bitmap (8)
 constexpr int kDenseTable = 66 * 1024;       // bytes of tables per block
 constexpr int kDenseGroups = 16;             // most groups per block
 constexpr int kDenseMin = 256;               // live groups per group of the index
+constexpr int kDenseBlocks = 2 * 152;        // two per SM
+constexpr int kDenseUnits = 200;             // fewest units (groups x query slices)
 
 // Per level, in st.bm_ctl: [0] live groups, [1] the dense form's next unit,
 // [2] S (0: more than 15 buckets), [3] groups per block, [4] queries that run.
 enum { kCtlLive = 0, kCtlUnit = 1, kCtlRows = 2, kCtlGroups = 3, kCtlRun = 4 };
 
-// The dense form pays when a group's table is read often enough: its words are
-// loaded once per block instead of once per query.  The line lies where both
-// forms take the same time: with 223 live groups per group of the index 112 us
-// dense against 99, with 387 320 against 304, with 646 155 against 183, with
-// 1,211 609 against 906, with 1,762 2.4 ms against 3.6.
+// The dense form's query slices, so that there are several units per block: slices
+// of at least 1,024 of `run` queries.
+__device__ __forceinline__ int dense_slices(int nT, int G, int run)
+{
+    const int chunks = nT * (kBmUint4 / G);
+    return max(1, min((kDenseBlocks * 4 + chunks - 1) / chunks, (run + 1023) / 1024));
+}
+
+// The dense form pays when a group's table is read often enough (its words are
+// loaded once per block instead of once per query) and its units fill the GPU: on a
+// small index most blocks have none.  The lines lie where both forms take about the
+// same time (live groups per group of the index: us count and dense).
+//   1,000,000 points, 64 projections, S = 16: 135: 199 and 251, 175: 236 and 274,
+//     295: 310 and 256, 386: 429 and 398, 689: 538 and 415, 1,969: 1,274 and 806;
+//     S = 8: 125: 173 and 171, 256: 308 and 301, 539: 457 and 308; S = 4: 165: 385
+//     and 118, 438: 534 and 258 (units 496 and more);
+//   200,000 points, 48 projections, S = 16 and 448 units: 261: 64 and 55, 610: 106
+//     and 84; S = 8 and 224 units: 262: 59 and 44; S = 4: 426 with 112 units 118 and
+//     114, 1,186 with 224 224 and 160;
+//   100,000 points, 64 projections, S = 4: 667 with 64 units 80 and 236, 774 with 128
+//     111 and 160, 1,967 with 192 201 and 235, 2,338 with 256 291 and 231;
+//   30,000 points, 40 projections, S = 4: 3,271 with 64 units 59 and 195; S = 8: 1,836
+//     with 64 54 and 112, 5,504 with 192 88 and 114; S = 16: 5,501 with 384 86 and 84.
 __device__ __forceinline__ bool dense_level(const IndexView &ix, const QueryState &st)
 {
-    return st.bm_ctl[kCtlRows] > 0 &&
-           st.bm_ctl[kCtlLive] >= (uint32_t)kDenseMin * (uint32_t)ix.nT * kBmUint4;
+    const int S = (int)st.bm_ctl[kCtlRows], G = (int)st.bm_ctl[kCtlGroups];
+    return S > 0 &&
+           st.bm_ctl[kCtlLive] >= (uint32_t)kDenseMin * (uint32_t)ix.nT * kBmUint4 &&
+           ix.nT * (kBmUint4 / G) * dense_slices(ix.nT, G, (int)st.bm_ctl[kCtlRun]) >= kDenseUnits;
 }
 
 // Buckets of projection i at a level (one past the last stored level).
@@ -850,10 +872,9 @@ __global__ void __launch_bounds__(DN_THREADS, 2) bm_dense_kernel(IndexView ix, i
     const int nb = (int)st.bm_ctl[kCtlRun];  // queries that run
     const int S = (int)st.bm_ctl[kCtlRows], G = (int)st.bm_ctl[kCtlGroups];
     const int words = table_words(mp, S);
-    // queries in slices, so that there are several units per block
     const int per_tile = kBmUint4 / G;
     const int chunks = nT * per_tile;
-    const int slices = max(1, min((int)(gridDim.x * 4 + chunks - 1) / chunks, (nb + 1023) / 1024));
+    const int slices = dense_slices(nT, G, nb);
     const int per_slice = ((nb + slices - 1) / slices + 31) & ~31;
     uint32_t *amask = st.bm_amask + (int64_t)(level & 1) * st.cln_par * kSumWords;
     for (int i = threadIdx.x; i < m; i += DN_THREADS) sh.nbk[i] = buckets_at(ix, i, level, R);
@@ -2464,7 +2485,7 @@ qw_status launch_bm_level(const IndexView &ix, int nb, int level, int64_t R, int
         if (nb >= kDenseMin) {
             const size_t smem = dense_smem_bytes();
             QW_TRY(allow_smem(bm_dense_kernel, smem));
-            bm_dense_kernel<<<2 * 152, DN_THREADS, smem, s>>>(ix, level, R, l, st, ctl);
+            bm_dense_kernel<<<kDenseBlocks, DN_THREADS, smem, s>>>(ix, level, R, l, st, ctl);
             QW_CUDA_TRY(cudaGetLastError());
         }
         return QW_OK;
