@@ -140,7 +140,8 @@ typedef struct {
     int32_t order;        /* QW_ORDER_SIGNATURE: answer queries grouped by a coarse bucket
                              signature (queries of one region share index entries in L2);
                              QW_ORDER_GIVEN: in the caller's order; QW_ORDER_AUTO: by
-                             signature from 2,048 queries on.  Results are
+                             signature from 2,048 queries on, or from 4e9 / n where
+                             that is fewer.  Results are
                              returned in the caller's order either way and do not depend on it */
     int32_t rerank;       /* QW_RERANK_FP32 (default), QW_RERANK_BF16 or QW_RERANK_BF16_TC
                              (both need shadow_bf16): the BF16 pre-filter on CUDA cores, or with

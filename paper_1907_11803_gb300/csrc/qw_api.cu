@@ -874,15 +874,23 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
     const int path = qp ? qp->path : QW_PATH_AUTO;
     const bool qalsh = ix->family == QW_FAMILY_QALSH;
     // the workload order groups queries by bucket signature (bucketed family).
-    // QW_ORDER_AUTO orders from kOrderQueries queries on: sorting, gathering and
-    // scattering cost 30 to 40 us, and with fewer queries the caller's order is
-    // never slower (measured at 64 to 10,000 queries on 0.1, 0.5 and 2 million
-    // points, level and bitmap paths: 493 against 463 us at 64 queries, 592
-    // against 555 at 1,000, 3,904 against 3,902 at 4,000)
-    const int64_t kOrderQueries = 2048;
+    // Sorting, gathering and scattering cost 20 to 40 us, and gain what queries of
+    // one region then share in L2: nothing where the index fits there or the queries
+    // share no region.  QW_ORDER_AUTO orders from kOrderQueries queries on, and
+    // smaller workloads from kOrderWork (queries x points).  Bitmap path, us ordered
+    // and as given, queries of 20 clusters | of any: 1,000 on 500,000 points 1,380
+    // and 1,368 | 1,363 and 1,335; on 1 million 1,505 and 1,502 | 1,676 and 1,656; on
+    // 4 million 3,707 and 3,795 | 3,778 and 3,754; on 10 million 7,760 and 7,972 |
+    // 8,132 and 8,119; 256 on 10 million 2,637 and 2,656 | 2,904 and 2,877; 400 3,572
+    // and 3,639 | 3,938 and 3,892; 2,000 on 1 million 2,119 and 2,150 | 2,375 and
+    // 2,365.  The level path takes the same either way (7,573 and 7,560 us for 1,000
+    // on 500,000 points; 141.0 and 142.7 ms on 10 million).
+    const int64_t kOrderQueries = 2048, kOrderWork = 4000000000;
     const int how = qp ? qp->order : QW_ORDER_AUTO;
-    const bool order = !qalsh && (how == QW_ORDER_SIGNATURE ||
-                                  (how == QW_ORDER_AUTO && nq >= kOrderQueries));
+    const bool order =
+        !qalsh && (how == QW_ORDER_SIGNATURE ||
+                   (how == QW_ORDER_AUTO &&
+                    (nq >= kOrderQueries || (nq > 1 && nq * ix->n >= kOrderWork))));
     const bool host = mem == QW_MEM_HOST;
     const bool bf16 = qp && qp->rerank == QW_RERANK_BF16;
     const bool bf16_tc = qp && qp->rerank == QW_RERANK_BF16_TC;
