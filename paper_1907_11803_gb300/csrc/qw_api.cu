@@ -1671,8 +1671,8 @@ qw_status qw_autotune(qw_index *ix, const float *queries, int64_t nq, int32_t k,
             qw_query_params alt = cur;
             alt.graph = 1;
             if ((status = try_alt(alt)) != QW_OK) break;
-            // tile shape of the filter / fused kernels: tiles per warp
-            if (cur.bitmap_loads != QW_LOADS_TMA) {
+            // tile shape of the fused kernel: tiles per warp (no other kernel has one)
+            if (cur.bitmap_loads == QW_LOADS_FUSED) {
                 const qw_query_params keept = cur;
                 for (int tw : {4, 16}) {
                     qw_query_params a2 = keept;
