@@ -575,7 +575,10 @@ qw_status qw_autotune(qw_index *index, const float *queries, int64_t nq, int32_t
  * model returns QW_ERR_ARG for a NULL model or pointer argument (and names the
  * problem in qw_last_error), QW_ERR_OOM when device memory runs out and
  * QW_ERR_CUDA on a CUDA error.  qw_mlp_loss_grad and qw_mlp_train wait for
- * their stream; qw_mlp_predict only enqueues its kernels on it. */
+ * their stream; qw_mlp_predict only enqueues its kernels on it.  A model keeps,
+ * besides its parameters, the activations of the most rows of a call and up to
+ * 256 MiB of partial weight gradients (none where that memory is not to be had:
+ * the gradient is then formed in one piece) until it is freed. */
 typedef struct qw_mlp qw_mlp;
 
 /* A model with zeroed parameters, owned by the caller until qw_mlp_free.

@@ -401,17 +401,23 @@ struct qw_mlp {
         const int64_t fit = kPartBytes / (np * (int64_t)sizeof(float));
         return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(kSplits, n / 64), fit));
     }
-    const float *partials(int n) const { return (splits_of(n) == 1 ? grad : part).as<float>(); }
+    int pieces = 1;  // of the last backward pass
+    const float *partials() const { return (pieces == 1 ? grad : part).as<float>(); }
 
     // loss sum into scalar[0] and the pieces' gradients (mean over n rows):
-    // gradient i = the sum over the pieces of partials(n)[piece * np + i]
+    // gradient i = the sum over the pieces of partials()[piece * np + i].  Without
+    // memory for the partial sums the rows are one piece.
     qw_status backward(const float *X, const int32_t *y, int n, cudaStream_t s)
     {
         const __half *h = p16.as<__half>();
         float *loss = scalar.as<float>();
-        const int S = splits_of(n);
+        pieces = splits_of(n);
+        if (pieces > 1 && part.ensure((size_t)pieces * np * sizeof(float)) != QW_OK) {
+            clear_error();
+            pieces = 1;
+        }
+        const int S = pieces;
         const int kper = ((n + S - 1) / S + GK - 1) / GK * GK;
-        if (S > 1) QW_TRY(part.ensure((size_t)S * np * sizeof(float)));
         float *g = S > 1 ? part.as<float>() : grad.as<float>();
         softmax_rows_kernel<<<(n + 7) / 8, 256, 0, s>>>(Z3, n, C, y, 1.0f / (float)n, D3, loss,
                                                         nullptr);
@@ -513,9 +519,8 @@ qw_status qw_mlp_loss_grad(qw_mlp *mp, const float *X, const int32_t *y, int64_t
     QW_CUDA_TRY(cudaMemsetAsync(mp->scalar.p, 0, 64, s));
     QW_TRY(mp->forward(X, (int)n, s));
     QW_TRY(mp->backward(X, y, (int)n, s));
-    const int splits = mp->splits_of((int)n);
-    if (grad && splits > 1) {
-        grad_sum_kernel<<<152 * 4, 256, 0, s>>>(mp->partials((int)n), mp->np, splits,
+    if (grad && mp->pieces > 1) {
+        grad_sum_kernel<<<152 * 4, 256, 0, s>>>(mp->partials(), mp->np, mp->pieces,
                                                 mp->grad.as<float>());
         QW_CUDA_TRY(cudaGetLastError());
     }
@@ -550,8 +555,8 @@ qw_status qw_mlp_train(qw_mlp *mp, const float *X, const int32_t *y, int64_t n, 
             mp->version += 1;
             const float c1 = 1.0f - powf(b1, (float)mp->step);
             const float c2 = 1.0f - powf(b2, (float)mp->step);
-            adam_kernel<<<152 * 4, 256, 0, s>>>(mp->p32.as<float>(), mp->partials(nb),
-                                                mp->splits_of(nb), mp->m1.as<float>(), mp->m2.as<float>(),
+            adam_kernel<<<152 * 4, 256, 0, s>>>(mp->p32.as<float>(), mp->partials(), mp->pieces,
+                                                mp->m1.as<float>(), mp->m2.as<float>(),
                                                 mp->p16.as<__half>(), mp->np, lr, b1, b2, eps, c1,
                                                 c2);
             QW_CUDA_TRY(cudaGetLastError());
