@@ -732,8 +732,13 @@ qw_status launch_hash(const float *V, int64_t nv, int d, const float *A, const f
     } else {
         const int bn = m <= 32 ? 32 : 64;
         const int64_t cb = (m + bn - 1) / bn;
-        // 256 rows per block once that gives every SM two blocks, else 64
-        const bool wide = (nv + 255) / 256 * cb >= 2 * 152;
+        // 256 rows per block from 100 blocks on, else 64: with fewer, the smaller
+        // blocks' use of every SM outweighs their reads of A (64 and 256 rows, us, 128
+        // dimensions x 64 projections: 75 blocks 52 and 57, 118 71 and 58, 196 84 and
+        // 68, 301 101 and 70, 1,172 259 and 181; 512 x 64: 75 96 and 111, 118 137 and
+        // 110; 128 x 32: 75 45 and 49, 118 57 and 48; 64 x 127: 64 50 and 57, 150 57
+        // and 57, 236 73 and 62)
+        const bool wide = (nv + 255) / 256 * cb >= 100;
         const int64_t rb = wide ? (nv + 255) / 256 : (nv + 63) / 64;
         if (rb > 2147483647LL) return QW_ERR_ARG;
         const dim3 grid((unsigned)rb, (unsigned)cb, wide ? 1u : (unsigned)shares(rb * cb));
