@@ -255,7 +255,7 @@ def _l2_fields(l2) -> dict:
 
 
 def qw_hash(V: int, nv: int, d: int, A: int, b: int, m: int, w: float, H: int, stream: int = 0):
-    """Device pointers in, returns the number of FP64 recomputations."""
+    """Device pointers in, returns the number of entries near a bucket edge."""
     fix = C.c_int64(0)
     _check(load().qw_hash(V, nv, d, A, b, m, w, H, C.byref(fix), stream or None))
     return int(fix.value)
@@ -263,7 +263,7 @@ def qw_hash(V: int, nv: int, d: int, A: int, b: int, m: int, w: float, H: int, s
 
 def qw_hash_tc(V: int, nv: int, d: int, A: int, b: int, m: int, w: float, H: int,
                stream: int = 0):
-    """qw_hash on the tensor cores; returns the number of FP64 recomputations."""
+    """qw_hash on the tensor cores; returns the number of entries near a bucket edge."""
     fix = C.c_int64(0)
     _check(load().qw_hash_tc(V, nv, d, A, b, m, w, H, C.byref(fix), stream or None))
     return int(fix.value)
@@ -388,8 +388,8 @@ def _f32(t, name):
 
 def hash(V, A, b, w: float, tensor_cores: bool = False):
     """Bucket ids floor((A V^T + b) / w) of CUDA float32 tensors (tensor_cores:
-    qw_hash_tc).  Returns (H int32 nv x m on V's device, number of FP64
-    recomputations)."""
+    qw_hash_tc).  Returns (H int32 nv x m on V's device, number of entries
+    near a bucket edge)."""
     torch = _torch()
     _f32(V, "V"), _f32(A, "A"), _f32(b, "b")
     if not (V.is_cuda and A.is_cuda and b.is_cuda):

@@ -952,7 +952,7 @@ static qw_status run_impl(qw_index *ix, const float *queries, int64_t nq, int k,
         B = ix->tuned_batch;
     if (B == 0) {
         // workspace of one batch: 2 GB of counters on the level path; the
-        // bitmap path (about 4.3 MB per query at 1M points) takes up to 48 GB,
+        // bitmap path (about 2.4 MB per query at 1M points) takes up to 48 GB,
         // a sixth of the 280 GB HBM, so most workloads run as one batch
         const int64_t budget = use_bitmap ? kBitmapBudget : (int64_t)2 << 30;
         B = use_cluster ? (int64_t)65535

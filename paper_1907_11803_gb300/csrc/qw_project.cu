@@ -16,7 +16,11 @@
 // by w add at most 3u |u| + u.  Whenever the distance of u to the nearest
 // integer is not larger than that bound (or than 1e-5, i.e. 1e-5 w in
 // projection units, whichever is larger), floor(u) is not trusted and the entry
-// goes to the block's list (0.15 % of them at d = 128 on the benchmark's data).
+// goes to the block's list: 0.15 % of them at d = 128 on the benchmark's data, and
+// more as the rows' norm grows against w.  1,000,000 x 128 x 64, unit spread about
+// 0, 10, 100, 1,000 and 10,000, w = 4: 0.03, 0.3, 2.5, 25 and 100 % of the entries,
+// 512, 514, 710, 2,465 and 8,102 us (with an error sum per entry and FP64 for all
+// that it left open 1,498, 1,975, 6,595, 36,772 and 62,457).
 //
 // Pass 2 (same block) recomputes the listed entries, eight lanes each, in
 // pairs of floats: products and sums are split into a rounded value and its

@@ -277,8 +277,8 @@ __global__ void __launch_bounds__(TR_ROWS) tree_plane_kernel(Tree T, int n_chunk
 // Per chunk: each row's side of its node's hyperplane, and the coordinate sums
 // of both sides.  A block takes 256 rows at a time: warps form the rows'
 // projections, then threads own coordinates (256 / d threads share one, each a
-// part of the rows) and add the rows, now in L1, side by side.  Five blocks per SM
-// hide its loads: 12.0 ms at 300,000 x 512 (three with 80 registers: 26).
+// part of the rows) and add the rows, now in L1, side by side.  Held to five blocks
+// per SM, 48 registers: 12.0 ms at 300,000 x 512.
 __global__ void __launch_bounds__(TR_ROWS, 5) tree_assign_kernel(Tree T, bool in_smem)
 {
     extern __shared__ float sums_s[];
