@@ -679,36 +679,37 @@ def run_ours(args):
                           "collision counting)" if qalsh else
                           "level_kernel (bucket-range search + collision counting)")}[dom]
     if bitmap and dom == "level":
-        if chosen_kw.get("loads", "tma") == "fused":
-            # one pass: per (query, tile, level) the m bucket summaries (32 B);
-            # per live 128-id group the previous and the new candidate word and
-            # the bitmap words of the projections touching it (16 B each)
+        if chosen_kw.get("loads", "tma") in ("direct", "fused"):
+            # the levels' inputs and outputs, each once: per batch the bitmaps
+            # (and summaries, 1/128 of that) of every level that is some query's last,
+            # or the live groups' words (16 B per projection that touches the group)
+            # where those are fewer; per (query, tile, level) the live mask (32 B) and
+            # per live 128-id group its candidate word (16 B), written
             dom_name = ("bm_fused_kernel (summary filter and bit-sliced collision counts of the "
-                        "live 128-id groups in one launch)")
-            count_bytes = ((prof["level_passes"] / steps) * index.info.n_tiles * s.m * 32.0
-                           + (prof["bitmap_live_groups"] / steps) * 32.0
-                           + (prof["bitmap_live_words"] / steps) * 16.0)
-        elif chosen_kw.get("loads", "tma") == "direct":
-            # the same algorithmic bytes as the one-pass form: per (query, tile,
-            # level) the m bucket summaries (32 B); per live 128-id group the
-            # previous and the new candidate word and the bitmap words of the
-            # projections touching it (16 B each).  The work list between the
-            # passes is the implementation's, not the method's.
-            dom_name = ("bm_filter_kernel + bm_count_kernel (summary filter, then bit-sliced "
-                        "collision counts of the live 128-id groups)")
-            count_bytes = ((prof["level_passes"] / steps) * index.info.n_tiles * s.m * 32.0
-                           + (prof["bitmap_live_groups"] / steps) * 32.0
-                           + (prof["bitmap_live_words"] / steps) * 16.0)
+                        "live 128-id groups in one launch)"
+                        if chosen_kw.get("loads") == "fused" else
+                        "bm_filter_kernel + bm_count_kernel / bm_dense_kernel (summary filter, "
+                        "then bit-sliced collision counts of the live 128-id groups, from the "
+                        "bitmaps or from tables in shared memory)")
+            span = np.empty(s.m, np.int32)
+            qw.qw_index_export(index.handle, 0, span.ctypes.data, 0, 0)
+            last = np.unique(st[:, 0]) - 1
+            per_tile = sum(int((span.astype(np.int64) // s.c ** int(lv) + 1).sum()) for lv in last)
+            n_batches = prof["timed_launches"]["rerank"] / steps
+            level_bitmaps = n_batches * per_tile * index.info.n_tiles * 4096.0
+            count_bytes = (min(level_bitmaps, (prof["bitmap_live_words"] / steps) * 16.0)
+                           + level_bitmaps / 128.0
+                           + (prof["level_passes"] / steps) * index.info.n_tiles * 32.0
+                           + (prof["bitmap_live_groups"] / steps) * 16.0)
         else:
             # per (query, level) pass and tile: the m bucket bitmaps, the previous
             # level's candidate bitmap and the new one, 4 KiB each
             dom_name = "bm_level_tma_kernel (bit-sliced collision counts, TMA-staged bitmaps)"
             count_bytes = (prof["level_passes"] / steps) * index.info.n_tiles * (s.m + 2) * 4096.0
-    # launches actually run; for the two-pass bitmap level a "launch" is one
-    # level pass (its filter and count launches; the bucket numbers of each
-    # pass are timed apart in their own class)
-    two_pass = bitmap and dom == "level" and chosen_kw.get("loads", "tma") in ("direct", "fused")
-    dom_launches = (prof["timed_launches"]["bucket"] if two_pass else prof["launches"][dom]) / steps
+    # launches of the class's kernels (bitmap path, direct loads: the filter and the
+    # one or two count kernels of every level; the buckets' numbers are a class of
+    # their own)
+    dom_launches = prof["launches"][dom] / steps
     dom_ms = prof["ms"][dom] / steps
     per_launch_bytes = count_bytes / max(dom_launches, 1)
     per_launch_s = (dom_ms / 1e3) / max(dom_launches, 1)

@@ -248,7 +248,7 @@ typedef struct {
  * QW_PATH_CLUSTER: one persistent launch of thread-block clusters; a cluster
  *   answers one query at a time with its counters in shared memory for all
  *   levels and pulls the next query from a work queue; indexes of up to
- *   96 tiles (3,145,728 points).
+ *   80 tiles (2,621,440 points).
  * QW_PATH_BITMAP: the level loop of QW_PATH_LEVELS, but the collision counts
  *   of a (tile, query) are recomputed at every level as the bit-sliced sum of
  *   the m precomputed bitmaps of the query's level-L buckets (no per-entry
