@@ -14,16 +14,16 @@
 // to count.  FP32 sums serve where they are taken of what tells a node's points
 // apart: every coordinate is read as its difference from the node's first point
 // (exact to a rounding, so that an offset common to the data costs nothing), and a
-// hyperplane's normal is scaled to a largest component of 1 (only the side and the
-// order of distances count), so that no product leaves the range that the
-// coordinates themselves fit.  Sums of a chunk's differences stay below FP32's
+// hyperplane's normal is divided by the largest component of the first one's (only
+// the side and the order of distances count), so that no product leaves the range
+// that the coordinates themselves fit.  Sums of a chunk's differences stay below FP32's
 // largest number for coordinates up to about 1e33.
 //
 // All nodes of a level are split together.  A node's points are cut in chunks
 // of whole blocks (256 rows, more for large nodes: at most kMaxChunks chunks
 // per node); the kernels of a level work on chunks, those that combine a
 // node's chunks (in chunk order: the tree is the same for every build) on
-// nodes.  What bounds it is reading the rows five times a level: 18 ms at
+// nodes.  What bounds it is reading the rows five times a level: 17 ms at
 // 1,000,000 x 128 (21 levels; 8.4 ms of it the side sums), against more than a
 // second on 16 host cores in FP64, beside copying the data there.  The host
 // only launches: it reads three counters per level.
@@ -48,7 +48,7 @@ struct Tree {
     const float *A;
     int64_t n;
     int d, m;
-    int dv;                  // floats per row of v (d + 1, padded to 16 bytes)
+    int dv;                  // floats per row of v (d + 2, padded to 16 bytes)
     bool vec;                // rows in 16-byte pieces
     int32_t *perm, *perm2;   // the order, and the split nodes' next one
     float *t;                // signed distance to the node's hyperplane (times |v|)
@@ -57,7 +57,7 @@ struct Tree {
     int32_t *lo2, *hi2, *c02, *o2;
     int32_t *cut;            // per node, points of the first child
     int32_t *node, *node2;   // per chunk, its node
-    float *v;                // per node, c2 - c1 scaled (d), then the threshold
+    float *v;                // per node, c2 - c1 scaled (d), the threshold, the scale
     float *part;             // per chunk, coordinate sums of both sides (2 d), of the
                              // differences from the node's first point
     int32_t *below;          // per chunk, points of the first side
@@ -197,10 +197,10 @@ __device__ __forceinline__ float block_reduce(float x, float *tmp)
     return s;
 }
 
-// Per node: the hyperplane between two centroids, v = c2 - c1 over its largest
-// component and the threshold v . (c1 + c2) / 2, from the seeds (round 0) or from
-// the sums of the chunks' sides.  A side without points leaves the hyperplane as it
-// is.
+// Per node: the hyperplane between two centroids, v = c2 - c1 over the node's scale
+// (the largest component between the seeds) and the threshold v . (c1 + c2) / 2, from
+// the seeds (round 0) or from the sums of the chunks' sides.  A side without points
+// leaves the hyperplane as it is.
 __global__ void __launch_bounds__(TR_ROWS) tree_plane_kernel(Tree T, int n_chunks, int n_nodes,
                                                              bool seeds)
 {
@@ -252,23 +252,19 @@ __global__ void __launch_bounds__(TR_ROWS) tree_plane_kernel(Tree T, int n_chunk
             }
         }
     };
-    // the centroids' middle takes the place of the sums of the node's first chunk (a
-    // coordinate's sums are read by its thread alone)
-    float *mid = T.part + (int64_t)k0 * 2 * d;
-    float most = 0.0f;
+    float most = seeds ? 0.0f : v[d + 1];
+    if (seeds) {
+        for (int c = threadIdx.x; c < d; c += TR_ROWS) most = fmaxf(most, fabsf(x2[c] - x1[c]));
+        most = block_reduce<true>(most, tmp);
+        if (threadIdx.x == 0) v[d + 1] = most;
+    }
+    float q = 0.0f;
     for (int c = threadIdx.x; c < d; c += TR_ROWS) {
         float a, b;
         centroids(c, a, b);
-        mid[c] = 0.5f * a + 0.5f * b;
-        v[c] = b - a;
-        most = fmaxf(most, fabsf(b - a));
-    }
-    most = block_reduce<true>(most, tmp);
-    float q = 0.0f;
-    for (int c = threadIdx.x; c < d; c += TR_ROWS) {
-        const float w = most > 0.0f ? v[c] / most : 0.0f;
+        const float w = most > 0.0f ? (b - a) / most : 0.0f;
         v[c] = w;
-        q += w * mid[c];
+        q += w * (0.5f * a + 0.5f * b);
     }
     q = block_reduce<false>(q, tmp);
     if (threadIdx.x == 0) v[d] = q;
@@ -552,7 +548,7 @@ qw_status locality_order(const float *X, int64_t n, int d, const float *A, int m
     T.n = n;
     T.d = d;
     T.m = m;
-    T.dv = (d + 4) / 4 * 4;
+    T.dv = (d + 5) / 4 * 4;
     T.vec = d % 4 == 0 && ((uintptr_t)X | (uintptr_t)A) % 16 == 0;
     // at most n / kGroupIds nodes a level (every node holds more than
     // kGroupIds points), and chunks for them
